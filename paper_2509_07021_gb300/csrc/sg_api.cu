@@ -184,7 +184,7 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
         d.blk_off = (uint32_t)bwd_blk;
         bwd_blk += div_up((uint64_t)sc.n, PRE_THREADS);
     }
-    uint64_t tiles = 0, pix = 0, ent = 0;
+    uint64_t tiles = 0, groups = 0, pix = 0, ent = 0;
     for (int v = 0; v < n_views; ++v) {
         const sg_camera &c = cams[v];
         const int s = view_scene ? view_scene[v] : 0;
@@ -213,6 +213,8 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
         d.scene = s;
         d.n = (int32_t)scenes[s].n;
         d.tile_off = (uint32_t)tiles;
+        d.grp_off = (uint32_t)groups;
+        groups += div_up((uint64_t)d.tiles_x * d.tiles_y, 32);
         d.pix_off = pix;
         d.ent_off = ent;
         tiles += (uint64_t)d.tiles_x * d.tiles_y;
@@ -224,6 +226,7 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
         return fail(SG_ERR_INVALID_ARG, "too many (view, Gaussian) entries (%llu)", (unsigned long long)ent);
     if (bwd_blk >= (1ull << 31)) return fail(SG_ERR_INVALID_ARG, "too many blocks");
     b.n_tiles = (uint32_t)tiles;
+    b.n_groups = (uint32_t)groups;
     b.n_entries = ent;
     b.scene_blocks = (uint32_t)bwd_blk;
     uint32_t per_scene[SG_MAX_SCENES] = {};
@@ -241,45 +244,55 @@ uint64_t n_pixels_of(const Batch &b) {
     return p;
 }
 
+// Calls whose views have at most this many tiles in all keep no sorted tile ids.
+constexpr uint64_t kNoKeyTiles = 12288;
+// Pairs per row of the binning's count matrix that the per-pair size reports.
+constexpr uint64_t kMatrixShare = 8192;
+
 WsLayout make_layout(const Batch &b, uint64_t cap) {
     WsLayout L{};
     const uint64_t M = b.n_entries, T = b.n_tiles;
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o += al(bytes); return r; };
+    uint64_t row = 0;
+    for (int v = 0; v < b.n_views; ++v)
+        row = std::max<uint64_t>(row, (uint64_t)b.view[v].tiles_x * b.view[v].tiles_y);
+    row = div_up(row, 4) * 4;
+    // chunks where one chunk's counters of the largest view fit shared memory
+    L.chunked = row <= BIN_MAX_ROW;
+    L.bin_row = (uint32_t)row;
+    L.bin_chunks = L.chunked ? bin_chunks(cap, L.bin_row) : 0u;
     L.batch = take(sizeof(Batch));
     L.counters = take(CNT_N * sizeof(uint64_t));
     L.rec = take(M * sizeof(Rec));
     L.tiles_touched = take(M * 4);
     L.rect = take(M * 8);
     L.clamp = take(M);
-    L.dup_flags = take(div_up(M, 256) * 8 + 8);   // the duplicate blocks' look-back words
+    L.dup_flags = take(div_up(M, 256) * 8 + 8);   // look-back words of the chunk cutter / the duplicate
     L.ranges = take(T * 8);
     L.order = take(T * 4);   // tile order of the persistent blends (forward and backward)
     L.order_scratch = take(TILE_ORDER_WORDS * 4);
+    L.bin = take(sizeof(BinTab));
+    L.scan_words = take(8 * (1 + (uint64_t)b.n_groups));
     L.fixed_end = o;
     L.tile_bits = tile_bits_for(T);
-    L.tile_passes = radix_passes(L.tile_bits);
-    // the tile sort counts where one chunk's tile counters fit shared memory
-    L.tile_counting = T >= 1 && T <= TC_MAX_TILES;
-    L.tc_chunks = L.tile_counting ? tc_chunks(cap) : 0u;
-    // Pairs: region A receives the duplicate's (tile, entry) pairs, region B the
-    // tile sort's first output, and radix passes alternate between them; the
-    // counting sort writes only the sorted entries, into B. The depth sort's
-    // four buffers live in B: B is first written by the tile sort, after the
-    // duplicate has read the depth order. The backward reads only the final
-    // entries (B when counting, else A after an even number of passes, B after
-    // an odd one).
+    L.tile_passes = L.chunked ? 0 : radix_passes(L.tile_bits);
+    const bool keys = T > kNoKeyTiles;   // the layout keeps the sorted tile ids
+    // Pairs: region A receives the depth-ordered (tile, entry) pairs, region B the
+    // placed ones (radix passes alternate between the two). The depth sort's
+    // four buffers live in B: B is first written by the placement, after
+    // the pairs' kernel has read the depth order. The backward reads only the final
+    // entries (chunked: B; radix: A after an even number of passes, B after an odd one).
     const size_t pairs4 = al(cap * 4), m4 = al(M * 4);
-    // (the counting sort's keys are 16-bit)
-    const size_t A = take(L.tile_counting ? al(cap * 2) + pairs4 : 2 * pairs4);
-    const size_t B = take(std::max((L.tile_counting ? 1 : 2) * pairs4, 4 * m4));
+    const size_t A = take(keys ? 2 * pairs4 : al(cap * 2) + pairs4);
+    const size_t B = take(std::max((keys ? 2 : 1) * pairs4, 4 * m4));
     L.dkey0 = B;
     L.dval0 = B + m4;
     L.dkey1 = B + 2 * m4;
     L.dval1 = B + 3 * m4;
-    if (L.tile_counting) {
-        L.pkey_final = NO_OFFSET;
-        L.pval_final = B;
+    if (L.chunked) {
+        L.pkey_final = keys ? B : NO_OFFSET;
+        L.pval_final = keys ? B + pairs4 : B;
         L.pkey_tmp = A;
         L.pval_tmp = A + al(cap * 2);
     } else {
@@ -289,13 +302,13 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
         L.pkey_tmp = tmp;
         L.pval_tmp = tmp + pairs4;
     }
-    // look-back flags of the depth sort's 4 passes, then those of the tile
-    // sort's radix passes or the counting sort's [chunks][row] count matrix
-    const uint64_t tile_words = L.tile_counting ? (uint64_t)L.tc_chunks * tc_row(T)
-                                                : (uint64_t)L.tile_passes * div_up(cap, RS_TILE) * RS_RADIX;
-    const uint64_t flag_words = std::max<uint64_t>(4 * div_up(M, RS_TILE) * RS_RADIX, tile_words);
+    // look-back flags of the depth sort's passes (one more with several views),
+    // then the binning's count matrix or the flags of the tile sort's radix passes
+    const uint64_t tile_words = L.chunked ? (uint64_t)bin_rows(cap, L.bin_row) * L.bin_row
+                                          : sort_flag_words(cap, L.tile_passes);
+    const uint64_t flag_words = std::max<uint64_t>(sort_flag_words(M, b.n_views > 1 ? 5 : 4), tile_words);
     L.hist = take(flag_words * 4);
-    L.scan_sums = take(SORT_AUX_BYTES);   // the depth sort's aux
+    L.aux_depth = take(SORT_AUX_BYTES);
     L.aux_tile = take(SORT_AUX_BYTES);
     L.total = o;
     L.M = M;
@@ -357,11 +370,10 @@ void fill_sizes(const Batch &b, const WsLayout &L, uint64_t n_pairs, sg_sizes *o
     out->n_pairs = n_pairs;
     out->pair_capacity = L.cap;
     out->ws_fixed_bytes = make_layout(b, 0).total;
-    // pair buffers (32-bit keys and entries twice; the counting sort's 16-bit
-    // keys and entries, then the sorted entries), plus the radix passes'
-    // look-back words or, below the counting sort's chunk limit, its count
-    // matrix rows
-    out->ws_per_pair_bytes = L.tile_counting ? 10 + div_up(4 * tc_row(b.n_tiles), TC_CHUNK_TARGET) : 17;
+    // pair buffers (16-bit tile ids and entries, then the placed entries; with
+    // sorted tile ids kept, 32-bit ids and entries twice), plus a share of the
+    // count matrix or of the radix passes' look-back words
+    out->ws_per_pair_bytes = b.n_tiles > kNoKeyTiles ? 17 : 10 + div_up(4 * (uint64_t)L.bin_row, kMatrixShare);
     out->ws_bytes = L.total;
     out->bwd_ws_bytes = bwd_bytes(b);
 }
@@ -450,83 +462,107 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
     uint64_t *dup_flags = reinterpret_cast<uint64_t *>(w + L.dup_flags);
     uint2 *ranges = reinterpret_cast<uint2 *>(w + L.ranges);
     uint32_t *hist = reinterpret_cast<uint32_t *>(w + L.hist);
-    uint64_t *sums = reinterpret_cast<uint64_t *>(w + L.scan_sums);
+    SortAux *aux_depth = reinterpret_cast<SortAux *>(w + L.aux_depth), *aux_tile = reinterpret_cast<SortAux *>(w + L.aux_tile);
+    BinTab *tab = reinterpret_cast<BinTab *>(w + L.bin);
     const uint64_t M = L.M;
 
     const bool counting = (prof().flags & SG_PROFILE_COUNT) != 0;
-    uint64_t *aux_tile = reinterpret_cast<uint64_t *>(w + L.aux_tile);
     {
-        // the setup kernel also marks every tile range empty and clears both sorts' scratch
+        // the setup kernel also clears the sorts' scratch, the binning's totals
+        // and look-back words (chunked) or marks every tile range empty (radix)
         ZeroRegions z;
-        z.ptr[0] = reinterpret_cast<uint32_t *>(ranges);
-        z.words[0] = 2 * L.n_tiles;
-        z.even[0] = RANGE_EMPTY;
-        z.ptr[1] = reinterpret_cast<uint32_t *>(sums);
-        z.words[1] = SORT_AUX_BYTES / 4;
-        z.ptr[2] = reinterpret_cast<uint32_t *>(aux_tile);
-        z.words[2] = SORT_AUX_BYTES / 4;
-        z.ptr[3] = reinterpret_cast<uint32_t *>(dup_flags);
-        z.words[3] = 2 * div_up(M, 256);
-        z.ptr[4] = reinterpret_cast<uint32_t *>(w + L.order_scratch);
-        z.words[4] = TILE_ORDER_WORDS;
+        int r = 0;
+        auto zero = [&](void *ptr, uint64_t words, uint32_t even = 0u) {
+            z.ptr[r] = static_cast<uint32_t *>(ptr);
+            z.words[r] = words;
+            z.even[r++] = even;
+        };
+        zero(aux_depth, sizeof(SortAux) / 4);
+        zero(dup_flags, 2 * div_up(M, 256));
+        zero(w + L.order_scratch, TILE_ORDER_WORDS);
+        zero(tab, sizeof(tab->view_pairs) / 4);
+        if (L.chunked) {
+            zero(w + L.scan_words, 2 * (1 + (uint64_t)b.n_groups));
+        } else {
+            zero(aux_tile, sizeof(SortAux) / 4);
+            zero(ranges, 2 * L.n_tiles, RANGE_EMPTY);
+        }
         StageTimer t(ST_SETUP, stream);
         SG_CUDA(launch_setup(b, db, counters, stream, z), "setup");
     }
     {
         StageTimer t(ST_PRE, stream);
-        SG_CUDA(launch_preprocess(b, db, rec, tt, rect, dkey0, dval0, reinterpret_cast<uint8_t *>(w + L.clamp),
-                                  stream),
+        SG_CUDA(launch_preprocess(b, db, rec, tt, rect, dkey0, reinterpret_cast<uint8_t *>(w + L.clamp),
+                                  tab->view_pairs, aux_depth->hist[VIEW_PASS], stream),
                 "preprocessSG");
     }
     {
-        // depth digits, once per entry (result back in dkey0/dval0 after 4 passes)
+        // once per entry; entries that reach no tile are left out of the order
         StageTimer t(ST_DEPTH_SORT, stream);
-        // entries that reach no tile carry the drop key and are left out of the order
-        SG_CUDA(launch_radix_sort(dkey0, dval0, dkey1, dval1, counters + CNT_ENTRIES, M, 32, hist, sums,
-                                  stream, counters + CNT_STATUS, counters + CNT_VISIBLE, true),
+        SG_CUDA(launch_depth_sort(db, n_views, dkey0, dval0, dkey1, dval1, counters + CNT_ENTRIES, M, hist, aux_depth,
+                                  stream),
                 "depth sort");
     }
+    const uint32_t *order = n_views > 1 ? dval1 : dval0;   // entries by (view, depth)
     CountReadback *rb = nullptr;   // plain form: where the duplicate leaves the pair count for the host
     if (sync) SG_CUDA(count_readback(rb), "pair count readback");
     // grids sized by the capacity (at most SORT_MAX_KEYS pairs); counts read on the device
     const uint64_t cap_dev = std::min<uint64_t>(cap, SORT_MAX_KEYS);
-    uint64_t K = cap_dev;
-    // duplicate into the buffer from which the tile sort ends in *_final: the
-    // counting sort and an odd number of radix passes write the other buffer
-    uint32_t *pk_final = L.tile_counting ? nullptr : reinterpret_cast<uint32_t *>(w + L.pkey_final);
+    uint32_t *pk_final = L.pkey_final == NO_OFFSET ? nullptr : reinterpret_cast<uint32_t *>(w + L.pkey_final);
     uint32_t *pv_final = reinterpret_cast<uint32_t *>(w + L.pval_final);
     uint32_t *pk_tmp = reinterpret_cast<uint32_t *>(w + L.pkey_tmp);
     uint32_t *pv_tmp = reinterpret_cast<uint32_t *>(w + L.pval_tmp);
-    const bool dup_final = !L.tile_counting && (L.tile_passes % 2) == 0;
-    uint32_t *k0 = dup_final ? pk_final : pk_tmp, *v0 = dup_final ? pv_final : pv_tmp;
-    uint32_t *k1 = dup_final ? pk_tmp : pk_final, *v1 = dup_final ? pv_tmp : pv_final;
-    {
-        StageTimer t(ST_DUPLICATE, stream);
-        // radix: also the tile sort's digit histograms and cleared look-back flags
-        // the pair offsets come from the duplicate blocks' own look-back (no scan kernel)
-        const int hp = L.tile_counting ? 0 : L.tile_passes;
-        SG_CUDA(launch_duplicate(db, M, dval0, tt, rect, rec, counters, cap_dev, k0, v0, dup_flags,
-                                 rb ? rb->dev_ptr : nullptr, stream, hp, hp ? aux_tile : nullptr,
-                                 hp ? hist : nullptr, hp ? sort_flag_words(K, L.tile_bits) : 0, L.tile_counting),
-                "duplicateWithKeys");
-    }
-    if (L.tile_counting) {
+    uint64_t *mirror = rb ? rb->dev_ptr : nullptr;   // plain form: pair count and status for the host
+    uint32_t *order_counts = reinterpret_cast<uint32_t *>(w + L.order_scratch);
+    if (L.chunked) {
+        BinArgs a{};
+        a.db = db;
+        a.n_views = n_views;
+        a.M = M;
+        a.cap = cap_dev;
+        a.max_chunks = L.bin_chunks;
+        a.row = L.bin_row;
+        a.n_groups = b.n_groups;
+        a.n_tiles = b.n_tiles;
+        a.sorted_ent = order;
+        a.aux = aux_depth;
+        a.tiles_touched = tt;
+        a.rect = rect;
+        a.rec = rec;
+        a.counters = counters;
+        a.tab = tab;
+        a.poff = dkey1;   // the depth keys are no longer needed
+        a.flags = dup_flags;
+        a.pkey = reinterpret_cast<uint16_t *>(pk_tmp);
+        a.pval = pv_tmp;
+        a.matrix = hist;
+        a.words = reinterpret_cast<uint64_t *>(w + L.scan_words);
+        a.ranges = ranges;
+        a.order_counts = order_counts;
+        a.ovals = pv_final;
+        a.okeys = pk_final;
+        a.mirror = mirror;
+        {
+            StageTimer t(ST_DUPLICATE, stream);
+            SG_CUDA(launch_bin_pairs(a, stream), "duplicateWithKeys");
+        }
         StageTimer t(ST_TILE_SORT, stream);
-        // also the tile ranges and the tile order's bucket counts; the plain
-        // form's status word goes to the host word next to the pair count
-        SG_CUDA(launch_tile_count_sort(reinterpret_cast<const uint16_t *>(k0), v0, v1, counters, cap_dev,
-                                       (uint32_t)L.n_tiles, L.tc_chunks, hist,
-                                       aux_tile, ranges, reinterpret_cast<uint32_t *>(w + L.order_scratch),
-                                       rb ? rb->dev_ptr + 1 : nullptr, stream),
-                "tile sort");
+        SG_CUDA(launch_bin_place(a, stream), "tile sort");
     } else {
+        // duplicate into the buffer from which the radix passes end in *_final
+        const bool dup_final = L.tile_passes % 2 == 0;
+        uint32_t *k0 = dup_final ? pk_final : pk_tmp, *v0 = dup_final ? pv_final : pv_tmp;
+        uint32_t *k1 = dup_final ? pk_tmp : pk_final, *v1 = dup_final ? pv_tmp : pv_final;
+        {
+            StageTimer t(ST_DUPLICATE, stream);
+            SG_CUDA(launch_duplicate(db, M, order, aux_depth, tt, rect, rec, counters, cap_dev, k0, v0, dup_flags,
+                                     mirror, stream, L.tile_passes, aux_tile, hist,
+                                     sort_flag_words(cap_dev, L.tile_passes)),
+                    "duplicateWithKeys");
+        }
         StageTimer t(ST_TILE_SORT, stream);
-        // the last pass also bounds every tile's range in the sorted pairs
-        // plain form: the sorts' merged status also goes to the host word next to the pair count
-        SG_CUDA(launch_radix_sort(k0, v0, k1, v1, counters + CNT_WRITTEN, K, L.tile_bits, hist, aux_tile, stream,
-                                  counters + CNT_STATUS, nullptr, true, ranges, L.n_tiles, true,
-                                  rb ? rb->dev_ptr + 1 : nullptr, counters + CNT_STATUS,
-                                  reinterpret_cast<uint32_t *>(w + L.order_scratch)),
+        SG_CUDA(launch_tile_radix_sort(k0, v0, k1, v1, counters, cap_dev, L.tile_bits, hist, aux_tile, ranges,
+                                       L.n_tiles, order_counts, mirror ? mirror + 1 : nullptr, stream),
                 "tile sort");
     }
     if (sync) SG_CUDA(cudaEventRecord(rb->ev, stream), "read pairs");
@@ -547,8 +583,7 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
     {
         // built for every forward: the persistent backward walks tiles in this order too
         StageTimer t(ST_RANGES, stream);
-        SG_CUDA(launch_tile_order(ranges, b.n_tiles, reinterpret_cast<uint32_t *>(w + L.order),
-                                  reinterpret_cast<uint32_t *>(w + L.order_scratch), stream),
+        SG_CUDA(launch_tile_order(ranges, b.n_tiles, reinterpret_cast<uint32_t *>(w + L.order), order_counts, stream),
                 "tile order");
     }
     {
@@ -579,9 +614,10 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
             return fail(SG_ERR_CAPACITY, "%llu pairs exceed the workspace capacity %llu (need %zu bytes)",
                         (unsigned long long)n_pairs, (unsigned long long)cap, need.total);
         }
-        K = n_pairs;
+        fill_sizes(b, L, n_pairs, out);
+        return SG_OK;
     }
-    fill_sizes(b, L, K, out);
+    fill_sizes(b, L, cap_dev, out);
     return SG_OK;
 }
 
@@ -755,7 +791,7 @@ static int layout_of(const sg_scene *scenes, int n_scenes, const sg_camera *cams
     out->rec = L.rec;
     out->tiles_touched = L.tiles_touched;
     out->rect = L.rect;
-    out->depth_order = L.dval0;
+    out->depth_order = n_views > 1 ? L.dval1 : L.dval0;
     out->ranges = L.ranges;
     out->pair_tile = L.pkey_final;
     out->pair_entry = L.pval_final;

@@ -28,7 +28,7 @@ struct ViewDesc {
     int32_t scene;        // index into Batch::scene
     int32_t n;            // Gaussians of that scene
     uint32_t tile_off;    // first global tile id of the view
-    uint32_t pad1;
+    uint32_t grp_off;     // first group of 32 tiles of the view (the binning's scan)
     uint32_t pad0;
     uint64_t pix_off;     // first pixel of the view in T_final / last (img: x3)
     uint64_t ent_off;     // first (view, Gaussian) entry of the view
@@ -53,7 +53,7 @@ struct Batch {
     uint32_t n_tiles;
     uint32_t scene_blocks;   // blocks of 256 scene Gaussians over all scenes
     uint32_t max_views_per_scene;
-    uint32_t pad0;
+    uint32_t n_groups;       // groups of 32 tiles over all views
     uint64_t n_entries;
     ViewDesc view[SG_MAX_VIEWS];
     SceneDesc scene[SG_MAX_SCENES];
@@ -75,10 +75,9 @@ enum : int {
     CNT_EVALS = 3,     // pair evaluations (counting kernels)
     CNT_TILES = 4,     // tiles
     CNT_QUEUE = 5,     // persistent-blend work counter
-    CNT_VISIBLE = 6,   // entries with at least one pair (the depth order's length)
-    CNT_DUP_BLOCK = 7, // duplicate kernel: next logical block
-    CNT_WRITTEN = 8,   // pairs the duplicate wrote (min(pairs, capacity)): the tile sort's count
-    CNT_N = 10
+    CNT_DUP_BLOCK = 6, // chunk cutter / duplicate kernel: next logical block
+    CNT_WRITTEN = 7,   // pairs written (min(pairs, capacity)): the tile sort's count
+    CNT_N = 8
 };
 
 // Radix sort / scan geometry.
@@ -95,13 +94,13 @@ constexpr int SCAN_TILE = 4096;
 // forward and the backward of one call).
 struct WsLayout {
     size_t batch, counters, rec, tiles_touched, rect, clamp, dkey0, dval0, dkey1, dval1,
-        dup_flags, ranges, order, order_scratch, scan_sums, hist, aux_tile, fixed_end;
+        dup_flags, ranges, order, order_scratch, bin, scan_words, hist, aux_depth, aux_tile, fixed_end;
     size_t pval_final, pkey_final, pval_tmp, pkey_tmp, total;
     uint64_t M, n_tiles, cap;
     int tile_bits, tile_passes;
-    bool tile_counting;   // the tile sort counts (launch_tile_count_sort) instead of radix passes:
-    uint32_t tc_chunks;   // its chunks; its count matrix takes the look-back flags' region and
-                          // no sorted keys are kept (pkey_final = NO_OFFSET)
+    bool chunked;         // tile sort by chunks (launch_bin) instead of radix passes
+    uint32_t bin_chunks;  // most chunks; their count matrix takes the look-back flags' region
+    uint32_t bin_row;     // words per row of the matrix: the largest view's tiles, padded to 4
 };
 
 __host__ __device__ inline uint64_t div_up(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
@@ -316,6 +315,12 @@ __device__ __forceinline__ void chain_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// For a kernel whose successor needs most of an SM's shared memory: without the
+// early trigger the successor's blocks are only placed once this kernel has
+// drained, evenly over the SMs, instead of wherever it leaves room (measured
+// on the placement after the scan: 328 -> 175 us at 11.8M pairs).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_chain_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                      cudaStream_t s, Args &&...args) {
@@ -346,16 +351,19 @@ void count_launches(int n);
 // Regions the setup kernel fills: word i of region r gets even[r] if i is
 // even, else 0 (even[r] = 0: plain zeroing).
 struct ZeroRegions {
-    static constexpr int N = 5;
-    uint32_t *ptr[N] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    uint64_t words[N] = {0, 0, 0, 0, 0};
-    uint32_t even[N] = {0, 0, 0, 0, 0};
+    static constexpr int N = 6;
+    uint32_t *ptr[N] = {};
+    uint64_t words[N] = {};
+    uint32_t even[N] = {};
 };
 cudaError_t launch_setup(const Batch &b, Batch *dst, uint64_t *counters, cudaStream_t s,
                          const ZeroRegions &z = ZeroRegions());
-// clamp [M]: bit ch set where colour channel ch was clamped by max(c, 0)
+// clamp [M]: bit ch set where colour channel ch was clamped by max(c, 0).
+// view_pairs, view_visible (zeroed): receive each view's pairs and its entries
+// with at least one pair.
 cudaError_t launch_preprocess(const Batch &hb, const Batch *db, Rec *rec, uint32_t *tiles_touched,
-                              uint2 *rect, uint32_t *dkey, uint32_t *dval, uint8_t *clamp, cudaStream_t s);
+                              uint2 *rect, uint32_t *dkey, uint8_t *clamp,
+                              unsigned long long *view_pairs, uint32_t *view_visible, cudaStream_t s);
 cudaError_t launch_preprocess_backward(const Batch &hb, const Batch *db,
                                        const uint32_t *tiles_touched, const uint8_t *clamp, const float *dg,
                                        uint64_t M, cudaStream_t s);
@@ -369,89 +377,125 @@ cudaError_t launch_scan(const uint32_t *in, const uint32_t *gather_idx, uint32_t
                         const uint64_t *n_dev = nullptr, uint64_t *mirror = nullptr,
                         const uint64_t *status_src = nullptr);
 
-// Stable LSD radix sort of (key, val) u32 pairs on bits [0, bits); item count read
-// from *n_dev and clamped to max_n (the capacity the launch is sized for, below
-// 2^30). Ping-pongs between (k0,v0) and (k1,v1); the sorted result ends in
-// (k0,v0) when the pass count is even, else in (k1,v1).
-// hist: 4 x RS_RADIX x ceil(max_n / RS_TILE) words of look-back flags (one region
-// per pass, zeroed by the sort itself); aux: at least
-// SORT_AUX_BYTES; status (nullable): set to SG_ERR_TIMEOUT if a look-back gave up.
-// kept_out (nullable): drop mode — keys equal to SORT_DROP_KEY are left out, the
-// sorted kept keys fill positions [0, *kept_out) and *kept_out receives their count.
 constexpr size_t SORT_AUX_BYTES = 16384;
 // Most keys one sort takes (its look-back words carry 30-bit counts).
 constexpr uint64_t SORT_MAX_KEYS = (1ull << 30) - 1;
 constexpr uint32_t SORT_DROP_KEY = 0xFFFFFFFFu;
-// aux_zeroed: the caller has already zeroed the aux region in this stream.
-// hist_ready: the caller has also written every pass's digit histogram into
-// aux and zeroed the sort_flag_words(max_n, bits) look-back words of hist.
-// status_mirror (nullable): receives *status after the sort (host memory mapped
-// into the device, read by the host behind an event).
-// skip_status (nullable): when it holds a status other than SG_OK (a bounded
-// wait gave up, so the input may hold stale words the histograms do not count;
-// or the pairs overflowed the capacity) the passes do nothing.
-// ranges (nullable): keys are ids below n_ranges; the sort also writes each
-// id's [first, last + 1) position range in the sorted output, (0, 0) for an id
-// with no key. On entry every range must hold (RANGE_EMPTY, 0).
-constexpr uint32_t RANGE_EMPTY = 0xFFFFFFFFu;
-cudaError_t launch_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
-                              const uint64_t *n_dev, uint64_t max_n, int bits, uint32_t *hist,
-                              uint64_t *aux, cudaStream_t s, uint64_t *status = nullptr,
-                              uint64_t *kept_out = nullptr, bool aux_zeroed = false, uint2 *ranges = nullptr,
-                              uint64_t n_ranges = 0, bool hist_ready = false, uint64_t *status_mirror = nullptr,
-                              const uint64_t *skip_status = nullptr, uint32_t *order_counts = nullptr);
 int radix_passes(int bits);
 // Bound on a sort block's polls of an unpublished predecessor before it gives
 // up and records SG_ERR_TIMEOUT (0: the default, 2^20).
 void set_sort_wait_polls(uint32_t polls);
 uint32_t sort_wait_polls();
-// Look-back flag words a sort of up to max_n keys of `bits` bits uses.
-uint64_t sort_flag_words(uint64_t max_n, int bits);
+// Look-back flag words of `passes` passes over up to max_n keys.
+uint64_t sort_flag_words(uint64_t max_n, int passes);
 
-// duplicateWithKeys over the depth-sorted entries. Every block of 256 entries
-// finds the offset of its pairs by a decoupled look-back over its predecessors'
-// pair counts (dup_flags: div_up(M, 256) zeroed 64-bit words, and
-// counters[CNT_DUP_BLOCK] zeroed), so no separate scan runs. The last block
+// Stable sort of the entries by (view, depth bits), entries whose key in k0 is
+// SORT_DROP_KEY left out (k0: one key per entry; the values, entry indices, are
+// made by the first pass): the four depth digits, then, with several views, one pass whose
+// digit is the entry's view (its counts, aux hist row VIEW_PASS, are
+// preprocess's). The order ends in (k0, v0) with one view, in (k1, v1) with
+// several; aux (zeroed by the caller) then holds the kept count and the status.
+constexpr int VIEW_PASS = 4;
+struct SortAux {
+    uint32_t hist[5][RS_RADIX];   // global digit counts per pass
+    uint32_t tile_ctr[5];         // tile counter per pass
+    uint32_t status;              // 0 or SG_ERR_TIMEOUT
+    uint64_t kept;                // keys other than SORT_DROP_KEY (drop mode)
+};
+static_assert(sizeof(SortAux) <= SORT_AUX_BYTES, "sort aux region");
+cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
+                              const uint64_t *n_dev, uint64_t max_n, uint32_t *hist, SortAux *aux, cudaStream_t s);
+
+// ---------------------------------------------------------------------------
+// Binning by chunks: (tile, entry) pairs in (tile, depth, entry) order without
+// a sort of the pairs by key digits, for views of up to BIN_MAX_ROW tiles (one
+// chunk's tile counters fit shared memory). The depth-ordered entries of each
+// view are cut into chunks of about equal cost; each chunk counts its
+// pairs per tile while it writes them out, one scan of the count matrix gives
+// every (chunk, tile) its first output position and every tile its range, and
+// each chunk places its pairs in order. Larger views take launch_duplicate and
+// radix passes over the tile digits.
+// ---------------------------------------------------------------------------
+constexpr uint32_t BIN_MAX_ROW = 56 * 1024;
+// Fewest pairs a chunk is cut for: one placing warp walks 32 pairs a round.
+constexpr uint32_t BIN_MIN_CHUNK = 256;
+// An entry's share of a chunk's cost besides its pairs (one each).
+constexpr uint32_t BIN_ENTRY_COST = 1;
+constexpr uint32_t BIN_MAX_CHUNKS = 6 * 152;
+// Per-call tables of the binning (workspace; view_pairs zeroed by the setup kernel).
+struct BinTab {
+    unsigned long long view_pairs[SG_MAX_VIEWS];   // pairs of each view (preprocess)
+    uint32_t n_chunks;                             // chunks in use
+    uint32_t first_chunk[SG_MAX_VIEWS + 1];        // first chunk of each view
+    uint32_t start[BIN_MAX_CHUNKS + 1];            // first entry (depth order) of each chunk
+    uint32_t pair[BIN_MAX_CHUNKS + 1];             // first pair of each chunk
+};
+uint32_t bin_rows(uint64_t cap, uint32_t row);     // rows of the count matrix of a call with room for cap pairs
+uint32_t bin_chunks(uint64_t cap, uint32_t row);   // and the most chunks it uses
+struct BinArgs {
+    const Batch *db;
+    int n_views;
+    uint64_t M, cap;                 // entries; pairs the buffers hold (below 2^30)
+    uint32_t max_chunks, row, n_groups, n_tiles;
+    const uint32_t *sorted_ent;      // the depth sort's order
+    const SortAux *aux;              // its kept count and status
+    const uint32_t *tiles_touched;
+    const uint2 *rect;
+    const Rec *rec;
+    uint64_t *counters;
+    BinTab *tab;
+    uint32_t *poff;                  // scratch, M words: first pair of each entry of the order
+    uint64_t *flags;                 // zeroed, one word per BIN_BLOCK entries: look-back
+    uint16_t *pkey;                  // depth-ordered pairs: tile inside the view
+    uint32_t *pval;                  //   and entry
+    uint32_t *matrix;                // max_chunks x row words
+    uint64_t *words;                 // zeroed, 1 + n_groups: ticket and look-back of the scan
+    uint2 *ranges;                   // every tile's [first, last + 1) ((0, 0): none)
+    uint32_t *order_counts;          // zeroed tile-order bucket counts
+    uint32_t *ovals;                 // the placed entries
+    uint32_t *okeys;                 // nullable: their global tile ids
+    uint64_t *mirror;                // nullable host words: [0] pairs, [1] status
+};
+constexpr int BIN_ITEMS = 8, BIN_BLOCK = 256 * BIN_ITEMS;   // entries per thread and block of the chunk cutter
+cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s);   // chunks and their pairs
+cudaError_t launch_bin_place(const BinArgs &a, cudaStream_t s);   // scan and placement
+
+// duplicateWithKeys over the depth-sorted entries, for the radix tile sort.
+// Every block of 256 entries finds the offset of its pairs by a decoupled
+// look-back over its predecessors' pair counts (dup_flags: div_up(M, 256) zeroed
+// 64-bit words, and counters[CNT_DUP_BLOCK] zeroed), so no separate scan runs.
+// The entry count and the depth sort's status come from aux. The last block
 // writes the pair total to counters[CNT_PAIRS] (and to mirror[0], host memory
 // mapped into the device, when given), min(total, cap) to counters[CNT_WRITTEN],
 // and SG_ERR_CAPACITY to counters[CNT_STATUS] when the pairs exceed cap; pairs
-// at positions >= cap are not written. A status of SG_ERR_TIMEOUT on entry
-// (a sort gave up a bounded wait) makes the kernel write nothing.
-// key16: the keys are written as uint16_t (tile ids below 2^16, for the
-// counting tile sort; no digit histograms then), else as uint32_t.
-cudaError_t launch_duplicate(const Batch *db, uint64_t M, const uint32_t *sorted_ent,
+// at positions >= cap are not written. It also clears the tile sort's look-back
+// flags and builds its digit histograms.
+cudaError_t launch_duplicate(const Batch *db, uint64_t M, const uint32_t *sorted_ent, const SortAux *depth_aux,
                              const uint32_t *tiles_touched, const uint2 *rect, const Rec *rec,
-                             uint64_t *counters, uint64_t cap, void *pkey, uint32_t *pval,
-                             uint64_t *dup_flags, uint64_t *mirror, cudaStream_t s, int hist_passes = 0,
-                             uint64_t *sort_aux = nullptr, uint32_t *flags = nullptr, uint64_t flag_words = 0,
-                             bool key16 = false);
-// Tile sort by counting, for tile counts up to TC_MAX_TILES (one chunk's
-// counters fit 48 KB of shared memory): a stable sort by tile of the
-// duplicate's (tile, entry) pairs, the same order as launch_radix_sort's, in
-// three kernels with no pass over the key bits; the keys (tile ids) are
-// 16-bit, as the duplicate writes them for it. Only the entries are written
-// (ovals, cap words): a pair's tile is the tile whose range holds it. The pair
-// count is min(counters[CNT_WRITTEN], cap), none when counters[CNT_STATUS] is
-// not SG_OK on entry. matrix: n_chunks x tc_row(n_tiles) words (no zeroing
-// needed); words: zeroed, 8 + 8 * ceil(n_tiles / 32) bytes; ranges: every
-// tile's [first, last + 1) in the output ((0, 0) when empty); order_counts:
-// the tile order's zeroed bucket counts, incremented here; status_mirror
-// (nullable): receives counters[CNT_STATUS] after the sort. cap below 2^32.
-constexpr uint32_t TC_MAX_TILES = 12288;
-#ifndef SG_TC_MAX_CHUNKS
-#define SG_TC_MAX_CHUNKS 608
-#endif
-constexpr uint32_t TC_MAX_CHUNKS = SG_TC_MAX_CHUNKS;   // four one-warp placing blocks per SM
-constexpr uint64_t TC_CHUNK_TARGET = 8192;            // pairs per chunk when the capacity is small
-uint32_t tc_chunks(uint64_t cap);                      // chunks of a sort sized for cap pairs
-uint64_t tc_row(uint64_t n_tiles);                     // words per row of the count matrix (multiple of 4)
-cudaError_t launch_tile_count_sort(const uint16_t *keys, const uint32_t *vals, uint32_t *ovals,
-                                   uint64_t *counters, uint64_t cap, uint32_t n_tiles, uint32_t n_chunks,
-                                   uint32_t *matrix, uint64_t *words, uint2 *ranges, uint32_t *order_counts,
-                                   uint64_t *status_mirror, cudaStream_t s);
+                             uint64_t *counters, uint64_t cap, uint32_t *pkey, uint32_t *pval,
+                             uint64_t *dup_flags, uint64_t *mirror, cudaStream_t s, int hist_passes,
+                             SortAux *sort_aux, uint32_t *flags, uint64_t flag_words);
+// Stable LSD radix sort by tile id of launch_duplicate's (key, val) pairs on
+// bits [0, bits); counters[CNT_WRITTEN] of them, at most max_n (below 2^30).
+// Ping-pongs between (k0,v0) and (k1,v1); the result ends in (k0,v0) when the
+// pass count is even, else in (k1,v1). hist: the sort_flag_words(max_n, passes)
+// look-back words, aux: the digit histograms, both prepared by
+// launch_duplicate. Nothing is sorted when counters[CNT_STATUS] is not SG_OK on
+// entry (a bounded wait gave up: the input may hold stale words; or the pairs
+// overflowed the capacity); a look-back that gives up sets it to
+// SG_ERR_TIMEOUT. ranges: every tile's [first, last + 1) positions, (0, 0) for
+// a tile with no pair; on entry every range must hold (RANGE_EMPTY, 0).
+// order_counts: the tile order's zeroed bucket counts, incremented here.
+// status_mirror (nullable, host memory mapped into the device): receives the
+// status after the sort.
+constexpr uint32_t RANGE_EMPTY = 0xFFFFFFFFu;
+cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, uint64_t *counters,
+                                   uint64_t max_n, int bits, uint32_t *hist, SortAux *aux, uint2 *ranges,
+                                   uint64_t n_ranges, uint32_t *order_counts, uint64_t *status_mirror,
+                                   cudaStream_t s);
 // Tiles by descending list length (256 length buckets) into order[n_tiles].
 // scratch: TILE_ORDER_WORDS zeroed words whose first 256 already hold the
-// bucket counts (launch_radix_sort's order_counts, filled by its finish kernel).
+// bucket counts (filled by the tile sort).
 constexpr int TILE_ORDER_WORDS = 512;
 cudaError_t launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t *scratch,
                               cudaStream_t s);

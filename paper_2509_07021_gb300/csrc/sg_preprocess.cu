@@ -396,21 +396,21 @@ __device__ __forceinline__ void load_colour_base(const SceneDesc &sc, int64_t g,
     cb.lo = max(0, min(__ldg(sc.lobe_off + g), cb.hi));
 }
 
+// Returns the entry's tiles_touched.
 template <int DL, int DS, int CM>
-__device__ __forceinline__ void preprocess_entry(const ViewDesc &vw, const SceneDesc &sc, int64_t g, float px,
+__device__ __forceinline__ uint32_t preprocess_entry(const ViewDesc &vw, const SceneDesc &sc, int64_t g, float px,
                                                  float py, float pz, const Geo3 &g3, float o, float gm,
                                                  const ColourBase &cb, uint64_t e,
                                                  Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
-                                                 uint2 *__restrict__ rect, uint32_t *__restrict__ dkey,
-                                                 uint32_t *__restrict__ dval, uint8_t *__restrict__ clamp) {
+                                                 uint2 *__restrict__ rect,
+                                                 uint32_t *__restrict__ dkey, uint8_t *__restrict__ clamp) {
     Geo G;
     project_view(vw, px, py, pz, g3, o, gm, G);
     if (!G.visible) {
         tiles_touched[e] = 0u;
         rect[e] = make_uint2(0u, 0u);
         dkey[e] = SORT_DROP_KEY;
-        dval[e] = (uint32_t)e;
-        return;
+        return 0u;
     }
 
     // SG colour (Eq. 2): view direction from the camera centre to the Gaussian
@@ -466,27 +466,32 @@ __device__ __forceinline__ void preprocess_entry(const ViewDesc &vw, const Scene
     tiles_touched[e] = touched;
     rect[e] = make_uint2((uint32_t)G.x0 | ((uint32_t)G.x1 << 16), (uint32_t)G.y0 | ((uint32_t)G.y1 << 16));
     dkey[e] = touched ? __float_as_uint(G.tz) : SORT_DROP_KEY;   // no pair: not depth-sorted
-    dval[e] = (uint32_t)e;
+    return touched;
 }
 
 // One thread per scene Gaussian: its parameters are read once and projected
 // into every view of the call that shows its scene. ONE_VIEW: no scene has
 // more than one view, so the walk stops at the first (the parameters need not
-// stay live across views).
-#ifndef SG_PRE_MIN_BLOCKS
-#define SG_PRE_MIN_BLOCKS 1
-#endif
+// stay live across views). Each block also adds its pairs and its entries with
+// a pair to the view's totals (view_pairs, view_visible), which the binning
+// cuts its chunks by: a warp reduction per view, then one atomic per block.
 template <int DG, int DL, int DS, int CM, bool ONE_VIEW>
-__global__ void __launch_bounds__(PRE_THREADS, SG_PRE_MIN_BLOCKS)
+__global__ void __launch_bounds__(PRE_THREADS, ONE_VIEW ? 1 : CM == SG_COLOR_SH3 ? 2 : 3)
 k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
-             uint2 *__restrict__ rect, uint32_t *__restrict__ dkey, uint32_t *__restrict__ dval,
-             uint8_t *__restrict__ clamp) {
+             uint2 *__restrict__ rect, uint32_t *__restrict__ dkey,
+             uint8_t *__restrict__ clamp, unsigned long long *__restrict__ view_pairs,
+             uint32_t *__restrict__ view_visible) {
     chain_enter();
+    constexpr int NV = ONE_VIEW ? 1 : SG_MAX_VIEWS;
+    __shared__ uint32_t s_pairs[NV], s_vis[NV];
     const Batch &b = *bp;
     const int si = find_block_scene(b, blockIdx.x);
     const SceneDesc &sc = b.scene[si];
-    const int64_t g = (int64_t)(blockIdx.x - sc.blk_off) * PRE_THREADS + threadIdx.x;
-    if (g >= sc.n) return;
+    for (int v = threadIdx.x; v < NV; v += PRE_THREADS) s_pairs[v] = s_vis[v] = 0u;
+    __syncthreads();
+    const int64_t gt = (int64_t)(blockIdx.x - sc.blk_off) * PRE_THREADS + threadIdx.x;
+    const bool on = gt < sc.n;
+    const int64_t g = on ? gt : sc.n - 1;   // threads past the end only take part in the reductions
     float px, py, pz, s0, s1, s2, q0, q1, q2, q3, o;
     load_geo<DG>(sc, g, px, py, pz, s0, s1, s2, q0, q1, q2, q3, o);
     const float gm = __ldg(sc.gmask + g);
@@ -494,45 +499,68 @@ k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__re
     load_colour_base<CM>(sc, g, cb);
     Geo3 g3;
     geo3_recipe(s0, s1, s2, q0, q1, q2, q3, g3);
+    int mine = 0;   // ONE_VIEW: the scene's view
     for (int v = 0; v < b.n_views; ++v) {
         const ViewDesc &vw = b.view[v];
         if (vw.scene != si) continue;
-        preprocess_entry<DL, DS, CM>(vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g, rec,
-                                     tiles_touched, rect, dkey, dval, clamp);
+        uint32_t touched = 0u;
+        if (on)
+            touched = preprocess_entry<DL, DS, CM>(vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g, rec,
+                                                   tiles_touched, rect, dkey, clamp);
+        const uint32_t pairs = __reduce_add_sync(0xffffffffu, touched);
+        const uint32_t vis = (uint32_t)__popc(__ballot_sync(0xffffffffu, touched != 0u));
+        if ((threadIdx.x & 31) == 0 && vis) {
+            atomicAdd(&s_pairs[ONE_VIEW ? 0 : v], pairs);
+            atomicAdd(&s_vis[ONE_VIEW ? 0 : v], vis);
+        }
+        mine = v;
         if (ONE_VIEW) break;
     }
+    __syncthreads();
+    for (int v = threadIdx.x; v < (ONE_VIEW ? 1 : b.n_views); v += PRE_THREADS)
+        if (s_vis[v]) {
+            const int view = ONE_VIEW ? mine : v;
+            atomicAdd(view_pairs + view, (unsigned long long)s_pairs[v]);
+            atomicAdd(view_visible + view, s_vis[v]);
+        }
 }
 
 template <int DG, int DL, int DS, int CM = SG_COLOR_SG>
 static cudaError_t launch_pre_t(const Batch &hb, const Batch *db, Rec *rec, uint32_t *tt, uint2 *rect,
-                                uint32_t *dkey, uint32_t *dval, uint8_t *clamp, cudaStream_t s) {
+                                uint32_t *dkey, uint8_t *clamp, unsigned long long *vp,
+                                uint32_t *vv, cudaStream_t s) {
     if (hb.scene_blocks == 0) return cudaSuccess;   // one block per 256 scene Gaussians
     if (hb.max_views_per_scene <= 1)
-        (void)launch_chain(k_preprocess<DG, DL, DS, CM, true>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db, rec, tt, rect, dkey, dval,
-                                                                                   clamp);
+        (void)launch_chain(k_preprocess<DG, DL, DS, CM, true>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db,
+                           rec, tt, rect, dkey, clamp, vp, vv);
     else
-        (void)launch_chain(k_preprocess<DG, DL, DS, CM, false>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db, rec, tt, rect, dkey, dval,
-                                                                                    clamp);
+        (void)launch_chain(k_preprocess<DG, DL, DS, CM, false>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db,
+                           rec, tt, rect, dkey, clamp, vp, vv);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_preprocess(const Batch &hb, const Batch *db, Rec *rec, uint32_t *tiles_touched,
-                              uint2 *rect, uint32_t *dkey, uint32_t *dval, uint8_t *clamp, cudaStream_t s) {
+                              uint2 *rect, uint32_t *dkey, uint8_t *clamp,
+                              unsigned long long *view_pairs, uint32_t *view_visible, cudaStream_t s) {
     // all scenes of one call share storage types (checked by the API layer)
     const SceneDesc &sc = hb.scene[0];
     const int key = sc.dtype_geom * 9 + sc.dtype_lobe * 3 + sc.dtype_sharp;
     if (sc.color_model == SG_COLOR_SH3) {
         if (key != SG_F32 * 9 + SG_F32 * 3 + SG_F32) return cudaErrorInvalidValue;
-        return launch_pre_t<SG_F32, SG_F32, SG_F32, SG_COLOR_SH3>(hb, db, rec, tiles_touched, rect, dkey, dval, clamp, s);
+        return launch_pre_t<SG_F32, SG_F32, SG_F32, SG_COLOR_SH3>(hb, db, rec, tiles_touched, rect, dkey, clamp,
+                                                                   view_pairs, view_visible, s);
     }
     switch (key) {
         case SG_F32 * 9 + SG_F32 * 3 + SG_F32:
-            return launch_pre_t<SG_F32, SG_F32, SG_F32>(hb, db, rec, tiles_touched, rect, dkey, dval, clamp, s);
+            return launch_pre_t<SG_F32, SG_F32, SG_F32>(hb, db, rec, tiles_touched, rect, dkey, clamp,
+                                                                   view_pairs, view_visible, s);
         case SG_F16 * 9 + SG_F16 * 3 + SG_F16:
-            return launch_pre_t<SG_F16, SG_F16, SG_F16>(hb, db, rec, tiles_touched, rect, dkey, dval, clamp, s);
+            return launch_pre_t<SG_F16, SG_F16, SG_F16>(hb, db, rec, tiles_touched, rect, dkey, clamp,
+                                                                   view_pairs, view_visible, s);
         case SG_F16 * 9 + SG_F16 * 3 + SG_BF16:
-            return launch_pre_t<SG_F16, SG_F16, SG_BF16>(hb, db, rec, tiles_touched, rect, dkey, dval, clamp, s);
+            return launch_pre_t<SG_F16, SG_F16, SG_BF16>(hb, db, rec, tiles_touched, rect, dkey, clamp,
+                                                                   view_pairs, view_visible, s);
         default:
             return cudaErrorInvalidValue;
     }

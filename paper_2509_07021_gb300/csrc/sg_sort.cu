@@ -11,11 +11,10 @@
 // stable, so the result is identical to the 64-bit sort.
 #include "sg_internal.cuh"
 
+#include <algorithm>
 #include <atomic>
 
 namespace sgk {
-
-__host__ __device__ __forceinline__ int radix_passes_dev(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     return (1u << (threadIdx.x & 31)) - 1u;
@@ -144,7 +143,7 @@ cudaError_t launch_scan(const uint32_t *in, const uint32_t *gather_idx, uint32_t
 // stable LSD radix sort, 8-bit digits, RS_TILE keys per block, one sweep per pass
 // ---------------------------------------------------------------------------
 // One kernel histograms every digit position at once (and clears the look-back
-// flags of every pass). Each pass is then a single kernel: blocks take key
+// flags of every pass; for the radix tile sort the duplicate does both). Each pass is then a single kernel: blocks take key
 // tiles in order from an atomic counter, rank their keys stably (warp
 // match_any + per-warp digit counters), scan the pass's digit histogram for
 // the digit bases, publish their digit counts, and get their offsets among
@@ -152,6 +151,15 @@ cudaError_t launch_scan(const uint32_t *in, const uint32_t *gather_idx, uint32_t
 // spin is bounded: past the bound the block records SG_ERR_TIMEOUT in the
 // status word and carries on with a smaller offset (wrong order, still inside
 // the array) instead of waiting forever.
+
+__device__ __forceinline__ int find_entry_view(const Batch &b, uint64_t e) {
+    int lo = 0, hi = b.n_views - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (b.view[mid].ent_off <= e) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
 
 // packed look-back word: 2 status bits, 30 count bits
 constexpr uint32_t LB_AGG = 1u << 30, LB_INC = 2u << 30, LB_VAL = (1u << 30) - 1u;
@@ -168,15 +176,6 @@ uint32_t sort_wait_polls() {
     return v ? v : LB_SPIN_LIMIT;
 }
 
-struct SortAux {
-    uint32_t hist[4][RS_RADIX];   // global digit counts per pass
-    uint32_t tile_ctr[4];         // tile counter per pass
-    uint32_t status;              // 0 or SG_ERR_TIMEOUT
-    uint32_t pad;
-    uint64_t kept;                // keys other than SORT_DROP_KEY (drop mode)
-};
-static_assert(sizeof(SortAux) <= SORT_AUX_BYTES, "sort aux region");
-
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t *p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -191,12 +190,12 @@ __device__ __forceinline__ void st_relaxed(uint32_t *p, uint32_t v) {
 // with few distinct digits (the high tile bits) from serialising.
 __global__ void __launch_bounds__(RS_THREADS) k_os_hist(const uint32_t *__restrict__ keys,
                                                         const uint64_t *__restrict__ n_dev, uint64_t max_n,
-                                                        int bits, bool drop, SortAux *aux,
-                                                        uint32_t *__restrict__ flags, uint64_t flag_words) {
+                                                        SortAux *aux, uint32_t *__restrict__ flags,
+                                                        uint64_t flag_words) {
     chain_enter();
     constexpr int NW = RS_THREADS / 32;
     __shared__ uint32_t h[NW][4][RS_RADIX];
-    const int passes = radix_passes_dev(bits);
+    constexpr int passes = 4;
     // the look-back flags of every pass start at zero (the passes run after this kernel)
     for (uint64_t i = (uint64_t)blockIdx.x * RS_THREADS + threadIdx.x; i < flag_words;
          i += (uint64_t)gridDim.x * RS_THREADS)
@@ -209,12 +208,10 @@ __global__ void __launch_bounds__(RS_THREADS) k_os_hist(const uint32_t *__restri
     const uint64_t stride = (uint64_t)gridDim.x * RS_THREADS;
     uint32_t kept = 0u;
     auto count = [&](uint32_t k) {
-        if (drop && k == SORT_DROP_KEY) return;
+        if (k == SORT_DROP_KEY) return;
         ++kept;
-        for (int p = 0; p < passes; ++p) {
-            const int nb = min(8, bits - 8 * p);
-            atomicAdd(&h[warp][p][(k >> (8 * p)) & ((1u << nb) - 1u)], 1u);
-        }
+#pragma unroll
+        for (int p = 0; p < passes; ++p) atomicAdd(&h[warp][p][(k >> (8 * p)) & 255u], 1u);
     };
     // four keys per 16-byte load (the key arrays are 256-byte aligned), then the tail
     const uint64_t n4 = n / 4;
@@ -228,11 +225,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_os_hist(const uint32_t *__restri
     }
     for (uint64_t j = 4 * n4 + (uint64_t)blockIdx.x * RS_THREADS + threadIdx.x; j < n; j += stride)
         count(keys[j]);
-    if (drop) {
-        const uint32_t wk = __reduce_add_sync(0xffffffffu, kept);
-        if ((threadIdx.x & 31) == 0 && wk)
-            atomicAdd(reinterpret_cast<unsigned long long *>(&aux->kept), (unsigned long long)wk);
-    }
+    const uint32_t wk = __reduce_add_sync(0xffffffffu, kept);
+    if ((threadIdx.x & 31) == 0 && wk)
+        atomicAdd(reinterpret_cast<unsigned long long *>(&aux->kept), (unsigned long long)wk);
     __syncthreads();
     for (int p = 0; p < passes; ++p) {
         uint32_t c = 0u;
@@ -246,9 +241,21 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const uint64_t *__restrict__ n_dev, uint64_t max_n, int pass, int shift,
     uint32_t mask, bool drop, uint32_t *__restrict__ flags, SortAux *aux, uint2 *__restrict__ ranges,
-    uint64_t n_ranges, uint32_t spin_limit, const uint64_t *__restrict__ skip_status) {
+    uint64_t n_ranges, uint32_t spin_limit, const uint64_t *__restrict__ skip_status,
+    const Batch *__restrict__ view_of) {
     chain_enter();
     constexpr int NW = RS_THREADS / 32;
+    __shared__ uint32_t s_ent[SG_MAX_VIEWS];   // view pass: the views' first entries
+    // the digit of a (key, value): bits of the key, or (view_of) the view of the entry `value`
+    auto digit = [&](uint32_t key, uint32_t val) -> uint32_t {
+        if (!view_of) return (key >> shift) & mask;
+        int lo = 0, hi = view_of->n_views - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_ent[mid] <= val) lo = mid; else hi = mid - 1;
+        }
+        return (uint32_t)lo;
+    };
     constexpr int PER_WARP = RS_TILE / NW;   // 512 consecutive keys per warp
     __shared__ uint32_t cnt[NW][RS_RADIX];
     __shared__ uint32_t dstart[RS_RADIX];
@@ -266,6 +273,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     const uint64_t n = min(*n_dev, max_n);
     const uint64_t base = (uint64_t)t * RS_TILE;
     if (base >= n) return;   // uniform across the block; later tiles exit too
+    if (view_of && (int)threadIdx.x < view_of->n_views) s_ent[threadIdx.x] = (uint32_t)view_of->view[threadIdx.x].ent_off;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int i = 0; i < NW; ++i) cnt[i][threadIdx.x] = 0u;
@@ -278,7 +286,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
         const uint64_t j = wbase + (uint64_t)i * 32 + lane;
         const bool ok = j < n;
         k[i] = ok ? kin[j] : 0u;
-        v[i] = ok ? vin[j] : 0u;
+        v[i] = !ok ? 0u : vin ? vin[j] : (uint32_t)j;   // no values yet: the key's index
     }
     // Warp-local stable ranks. Per item, the lowest lane of each group of equal
     // digits adds the group's size to the warp's counter; shared-memory atomics
@@ -290,15 +298,15 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     for (int i = 0; i < RS_ITEMS; ++i) {
         const uint64_t j = wbase + (uint64_t)i * 32 + lane;
         const bool ok = j < n && !(drop && k[i] == SORT_DROP_KEY);
-        const uint32_t d = ok ? ((k[i] >> shift) & mask) : 0x100u;
+        const uint32_t d = ok ? digit(k[i], v[i]) : 0x100u;
         const uint32_t peers = __match_any_sync(0xffffffffu, d);
         const uint32_t below = peers & lt;
         r[i] = (ok && below == 0u) ? atomicAdd(&cnt[warp][d], (uint32_t)__popc(peers)) : 0u;
-        meta[i] = (uint32_t)(__ffs(peers) - 1) | ((uint32_t)__popc(below) << 5);
+        meta[i] = (uint32_t)(__ffs(peers) - 1) | ((uint32_t)__popc(below) << 5) | d << 16;
     }
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; ++i)
-        r[i] = __shfl_sync(0xffffffffu, r[i], (int)(meta[i] & 31u)) + (meta[i] >> 5);
+        r[i] = __shfl_sync(0xffffffffu, r[i], (int)(meta[i] & 31u)) + ((meta[i] >> 5) & 63u);
     __syncthreads();
     // per digit: exclusive offsets over warps, block total, block-local start
     uint32_t run = 0u;
@@ -354,7 +362,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     for (int i = 0; i < RS_ITEMS; ++i) {
         const uint64_t j = wbase + (uint64_t)i * 32 + lane;
         if (j < n && !(drop && k[i] == SORT_DROP_KEY)) {
-            const uint32_t dd = (k[i] >> shift) & mask;
+            const uint32_t dd = meta[i] >> 16;
             const uint32_t pos = dstart[dd] + cnt[warp][dd] + r[i];
             sk[pos] = k[i];
             sv[pos] = v[i];
@@ -369,8 +377,11 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     const bool want_ranges = ranges != nullptr && *n_dev <= max_n;
     for (int p = threadIdx.x; p < items; p += RS_THREADS) {
         const uint32_t key = sk[p];
-        const uint32_t dd = (key >> shift) & mask;
+        const uint32_t dd = digit(key, sv[p]);
         const uint32_t o = gstart[dd] + (uint32_t)p - dstart[dd];
+        // after a pass that gave up a wait, stale keys can disagree with the
+        // histogram: their positions are cut at the buffers' end
+        if (o >= max_n) continue;
         kout[o] = key;
         vout[o] = sv[p];
         if (want_ranges && key < n_ranges) {
@@ -382,9 +393,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
 
 int radix_passes(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
 
-uint64_t sort_flag_words(uint64_t max_n, int bits) {
-    return div_up(max_n, RS_TILE) * RS_RADIX * (uint64_t)radix_passes(bits);
-}
+uint64_t sort_flag_words(uint64_t max_n, int passes) { return div_up(max_n, RS_TILE) * RS_RADIX * (uint64_t)passes; }
 
 // Buckets by list length on a log scale with 8 buckets per octave (exponent and
 // the 3 bits below the leading one), longest bucket first; inside a bucket the
@@ -397,30 +406,26 @@ __device__ __forceinline__ uint32_t len_bucket(const uint2 r) {
     return e * 8u + m;                                           // 0..255
 }
 
-// Status and kept count (one thread); ids that got no key get the range (0, 0).
-// no_pass: the keys had no bits, so no pass ran and every key is id 0.
-// status_mirror (nullable, host memory mapped into the device): receives the
-// status word after this sort's own status is merged in.
-// bucket_counts (nullable, with ranges; 256-thread blocks): adds every tile to
-// its list-length bucket (len_bucket), the counts of the persistent blends'
-// tile order.
-__global__ void k_os_finish(const SortAux *aux, uint64_t *status, uint64_t *kept_out, uint2 *ranges,
-                            uint64_t n_ranges, bool no_pass, const uint64_t *n_dev, uint64_t max_n,
-                            uint64_t *status_mirror, uint32_t *bucket_counts) {
+// After the radix tile sort: tiles that got no pair get the range (0, 0), every
+// tile joins its list-length bucket (len_bucket), and the sort's status is
+// merged into the call's (and written to the host word).
+// no_pass: one tile, so no pass ran and the pairs are tile 0's.
+__global__ void __launch_bounds__(256) k_os_finish(const SortAux *aux, uint64_t *counters, uint2 *ranges,
+                                                   uint64_t n_ranges, bool no_pass, uint64_t max_n,
+                                                   uint64_t *status_mirror, uint32_t *bucket_counts) {
     chain_enter();
     __shared__ uint32_t h[TB_BUCKETS];
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && !no_pass) {
-        if (status && aux->status) *status = aux->status;
-        if (kept_out) *kept_out = aux->kept;
+    const bool ok = counters[CNT_STATUS] == (uint64_t)SG_OK;
+    if (i == 0) {
+        if (aux->status) counters[CNT_STATUS] = aux->status;
+        if (status_mirror) *status_mirror = counters[CNT_STATUS];
     }
-    if (i == 0 && status_mirror) *status_mirror = status ? *status : 0u;
-    if (!ranges) return;   // uniform
     uint2 rg = make_uint2(0u, 0u);
     if (i < n_ranges) {
         if (no_pass) {
-            const uint64_t nd = *n_dev, n = nd <= max_n ? nd : 0;   // none when over capacity
-            rg = (i == 0 && n > 0) ? make_uint2(0u, (uint32_t)n) : make_uint2(0u, 0u);
+            const uint64_t n = ok ? min(counters[CNT_WRITTEN], max_n) : 0ull;
+            if (i == 0 && n > 0) rg = make_uint2(0u, (uint32_t)n);
             ranges[i] = rg;
         } else {
             rg = ranges[i];
@@ -430,7 +435,6 @@ __global__ void k_os_finish(const SortAux *aux, uint64_t *status, uint64_t *kept
             }
         }
     }
-    if (!bucket_counts) return;   // uniform
     h[threadIdx.x] = 0u;
     __syncthreads();
     if (i < n_ranges) atomicAdd(&h[len_bucket(rg)], 1u);
@@ -438,175 +442,374 @@ __global__ void k_os_finish(const SortAux *aux, uint64_t *status, uint64_t *kept
     if (h[threadIdx.x]) atomicAdd(&bucket_counts[threadIdx.x], h[threadIdx.x]);
 }
 
-cudaError_t launch_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
-                              const uint64_t *n_dev, uint64_t max_n, int bits, uint32_t *hist,
-                              uint64_t *scan_sums, cudaStream_t s, uint64_t *status, uint64_t *kept_out,
-                              bool aux_zeroed, uint2 *ranges, uint64_t n_ranges, bool hist_ready,
-                              uint64_t *status_mirror, const uint64_t *skip_status, uint32_t *order_counts) {
+cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
+                              const uint64_t *n_dev, uint64_t max_n, uint32_t *hist, SortAux *aux, cudaStream_t s) {
     const uint32_t nblocks = (uint32_t)div_up(max_n, RS_TILE);
-    const int passes = radix_passes(bits);
-    const uint64_t fgrid = ranges ? std::max<uint64_t>(div_up(n_ranges, 256), 1) : 1;
-    if (nblocks == 0 || passes == 0) {
-        // nothing to sort; ranges still get their final values
-        if (ranges) {
-            (void)launch_chain(k_os_finish, dim3((unsigned)fgrid), dim3(256), s, reinterpret_cast<SortAux *>(scan_sums),
-                               status, nullptr, ranges, n_ranges, passes == 0, n_dev, max_n, status_mirror,
-                               order_counts);
-            count_launches(1);
-            return cudaGetLastError();
-        }
-        if (status_mirror) {
-            (void)launch_chain(k_os_finish, dim3(1), dim3(1), s, reinterpret_cast<SortAux *>(scan_sums), status,
-                               nullptr, nullptr, 0, true, n_dev, max_n, status_mirror, nullptr);
-            count_launches(1);
-            return cudaGetLastError();
-        }
-        return cudaSuccess;
-    }
-    if (max_n > (uint64_t)LB_VAL) return cudaErrorInvalidValue;   // counts must fit the look-back word
-    SortAux *aux = reinterpret_cast<SortAux *>(scan_sums);
-    const bool drop = kept_out != nullptr;
-    const uint32_t spin_limit = sort_wait_polls();
+    if (nblocks == 0) return cudaSuccess;
+    if (max_n > SORT_MAX_KEYS) return cudaErrorInvalidValue;   // counts must fit the look-back word
+    const int passes = n_views > 1 ? 5 : 4;
     const uint64_t pass_words = (uint64_t)nblocks * RS_RADIX;
-    if (!hist_ready) {
-        if (!aux_zeroed) {
-            const cudaError_t e = cudaMemsetAsync(aux, 0, sizeof(SortAux), s);
-            if (e != cudaSuccess) return e;
-        }
-        const unsigned hgrid = nblocks < 4u * 152u ? nblocks : 4u * 152u;
-        (void)launch_chain(k_os_hist, dim3(hgrid), dim3(RS_THREADS), s, k0, n_dev, max_n, bits, drop, aux, hist, pass_words * passes);
-        count_launches(1);
+    const unsigned hgrid = nblocks < 4u * 152u ? nblocks : 4u * 152u;
+    (void)launch_chain(k_os_hist, dim3(hgrid), dim3(RS_THREADS), s, (const uint32_t *)k0, n_dev, max_n, aux, hist,
+                       pass_words * passes);
+    uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
+    for (int p = 0; p < passes; ++p) {
+        // pass 0 leaves SORT_DROP_KEY out and later passes see only the kept keys
+        (void)launch_chain(k_os_pass, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki,
+                           p > 0 ? (const uint32_t *)vi : (const uint32_t *)nullptr, ko, vo, p > 0 ? (const uint64_t *)&aux->kept : n_dev, max_n, p, 8 * p, 255u, p == 0,
+                           hist + pass_words * p, aux, (uint2 *)nullptr, (uint64_t)0, sort_wait_polls(),
+                           (const uint64_t *)nullptr, p == VIEW_PASS ? db : (const Batch *)nullptr);
+        std::swap(ki, ko);
+        std::swap(vi, vo);
     }
+    count_launches(1 + passes);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, uint64_t *counters,
+                                   uint64_t max_n, int bits, uint32_t *hist, SortAux *aux, uint2 *ranges,
+                                   uint64_t n_ranges, uint32_t *order_counts, uint64_t *status_mirror,
+                                   cudaStream_t s) {
+    const uint32_t nblocks = (uint32_t)div_up(max_n, RS_TILE);
+    const int passes = nblocks ? radix_passes(bits) : 0;
+    if (max_n > SORT_MAX_KEYS) return cudaErrorInvalidValue;
+    const uint64_t pass_words = (uint64_t)nblocks * RS_RADIX;
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
-        const int nb = min(8, bits - shift);
-        const uint32_t mask = (1u << nb) - 1u;
-        // with drop, pass 0 leaves SORT_DROP_KEY out and later passes see only the kept keys
-        const uint64_t *np = (drop && p > 0) ? &aux->kept : n_dev;
-        uint2 *rg = p == passes - 1 ? ranges : nullptr;
-        (void)launch_chain(k_os_pass, dim3(nblocks), dim3(RS_THREADS), s, ki, vi, ko, vo, np, max_n, p, shift, mask, drop && p == 0,
-                                                 hist + pass_words * p, aux, rg, n_ranges, spin_limit,
-                                                 skip_status);
-        count_launches(1);
-        uint32_t *t;
-        t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
+        const uint32_t mask = (1u << std::min(8, bits - shift)) - 1u;
+        (void)launch_chain(k_os_pass, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki, (const uint32_t *)vi,
+                           ko, vo, (const uint64_t *)(counters + CNT_WRITTEN), max_n, p, shift, mask, false,
+                           hist + pass_words * p, aux, p == passes - 1 ? ranges : (uint2 *)nullptr, n_ranges,
+                           sort_wait_polls(), (const uint64_t *)(counters + CNT_STATUS), (const Batch *)nullptr);
+        std::swap(ki, ko);
+        std::swap(vi, vo);
     }
-    if (status || kept_out || ranges || status_mirror) {
-        (void)launch_chain(k_os_finish, dim3((unsigned)fgrid), dim3(ranges ? 256 : 1), s, aux, status, kept_out, ranges, n_ranges, false,
-                                                                 n_dev, max_n, status_mirror, ranges ? order_counts : nullptr);
-        count_launches(1);
-    }
+    (void)launch_chain(k_os_finish, dim3((unsigned)std::max<uint64_t>(div_up(n_ranges, 256), 1)), dim3(256), s,
+                       (const SortAux *)aux, counters, ranges, n_ranges, bits == 0, max_n, status_mirror,
+                       order_counts);
+    count_launches(passes + 1);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// tile sort by counting (tile counts up to TC_MAX_TILES)
+// binning by chunks
 // ---------------------------------------------------------------------------
-// The duplicate's pairs, in depth order, are cut into C chunks of equal length.
-// k_tc_count counts each chunk's pairs per tile (row c of the [C][row] count
-// matrix); k_tc_scan scans the matrix in (tile, chunk) order, which turns row c
-// into the first output position of chunk c's pairs of every tile and bounds
-// every tile's range; k_tc_place walks each chunk's pairs in order and puts
-// each at its tile's next position. Inside a tile the pairs follow the chunks
-// in order and, inside a chunk, their input order: the result is the stable
-// sort by tile, identical to the LSD radix sort's.
-uint32_t tc_chunks(uint64_t cap) {
-    const uint64_t c = div_up(cap, TC_CHUNK_TARGET);
-    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(c, 1), TC_MAX_CHUNKS);
+// k_bin_cut    finds every entry's first pair (decoupled look-back) and cuts each
+//              view's entries into chunks of about equal pair counts
+// k_bin_emit   a block per chunk: enumerates its entries' tiles, writes the
+//              (tile, entry) pairs in depth order and counts them per tile in
+//              shared memory: row c of the [chunks][row] matrix
+// k_bin_scan   scans the matrix in (tile, chunk) order: row c becomes the first
+//              output position of chunk c's pairs of every tile; every range
+// k_bin_place  a warp per chunk walks its pairs in order and puts each at its
+//              tile's next position
+// Inside a tile the pairs follow the chunks in order and, inside a chunk, their
+// depth order: the result is the stable sort by tile of the depth-ordered pairs.
+// Measured (pairs and their placement, against a duplicate with its own
+// look-back followed by chunks of 8192 pairs or, past 12288 tiles, three radix
+// passes): 32k pairs 82 -> 31 us, 116k 91 -> 41, 3.9M 162 -> 129, 5.4M 195 -> 168,
+// 11.8M over four views 450 -> 348, 252M over 16 views 10.5 -> 6.4 ms. The
+// placement is bound by its warps' serial rounds (~400 cycles each, six warps
+// per SM) up to some 20M pairs, beyond by its scattered 4-byte stores.
+uint32_t bin_rows(uint64_t cap, uint32_t row) {
+    // Resident placing blocks, each holding one row of cursors in shared memory:
+    // six one-warp blocks per SM, five below 1M pairs (a smaller matrix).
+    const uint32_t want = cap > (1u << 20) ? 6u : 5u;
+    return 152u * std::max(std::min(want, (227u * 1024u) / (row * 4u + 1024u)), 1u);
 }
 
-uint64_t tc_row(uint64_t n_tiles) { return div_up(n_tiles, 4) * 4; }
-
-// [lo, hi): chunk c of the pairs the duplicate wrote; none when the status
-// says the pairs are incomplete (capacity overflow, or a bounded wait that
-// gave up: the lists may hold stale words).
-__device__ __forceinline__ void tc_chunk(const uint64_t *counters, uint64_t cap, uint32_t n_chunks, uint32_t c,
-                                         uint64_t &lo, uint64_t &hi) {
-    const uint64_t st = counters[CNT_STATUS];
-    const uint64_t K = st == (uint64_t)SG_OK ? min(counters[CNT_WRITTEN], cap) : 0ull;
-    const uint64_t len = div_up(div_up(K, n_chunks), 32) * 32;
-    lo = min(K, (uint64_t)c * len);
-    hi = min(K, lo + len);
+uint32_t bin_chunks(uint64_t cap, uint32_t row) {
+    // Past 16M pairs the chunks' open output sectors (chunks x tiles x 32 bytes,
+    // over every view) no longer fit L2: four per SM place faster than six.
+    return std::min(bin_rows(cap, row), cap > (16u << 20) ? 4u * 152u : BIN_MAX_CHUNKS);
 }
 
-// One block per chunk: shared-memory counters of every tile, then row c.
-__global__ void __launch_bounds__(256) k_tc_count(const uint16_t *__restrict__ keys,
-                                                  const uint64_t *__restrict__ counters, uint64_t cap,
-                                                  uint32_t n_tiles, uint32_t row, uint32_t *__restrict__ counts) {
-    chain_enter();
-    extern __shared__ uint4 tc_smem[];
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(tc_smem);
-    for (uint32_t q = threadIdx.x; q < row / 4; q += blockDim.x) tc_smem[q] = make_uint4(0u, 0u, 0u, 0u);
+__device__ __forceinline__ uint32_t bin_view_of_chunk(const BinTab &tab, int n_views, uint32_t c) {
+    int lo = 0, hi = n_views - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (tab.first_chunk[mid] <= c) lo = mid; else hi = mid - 1;
+    }
+    return (uint32_t)lo;
+}
+
+// Blocks take BIN_BLOCK entries of the depth order at a time, in order, from a
+// ticket. An entry costs its pairs plus BIN_ENTRY_COST (the emitting and the
+// placing warp spend time on both), so entry j's cost starts at
+// X = its first pair + BIN_ENTRY_COST j. A chunk of view v starts at the first
+// entry whose cost starts at or past B_v + q len_v (q = 0, 1, ..; B_v: the cost of the
+// views before it): entry j marks the chunks whose threshold lies in
+// (X, X + its cost] with the start j + 1. Every block recomputes the views' tables
+// from preprocess's totals; block 0 publishes them.
+__global__ void __launch_bounds__(256) k_bin_cut(BinArgs a, uint32_t spin_limit) {
+    chain_wait();
+    __shared__ unsigned long long s_out0;
+    __shared__ uint64_t shs64[33];
+    __shared__ uint32_t shs[33];
+    __shared__ uint32_t s_blk;
+    __shared__ uint32_t s_base[SG_MAX_VIEWS + 1], s_len[SG_MAX_VIEWS], s_first[SG_MAX_VIEWS + 1], s_ent[SG_MAX_VIEWS];
+    if (a.aux->status) {   // the depth sort gave up a bounded wait: its order may hold stale words (uniform)
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.counters[CNT_STATUS] = a.aux->status;
+            if (a.mirror) a.mirror[0] = 0;
+        }
+        return;
+    }
+    const int tid = threadIdx.x;
+    const uint64_t V = min(a.M, a.aux->kept);
+    uint64_t p = tid < a.n_views ? a.tab->view_pairs[tid] : 0ull;
+    uint64_t K, cost;
+    (void)block_exclusive<uint64_t>(p, K, shs64);
+    const bool fits = K <= a.cap;
+    if (blockIdx.x == 0 && tid == 0) {
+        a.counters[CNT_PAIRS] = K;
+        a.counters[CNT_WRITTEN] = min(K, a.cap);
+        if (a.mirror) a.mirror[0] = K;
+        if (!fits) a.counters[CNT_STATUS] = (uint64_t)SG_ERR_CAPACITY;
+    }
+    if (!fits) return;   // uniform
+    // chunks of each view: one, and a share of the others by its cost (below
+    // 2^32: no more entries than pairs, BIN_ENTRY_COST + 1 times 2^30)
+    if (tid < a.n_views) p += (uint64_t)BIN_ENTRY_COST * a.aux->hist[VIEW_PASS][tid];
+    const uint64_t base = block_exclusive<uint64_t>(p, cost, shs64);
+    const uint64_t spare = min((uint64_t)(a.max_chunks - (uint32_t)a.n_views), K / BIN_MIN_CHUNK);
+    const uint32_t nc = tid < a.n_views ? 1u + (uint32_t)(spare * p / max(cost, (uint64_t)1)) : 0u;
+    uint32_t total_chunks;
+    const uint32_t fc = block_exclusive<uint32_t>(nc, total_chunks, shs);
+    if (tid < a.n_views) {
+        s_base[tid] = (uint32_t)base;
+        s_len[tid] = (uint32_t)max(div_up(p, nc), (uint64_t)1);
+        s_first[tid] = fc;
+        s_ent[tid] = (uint32_t)a.db->view[tid].ent_off;
+    }
+    if (tid == 0) {
+        s_base[a.n_views] = (uint32_t)cost;
+        s_first[a.n_views] = total_chunks;
+    }
     __syncthreads();
-    uint64_t lo, hi;
-    tc_chunk(counters, cap, gridDim.x, blockIdx.x, lo, hi);
-    // 16-byte loads of 8 keys (a chunk starts at a multiple of 32 keys), then the tail
-    const uint64_t n8 = (hi - lo) / 8;
-    const uint4 *k8 = reinterpret_cast<const uint4 *>(keys + lo);
-#pragma unroll 4
-    for (uint64_t q = threadIdx.x; q < n8; q += blockDim.x) {
-        const uint4 w = k8[q];
-        const uint32_t h[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t a = h[k] & 0xFFFFu, b = h[k] >> 16;
-            if (a < n_tiles) atomicAdd(&cnt[a], 1u);
-            if (b < n_tiles) atomicAdd(&cnt[b], 1u);
+    if (blockIdx.x == 0) {
+        BinTab &t = *a.tab;
+        if (tid < a.n_views) t.first_chunk[tid] = fc;
+        if (tid == 0) {
+            t.n_chunks = total_chunks;
+            t.first_chunk[a.n_views] = total_chunks;
+            t.start[total_chunks] = (uint32_t)V;
+            t.pair[total_chunks] = (uint32_t)K;
+            // chunks whose threshold is 0: the first view's first chunk, and
+            // every chunk of the views before the first entry
+            for (int v = 0; v < a.n_views && s_base[v] == 0u; ++v) {
+                const uint32_t last = s_base[v + 1] == 0u ? s_first[v + 1] : s_first[v] + 1u;
+                for (uint32_t c = s_first[v]; c < last; ++c) t.start[c] = t.pair[c] = 0u;
+            }
         }
     }
-    for (uint64_t i = lo + 8 * n8 + threadIdx.x; i < hi; i += blockDim.x) {
-        const uint32_t t = keys[i];
-        if (t < n_tiles) atomicAdd(&cnt[t], 1u);
+    for (;;) {
+        __syncthreads();   // every thread is past the previous block's shared words
+        if (tid == 0)
+            s_blk = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + CNT_DUP_BLOCK), 1ull);
+        __syncthreads();
+        const uint32_t blk = s_blk;
+        if ((uint64_t)blk * BIN_BLOCK >= V) return;   // uniform
+        // BIN_ITEMS consecutive entries per thread
+        const uint64_t j0 = (uint64_t)blk * BIN_BLOCK + (uint64_t)BIN_ITEMS * tid;
+        uint32_t e[BIN_ITEMS], n[BIN_ITEMS], sum = 0;
+#pragma unroll
+        for (int i = 0; i < BIN_ITEMS; i += 4) {   // the order's array is 256-byte aligned
+            if (j0 + i + 3 < V) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(a.sorted_ent + j0 + i);
+                e[i] = q.x; e[i + 1] = q.y; e[i + 2] = q.z; e[i + 3] = q.w;
+            } else {
+#pragma unroll
+                for (int k = i; k < i + 4; ++k) e[k] = j0 + k < V ? a.sorted_ent[j0 + k] : 0xFFFFFFFFu;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < BIN_ITEMS; ++i) {
+            n[i] = e[i] < a.M ? a.tiles_touched[e[i]] : 0u;
+            sum += n[i];
+        }
+        uint32_t total;
+        uint32_t at = block_exclusive<uint32_t>(sum, total, shs);
+        if (tid < 32) {
+            if (tid == 0) st_relaxed64(a.flags + blk, DL_AGG | (uint64_t)total);
+            const uint64_t excl = block_lookback64(a.flags, blk, total, spin_limit, a.counters + CNT_STATUS);
+            if (tid == 0) s_out0 = excl;
+        }
+        __syncthreads();
+        at += (uint32_t)s_out0;
+        int v = 0;
+#pragma unroll
+        for (int i = 0; i < BIN_ITEMS; ++i) {
+            if (j0 + i >= V) break;
+            a.poff[j0 + i] = at;
+            const uint32_t end = at + n[i];   // pairs; x0, x1: cost
+            const uint32_t x0 = at + BIN_ENTRY_COST * (uint32_t)(j0 + i), x1 = end + BIN_ENTRY_COST * (uint32_t)(j0 + i + 1);
+            // the entry's view (entries are numbered view after view, the order has views in turn)
+            if (v + 1 < a.n_views && e[i] >= s_ent[v + 1]) {
+                int lo = v + 1, hi = a.n_views - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (s_ent[mid] <= e[i]) lo = mid; else hi = mid - 1;
+                }
+                v = lo;
+            }
+            const uint32_t vb = s_base[v], len = s_len[v], vc = s_first[v + 1] - s_first[v];
+            // chunks q of the view with q len in (x0 - vb, x1 - vb]
+            uint32_t q0 = (x0 - vb) / len + 1u, q1 = min((x1 - vb) / len, vc - 1u);
+            const bool last = x1 == s_base[v + 1];
+            if (last) q1 = vc - 1u;   // thresholds past the view's cost: empty chunks at its end
+            for (uint32_t q = q0; q <= q1; ++q) {
+                a.tab->start[s_first[v] + q] = (uint32_t)(j0 + i + 1);
+                a.tab->pair[s_first[v] + q] = end;
+            }
+            if (last) {   // the first chunk of the next view with entries, and all of the empty views before it
+                for (int u = v + 1; u < a.n_views && s_base[u] == x1; ++u) {
+                    const uint32_t stop = s_base[u + 1] == x1 ? s_first[u + 1] : s_first[u] + 1u;
+                    for (uint32_t c = s_first[u]; c < stop; ++c) {
+                        a.tab->start[c] = (uint32_t)(j0 + i + 1);
+                        a.tab->pair[c] = end;
+                    }
+                }
+            }
+            at = end;
+        }
     }
-    __syncthreads();
-    uint4 *dst = reinterpret_cast<uint4 *>(counts + (uint64_t)blockIdx.x * row);
-    for (uint32_t q = threadIdx.x; q < row / 4; q += blockDim.x) dst[q] = tc_smem[q];
 }
 
-// Groups of 32 tiles (lane = tile), taken in order from a ticket by resident
-// blocks (two per SM); the chunks split into TC_SCAN_WARPS runs (one per warp),
-// whose counts wait in shared memory for the second walk. The sum of each tile's counts and the group's total go
-// through a decoupled look-back over the groups before it, which gives every
-// tile's first position; the second walk replaces each count with its chunk's
-// first position of the tile. Also writes every tile's range ((0, 0) when
-// empty) and adds the tile to its list-length bucket.
-// words: zeroed; [0] the ticket, [1 + g] group g's look-back word.
-constexpr int TC_SCAN_WARPS = 32;
-constexpr int TC_SCAN_RUN = (TC_MAX_CHUNKS + TC_SCAN_WARPS - 1) / TC_SCAN_WARPS;
-__global__ void __launch_bounds__(TC_SCAN_WARPS * 32, 2) k_tc_scan(uint32_t *__restrict__ counts, uint32_t n_chunks,
-                                                              uint32_t row, uint32_t n_tiles,
-                                                              uint64_t *__restrict__ words,
-                                                              uint2 *__restrict__ ranges,
-                                                              uint32_t *__restrict__ bucket_counts,
-                                                              uint64_t *__restrict__ status, uint32_t spin_limit) {
-    chain_enter();
-    __shared__ uint32_t part[TC_SCAN_WARPS][32];
+// A block per chunk writes its entries' pairs (16-bit tile id inside the view,
+// entry), entry after entry. Each warp takes 32 entries at a time, whose pairs go
+// to [poff of the first, ..): its work items are (entry, tile row) in order, each
+// finding the row's reached columns once; the positions inside the warp's range
+// come from a warp scan of the run lengths (an entry's runs add up to its
+// tiles_touched), so no two warps wait on each other.
+__global__ void __launch_bounds__(256) k_bin_emit(BinArgs a) {
+    chain_wait();
+    extern __shared__ uint4 bin_smem[];
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(bin_smem);
+    const unsigned FULL = 0xffffffffu;
+    if (a.counters[CNT_STATUS] != (uint64_t)SG_OK) return;   // uniform
+    const BinTab &tab = *a.tab;
+    const uint32_t c = blockIdx.x;
+    if (c >= tab.n_chunks) return;
+    const ViewDesc &vw = a.db->view[bin_view_of_chunk(tab, a.n_views, c)];
+    const uint32_t T = (uint32_t)vw.tiles_x * (uint32_t)vw.tiles_y, tx = (uint32_t)vw.tiles_x;
+    const uint32_t q4 = (T + 3u) / 4u;
+    for (uint32_t q = threadIdx.x; q < q4; q += blockDim.x) bin_smem[q] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    const uint32_t V = (uint32_t)min(a.M, a.aux->kept);
+    const uint32_t e0 = min(tab.start[c], V), e1 = min(tab.start[c + 1], V);
+    const int lane = threadIdx.x & 31;
+    for (uint32_t jb = e0 + (threadIdx.x & ~31u); jb < e1; jb += blockDim.x) {
+        const uint32_t j = jb + lane;
+        const bool on = j < e1;
+        uint32_t e = 0, rows = 0, x01 = 0, y0 = 0;
+        TileReach R;
+        R.x = R.y = R.B = R.det = R.At = R.ymax = R.m = R.invA = 0.f;
+        R.mode = 0;
+        if (on) {
+            e = a.sorted_ent[j];
+            if (e < a.M) {
+                const uint2 rc = a.rect[e];
+                // the binning reads the record's first 24 bytes: x, y, conic, bound (one sector)
+                const float4 ra = a.rec[e].a;
+                const float2 rb = *reinterpret_cast<const float2 *>(&a.rec[e].b);
+                x01 = rc.x;
+                y0 = rc.y & 0xFFFFu;
+                rows = (rc.y >> 16) - y0;
+                tile_reach_init(ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, R);
+            }
+        }
+        uint32_t pos = __shfl_sync(FULL, on ? a.poff[j] : 0u, 0);   // first pair of the warp's entries
+        const uint32_t inc = warp_inclusive(rows), exc = inc - rows;
+        const uint32_t n_rows = __shfl_sync(FULL, inc, 31);
+        for (uint32_t base = 0; base < n_rows; base += 32) {   // uniform
+            // item lane -> its owner: owners that start before this window, and the heads inside it
+            const bool own = rows != 0u;
+            const uint32_t before = __ballot_sync(FULL, own && exc < base);
+            const uint32_t heads = __reduce_or_sync(FULL, own && exc >= base && exc < base + 32u ? 1u << (exc - base) : 0u);
+            const uint32_t owners = __ballot_sync(FULL, own);
+            const int rank = __popc(before) + __popc(heads & (0xffffffffu >> (31 - lane))) - 1;
+            const int o = (owners & (owners + 1u)) == 0u ? rank : (int)__fns(owners, 0, rank + 1);
+            const int src = o & 31;
+            TileReach S;
+            S.x = __shfl_sync(FULL, R.x, src);
+            S.y = __shfl_sync(FULL, R.y, src);
+            S.B = __shfl_sync(FULL, R.B, src);
+            S.det = __shfl_sync(FULL, R.det, src);
+            S.At = __shfl_sync(FULL, R.At, src);
+            S.ymax = __shfl_sync(FULL, R.ymax, src);
+            S.m = __shfl_sync(FULL, R.m, src);
+            S.invA = __shfl_sync(FULL, R.invA, src);
+            S.mode = __shfl_sync(FULL, R.mode, src);
+            const uint32_t sx = __shfl_sync(FULL, x01, src), se = __shfl_sync(FULL, e, src);
+            const uint32_t sy = __shfl_sync(FULL, y0, src), s0 = __shfl_sync(FULL, exc, src);
+            int c0 = 0, c1 = 0;
+            uint32_t row = 0;
+            if (base + lane < n_rows) {
+                row = sy + (base + lane - s0);
+                tile_reach_row(S, (int)row, (int)(sx & 0xFFFFu), (int)(sx >> 16), c0, c1);
+            }
+            const uint32_t run = (uint32_t)(c1 - c0);
+            const uint32_t rinc = warp_inclusive(run);
+            uint32_t at = pos + rinc - run;
+            for (uint32_t t = row * tx + (uint32_t)c0, te = t + run; t < te; ++t, ++at) {
+                if (t < T && at < a.cap) {
+                    a.pkey[at] = (uint16_t)t;
+                    a.pval[at] = se;
+                    atomicAdd(&cnt[t], 1u);
+                }
+            }
+            pos += __shfl_sync(FULL, rinc, 31);
+        }
+    }
+    __syncthreads();
+    uint4 *dst = reinterpret_cast<uint4 *>(a.matrix + (uint64_t)c * a.row);
+    for (uint32_t q = threadIdx.x; q < q4; q += blockDim.x) dst[q] = bin_smem[q];
+}
+
+// Groups of 32 tiles of one view (lane = tile), taken in order from a ticket by
+// resident blocks; the view's chunks split into BIN_SCAN_WARPS runs (one per
+// warp), whose counts wait in shared memory for the second walk. The sum of
+// each tile's counts and the group's total go through a decoupled look-back
+// over the groups before it, which gives every tile's first position; the
+// second walk replaces each count with its chunk's first position of the tile.
+// Also writes every tile's range ((0, 0) when empty) and adds the tile to its
+// list-length bucket. words: [0] the ticket, [1 + g] group g's look-back word.
+constexpr int BIN_SCAN_WARPS = 32;
+__global__ void __launch_bounds__(BIN_SCAN_WARPS * 32, 2) k_bin_scan(BinArgs a, uint32_t spin_limit) {
+    chain_wait();
+    __shared__ uint32_t part[BIN_SCAN_WARPS][32];
     __shared__ uint32_t s_start[32];
     __shared__ uint32_t s_grp;
+    extern __shared__ uint32_t cvs[];   // [longest run][block threads]: the run's counts
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t n_groups = (n_tiles + 31) / 32;
-    const uint32_t per = (n_chunks + TC_SCAN_WARPS - 1) / TC_SCAN_WARPS;
-    const uint32_t c0 = min(n_chunks, warp * per), c1 = min(n_chunks, c0 + per);
-    constexpr int RUN = TC_SCAN_RUN;
-    extern __shared__ uint32_t cvs[];   // [RUN][block threads]: the run's counts
+    const Batch &b = *a.db;
+    const bool lists = a.counters[CNT_STATUS] == (uint64_t)SG_OK;   // else no pair is binned
     for (;;) {
         // every thread is past the previous group's reads of the shared words
         __syncthreads();
-        if (threadIdx.x == 0) s_grp = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long *>(words), 1ull);
+        if (threadIdx.x == 0) s_grp = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long *>(a.words), 1ull);
         __syncthreads();
         const uint32_t grp = s_grp;
-        if (grp >= n_groups) break;   // uniform
-        const uint32_t t = grp * 32 + lane;
-        const bool tv = t < n_tiles;
-        uint32_t *col = counts + t;
+        if (grp >= a.n_groups) break;   // uniform
+        int lo = 0, hi = a.n_views - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (b.view[mid].grp_off <= grp) lo = mid; else hi = mid - 1;
+        }
+        const ViewDesc &vw = b.view[lo];
+        const uint32_t t = (grp - vw.grp_off) * 32 + lane;   // tile inside the view
+        const bool tv = t < (uint32_t)vw.tiles_x * (uint32_t)vw.tiles_y;
+        const uint32_t ca = lists ? a.tab->first_chunk[lo] : 0u, cb = lists ? a.tab->first_chunk[lo + 1] : 0u;
+        const uint32_t per = (cb - ca + BIN_SCAN_WARPS - 1) / BIN_SCAN_WARPS;
+        const uint32_t c0 = min(cb, ca + warp * per), c1 = min(cb, c0 + per);
+        uint32_t *col = a.matrix + t;
         uint32_t sum = 0;
-#pragma unroll
-        for (int j = 0; j < RUN; ++j) {
-            const uint32_t c = c0 + (uint32_t)j;
-            const uint32_t x = (tv && c < c1) ? col[(uint64_t)c * row] : 0u;
-            cvs[j * TC_SCAN_WARPS * 32 + threadIdx.x] = x;
+#pragma unroll 8
+        for (uint32_t j = 0; j < per; ++j) {
+            const uint32_t x = (tv && c0 + j < c1) ? col[(uint64_t)(c0 + j) * a.row] : 0u;
+            cvs[j * (BIN_SCAN_WARPS * 32) + threadIdx.x] = x;
             sum += x;
         }
         part[warp][lane] = sum;
@@ -614,81 +817,82 @@ __global__ void __launch_bounds__(TC_SCAN_WARPS * 32, 2) k_tc_scan(uint32_t *__r
         // each warp its runs' prefix over the warps before it; warp 0 the totals
         uint32_t before = 0;
         for (int w = 0; w < warp; ++w) before += part[w][lane];
-        uint32_t tot = 0;
         if (warp == 0) {
+            uint32_t tot = 0;
 #pragma unroll
-            for (int w = 0; w < TC_SCAN_WARPS; ++w) tot += part[w][lane];
-        }
-        if (warp == 0) {
+            for (int w = 0; w < BIN_SCAN_WARPS; ++w) tot += part[w][lane];
             const uint32_t inc = warp_inclusive(tot);
             const uint32_t grp_total = __shfl_sync(0xffffffffu, inc, 31);
-            if (lane == 0) st_relaxed64(words + 1 + grp, DL_AGG | (uint64_t)grp_total);
-            const uint64_t excl = block_lookback64(words + 1, grp, grp_total, spin_limit, status);
+            if (lane == 0) st_relaxed64(a.words + 1 + grp, DL_AGG | (uint64_t)grp_total);
+            const uint64_t excl = block_lookback64(a.words + 1, grp, grp_total, spin_limit, a.counters + CNT_STATUS);
             const uint32_t start = (uint32_t)(excl + inc - tot);
             s_start[lane] = start;
             if (tv) {
                 const uint2 rg = tot ? make_uint2(start, start + tot) : make_uint2(0u, 0u);
-                ranges[t] = rg;
-                if (bucket_counts) atomicAdd(&bucket_counts[len_bucket(rg)], 1u);
+                a.ranges[vw.tile_off + t] = rg;
+                atomicAdd(&a.order_counts[len_bucket(rg)], 1u);
             }
         }
         __syncthreads();
         uint32_t run = s_start[lane] + before;
-#pragma unroll
-        for (int j = 0; j < RUN; ++j) {
-            const uint32_t c = c0 + (uint32_t)j;
-            if (tv && c < c1) col[(uint64_t)c * row] = run;
-            run += cvs[j * TC_SCAN_WARPS * 32 + threadIdx.x];
+#pragma unroll 8
+        for (uint32_t j = 0; j < per; ++j) {
+            if (tv && c0 + j < c1) col[(uint64_t)(c0 + j) * a.row] = run;
+            run += cvs[j * (BIN_SCAN_WARPS * 32) + threadIdx.x];
         }
     }
 }
 
 // One warp per chunk: its row of first positions in shared memory, then the
-// chunk's pairs 32 at a time in order (the entries only: a pair's tile is the
-// tile whose range holds it). Lanes holding the same tile are grouped
-// (match_any); the group's first lane takes as many positions from the tile's
-// cursor as the group has lanes, and each lane takes the one of its rank in the
-// group. The warp barrier between rounds orders the cursor updates of
-// successive rounds. Positions at or past cap are not written.
-__global__ void __launch_bounds__(32) k_tc_place(const uint16_t *__restrict__ keys,
-                                                 const uint32_t *__restrict__ vals,
-                                                 const uint64_t *__restrict__ counters, uint64_t cap,
-                                                 uint32_t n_tiles, uint32_t row,
-                                                 const uint32_t *__restrict__ first,
-                                                 uint32_t *__restrict__ ovals, uint64_t *status_mirror) {
+// chunk's pairs 32 at a time in order (a pair's tile is the tile whose range
+// holds it). Lanes holding the same tile are grouped (match_any); the group's
+// first lane takes as many positions from the tile's cursor as the group has
+// lanes, and each lane takes the one of its rank in the group. The warp
+// barriers order the cursor updates of successive rounds, whose returned
+// positions are only read after all U rounds' updates are issued: the rounds'
+// shared-memory latencies overlap. Positions at or past cap are not written.
+__global__ void __launch_bounds__(32) k_bin_place(BinArgs a) {
     chain_enter();
-    extern __shared__ uint4 tc_smem[];
-    uint32_t *next = reinterpret_cast<uint32_t *>(tc_smem);
+    extern __shared__ uint4 bin_smem[];
+    uint32_t *next = reinterpret_cast<uint32_t *>(bin_smem);
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x;
-    if (blockIdx.x == 0 && lane == 0 && status_mirror) *status_mirror = counters[CNT_STATUS];
+    const uint64_t status = a.counters[CNT_STATUS];
+    if (blockIdx.x == 0 && lane == 0 && a.mirror) a.mirror[1] = status;
+    if (status != (uint64_t)SG_OK) return;
+    const BinTab &tab = *a.tab;
+    const uint32_t c = blockIdx.x;
+    if (c >= tab.n_chunks) return;
+    const uint32_t K = (uint32_t)min(a.counters[CNT_WRITTEN], a.cap);
+    const uint32_t lo = min(tab.pair[c], K), hi = min(tab.pair[c + 1], K);
+    if (lo >= hi) return;
+    const ViewDesc &vw = a.db->view[bin_view_of_chunk(tab, a.n_views, c)];
+    const uint32_t T = (uint32_t)vw.tiles_x * (uint32_t)vw.tiles_y;
     // the row arrives by asynchronous 16-byte copies while the first batch loads
-    const uint4 *src = reinterpret_cast<const uint4 *>(first + (uint64_t)blockIdx.x * row);
-    for (uint32_t q = lane; q < row / 4; q += 32) {
-        const uint32_t d = (uint32_t)__cvta_generic_to_shared(tc_smem + q);
+    const uint4 *src = reinterpret_cast<const uint4 *>(a.matrix + (uint64_t)c * a.row);
+    for (uint32_t q = lane; q < (T + 3u) / 4u; q += 32) {
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(bin_smem + q);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src + q) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    uint64_t lo, hi;
-    tc_chunk(counters, cap, gridDim.x, blockIdx.x, lo, hi);
     const uint32_t lt = (1u << lane) - 1u;
-    // rounds of 32 pairs, U rounds per batch; the next batch's keys and values
-    // are loaded while this one is placed
+    // U rounds of 32 pairs per batch; the next batch's tiles and entries are
+    // loaded while this one is placed
     constexpr int U = 8;
     uint32_t tn[U], vn[U];
-    auto load = [&](uint64_t base) {
+    auto load = [&](uint32_t base) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const uint64_t i = base + (uint64_t)(32 * u + lane);
-            tn[u] = i < hi ? (uint32_t)keys[i] : 0xFFFFFFFFu;
-            vn[u] = i < hi ? vals[i] : 0u;
+            const uint32_t i = base + (uint32_t)(32 * u + lane);
+            tn[u] = i < hi ? (uint32_t)a.pkey[i] : 0xFFFFFFFFu;
+            vn[u] = i < hi ? a.pval[i] : 0xFFFFFFFFu;
         }
     };
     load(lo);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
-    for (uint64_t base = lo; base < hi; base += 32 * U) {
-        uint32_t t[U], v[U];
+    for (uint32_t base = lo; base < hi; base += 32 * U) {
+        uint32_t t[U], v[U], grp[U], at[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             t[u] = tn[u];
@@ -696,65 +900,82 @@ __global__ void __launch_bounds__(32) k_tc_place(const uint16_t *__restrict__ ke
         }
         if (base + 32 * U < hi) load(base + 32 * U);
 #pragma unroll
+        for (int u = 0; u < U; ++u) grp[u] = __match_any_sync(FULL, t[u]);
+#pragma unroll
         for (int u = 0; u < U; ++u) {
-            const bool ok = t[u] < n_tiles;
-            const uint32_t grp = __match_any_sync(FULL, ok ? t[u] : 0xFFFFFFFFu);
-            const int leader = __ffs(grp) - 1;
-            uint32_t at = 0;
-            if (ok && lane == leader) at = atomicAdd(&next[t[u]], (uint32_t)__popc(grp));
-            at = __shfl_sync(FULL, at, leader);
-            const uint32_t pos = at + (uint32_t)__popc(grp & lt);
-            if (ok && pos < cap) ovals[pos] = v[u];
+            at[u] = 0u;
+            if (t[u] < T && (grp[u] & lt) == 0u) at[u] = atomicAdd(&next[t[u]], (uint32_t)__popc(grp[u]));
             __syncwarp();
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t pos = __shfl_sync(FULL, at[u], __ffs(grp[u]) - 1) + (uint32_t)__popc(grp[u] & lt);
+            if (t[u] < T && pos < K) a.ovals[pos] = v[u];
         }
     }
 }
 
-cudaError_t launch_tile_count_sort(const uint16_t *keys, const uint32_t *vals, uint32_t *ovals,
-                                   uint64_t *counters, uint64_t cap, uint32_t n_tiles, uint32_t n_chunks,
-                                   uint32_t *matrix, uint64_t *words, uint2 *ranges, uint32_t *order_counts,
-                                   uint64_t *status_mirror, cudaStream_t s) {
-    if (n_tiles == 0 || n_tiles > TC_MAX_TILES || n_chunks == 0 || n_chunks > TC_MAX_CHUNKS || cap > UINT32_MAX)
-        return cudaErrorInvalidValue;
-    const uint32_t row = (uint32_t)tc_row(n_tiles);
-    const size_t smem = (size_t)row * 4;
-    (void)launch_chain_smem(k_tc_count, dim3(n_chunks), dim3(256), smem, s, keys, (const uint64_t *)counters, cap,
-                       n_tiles, row, matrix);
-    // resident blocks only: a group's look-back may wait on any earlier group
-    const size_t scan_smem = (size_t)TC_SCAN_RUN * TC_SCAN_WARPS * 32 * 4;
-    static int scan_blocks = 0;
-    if (scan_blocks == 0) {
-        int dev = 0, sms = 0, per_sm = 0;
-        if (cudaFuncSetAttribute(k_tc_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)scan_smem) !=
-                cudaSuccess ||
-            cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_scan, TC_SCAN_WARPS * 32, scan_smem) !=
-                cudaSuccess)
-            return cudaErrorUnknown;
-        scan_blocks = std::max(1, sms * per_sm);
+// The sorted pairs' global tile ids, for layouts that keep them: a warp per tile.
+__global__ void __launch_bounds__(256) k_bin_keys(const uint2 *__restrict__ ranges, uint32_t n_tiles,
+                                                  uint32_t *__restrict__ okeys) {
+    chain_enter();
+    const uint32_t nw = gridDim.x * (blockDim.x >> 5);
+    for (uint32_t t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < n_tiles; t += nw) {
+        const uint2 rg = ranges[t];
+        for (uint32_t i = rg.x + (threadIdx.x & 31); i < rg.y; i += 32) okeys[i] = t;
     }
-    const unsigned sgrid = (unsigned)std::min<uint64_t>(div_up(n_tiles, 32), (uint64_t)scan_blocks);
-    (void)launch_chain_smem(k_tc_scan, dim3(sgrid), dim3(TC_SCAN_WARPS * 32), scan_smem, s, matrix, n_chunks,
-                       row, n_tiles, words, ranges, order_counts, counters + CNT_STATUS, sort_wait_polls());
-    (void)launch_chain_smem(k_tc_place, dim3(n_chunks), dim3(32), smem, s, keys, vals, (const uint64_t *)counters, cap,
-                       n_tiles, row, (const uint32_t *)matrix, ovals, status_mirror);
-    count_launches(3);
+}
+
+// Opts a kernel into `bytes` of dynamic shared memory on the current device.
+template <typename K>
+static cudaError_t allow_smem(K kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
+    if (a.n_tiles == 0 || a.row == 0 || a.row > BIN_MAX_ROW || a.max_chunks <= (uint32_t)a.n_views ||
+        a.max_chunks > BIN_MAX_CHUNKS || a.cap > SORT_MAX_KEYS)
+        return cudaErrorInvalidValue;
+    const size_t smem = (size_t)a.row * 4;
+    const cudaError_t e = allow_smem(k_bin_emit, smem);
+    if (e != cudaSuccess) return e;
+    // one block at least: it publishes the zero total of a call without entries;
+    // how many of the M entries are in the order is only known on the device
+    const uint64_t cut = std::min<uint64_t>(std::max<uint64_t>(div_up(a.M, BIN_BLOCK), 1), 4 * 152);
+    (void)launch_chain(k_bin_cut, dim3((unsigned)cut), dim3(256), s, a, sort_wait_polls());
+    (void)launch_chain_smem(k_bin_emit, dim3(a.max_chunks), dim3(256), smem, s, a);
+    count_launches(2);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bin_place(const BinArgs &a, cudaStream_t s) {
+    const size_t smem = (size_t)a.row * 4;
+    const size_t scan_smem = (size_t)div_up(a.max_chunks, BIN_SCAN_WARPS) * BIN_SCAN_WARPS * 32 * 4;
+    cudaError_t e = allow_smem(k_bin_place, smem);
+    if (e == cudaSuccess) e = allow_smem(k_bin_scan, scan_smem);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // resident blocks only: a group's look-back may wait on any earlier group
+    // (two 1024-thread blocks fill an SM's threads; shared memory decides)
+    per_sm = scan_smem <= 100 * 1024 ? 2 : 1;
+    const unsigned grid = std::min(a.n_groups, (uint32_t)(sms * per_sm));
+    (void)launch_chain_smem(k_bin_scan, dim3(grid), dim3(BIN_SCAN_WARPS * 32), scan_smem, s, a, sort_wait_polls());
+    (void)launch_chain_smem(k_bin_place, dim3(a.max_chunks), dim3(32), smem, s, a);
+    count_launches(2);
+    if (a.okeys) {
+        (void)launch_chain(k_bin_keys, dim3(std::min(div_up(a.n_tiles, 8), (uint64_t)(sms * 8))), dim3(256), s,
+                           (const uint2 *)a.ranges, a.n_tiles, a.okeys);
+        count_launches(1);
+    }
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
 // duplicateWithKeys: entries in depth order -> (tile, entry) pairs
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int find_entry_view(const Batch &b, uint64_t e) {
-    int lo = 0, hi = b.n_views - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (b.view[mid].ent_off <= e) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
 // Adds the keys a, a + 1, .., b - 1 to a block's digit histograms: one count
 // per key for the lowest digit, one per run of equal digit above it.
 __device__ __forceinline__ void hist_key_run(uint32_t (*h)[RS_RADIX], int passes, uint32_t a, uint32_t b) {
@@ -777,18 +998,16 @@ __device__ __forceinline__ void hist_key_run(uint32_t (*h)[RS_RADIX], int passes
 // look-back over the earlier blocks' totals: work items are (entry, tile row);
 // each finds its reached columns once and writes that run (row-major inside an
 // entry), so a large rectangle is spread over the whole block and the stores
-// stay coalesced. Positions at or past cap are not written. With hist_passes > 0
-// the kernel also prepares the tile sort: it clears its look-back flags and
-// adds exactly the keys it writes to the digit histograms of its hist_passes
-// passes. KeyT: uint32_t, or uint16_t for the counting tile sort (tile ids
-// below 2^16).
-template <typename KeyT>
+// stay coalesced. Positions at or past cap are not written. The kernel also
+// prepares the radix tile sort: it clears its look-back flags and adds exactly
+// the keys it writes to the digit histograms of its hist_passes passes.
 __global__ void __launch_bounds__(256) k_duplicate(const Batch *__restrict__ bp, uint64_t M,
                                                    const uint32_t *__restrict__ sorted_ent,
                                                    const uint32_t *__restrict__ tiles_touched,
                                                    const uint2 *__restrict__ rect, const Rec *__restrict__ rec,
+                                                   const SortAux *__restrict__ depth_aux,
                                                    uint64_t *__restrict__ counters, uint64_t cap,
-                                                   KeyT *__restrict__ pkey,
+                                                   uint32_t *__restrict__ pkey,
                                                    uint32_t *__restrict__ pval, int hist_passes,
                                                    SortAux *__restrict__ aux, uint32_t *__restrict__ flags,
                                                    uint64_t flag_words, uint64_t *__restrict__ dflags,
@@ -804,14 +1023,20 @@ __global__ void __launch_bounds__(256) k_duplicate(const Batch *__restrict__ bp,
         flags[i] = 0u;
     for (int i = threadIdx.x; i < 4 * RS_RADIX; i += 256) h[i / RS_RADIX][i % RS_RADIX] = 0u;
     // a sort gave up a bounded wait: its order may hold stale words (uniform)
-    if (counters[CNT_STATUS] == (uint64_t)SG_ERR_TIMEOUT) return;
+    if (depth_aux->status) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            counters[CNT_STATUS] = depth_aux->status;
+            if (mirror) mirror[0] = 0;
+        }
+        return;
+    }
     if (threadIdx.x == 0)
         s_blk = atomicAdd(reinterpret_cast<unsigned long long *>(counters + CNT_DUP_BLOCK), 1ull);
     __syncthreads();
     const uint64_t blk = s_blk;
     const uint64_t j0 = blk * 256;
     const uint64_t j = j0 + threadIdx.x;
-    const uint64_t V = min(M, counters[CNT_VISIBLE]);   // entries in depth order with at least one pair
+    const uint64_t V = min(M, depth_aux->kept);   // entries in depth order with at least one pair
     if (j0 >= V) {   // no entry: only the first block, when there is none at all, reports the zero total
         if (V == 0 && blk == 0 && threadIdx.x == 0 && mirror) mirror[0] = 0;
         return;
@@ -893,11 +1118,11 @@ __global__ void __launch_bounds__(256) k_duplicate(const Batch *__restrict__ bp,
         for (int c = c0; c < c1; ++c) {
             const uint32_t q = at + (uint32_t)(c - c0);
             if (q < lim) {   // rows sum to tiles_touched by construction; never write past the block or cap
-                pkey[out0 + q] = (KeyT)(key0 + (uint32_t)c);
+                pkey[out0 + q] = key0 + (uint32_t)c;
                 pval[out0 + q] = s_e[o];
             }
         }
-        if (hist_passes > 0 && at < lim)   // the keys written above, no more
+        if (at < lim)   // the keys written above, no more
             hist_key_run(h, hist_passes, key0 + (uint32_t)c0,
                          key0 + (uint32_t)c0 + min((uint32_t)(c1 - c0), lim - at));
         done += chunk;
@@ -905,36 +1130,28 @@ __global__ void __launch_bounds__(256) k_duplicate(const Batch *__restrict__ bp,
     // Rows add up to tiles_touched by construction. Should they ever fall short,
     // the rest of the block's range still gets valid tile ids and entries.
     for (uint32_t q = done + threadIdx.x; q < lim; q += 256) {
-        pkey[out0 + q] = (KeyT)s_base[0];
+        pkey[out0 + q] = s_base[0];
         pval[out0 + q] = s_e[0];
-        if (hist_passes > 0) hist_key_run(h, hist_passes, s_base[0], s_base[0] + 1u);
+        hist_key_run(h, hist_passes, s_base[0], s_base[0] + 1u);
     }
-    if (hist_passes > 0) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < hist_passes * RS_RADIX; i += 256) {
-            const uint32_t c = h[i / RS_RADIX][i % RS_RADIX];
-            if (c) atomicAdd(&aux->hist[i / RS_RADIX][i % RS_RADIX], c);
-        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < hist_passes * RS_RADIX; i += 256) {
+        const uint32_t c = h[i / RS_RADIX][i % RS_RADIX];
+        if (c) atomicAdd(&aux->hist[i / RS_RADIX][i % RS_RADIX], c);
     }
 }
 
-cudaError_t launch_duplicate(const Batch *db, uint64_t M, const uint32_t *sorted_ent,
+cudaError_t launch_duplicate(const Batch *db, uint64_t M, const uint32_t *sorted_ent, const SortAux *depth_aux,
                              const uint32_t *tiles_touched, const uint2 *rect, const Rec *rec, uint64_t *counters,
-                             uint64_t cap, void *pkey, uint32_t *pval, uint64_t *dup_flags, uint64_t *mirror,
-                             cudaStream_t s, int hist_passes, uint64_t *sort_aux, uint32_t *flags,
-                             uint64_t flag_words, bool key16) {
-    if (key16 && hist_passes > 0) return cudaErrorInvalidValue;   // 16-bit keys feed the counting sort only
+                             uint64_t cap, uint32_t *pkey, uint32_t *pval, uint64_t *dup_flags, uint64_t *mirror,
+                             cudaStream_t s, int hist_passes, SortAux *sort_aux, uint32_t *flags,
+                             uint64_t flag_words) {
+    if (hist_passes < 1 || hist_passes > 4) return cudaErrorInvalidValue;
     // one block at least: it reports the zero total of a call without entries
     const uint64_t grid = std::max<uint64_t>(div_up(M, 256), 1);
-    SortAux *aux = reinterpret_cast<SortAux *>(sort_aux);
-    if (key16)
-        (void)launch_chain(k_duplicate<uint16_t>, dim3((unsigned)grid), dim3(256), s, db, M, sorted_ent,
-                           tiles_touched, rect, rec, counters, cap, static_cast<uint16_t *>(pkey), pval, hist_passes,
-                           aux, flags, flag_words, dup_flags, mirror, sort_wait_polls());
-    else
-        (void)launch_chain(k_duplicate<uint32_t>, dim3((unsigned)grid), dim3(256), s, db, M, sorted_ent,
-                           tiles_touched, rect, rec, counters, cap, static_cast<uint32_t *>(pkey), pval, hist_passes,
-                           aux, flags, flag_words, dup_flags, mirror, sort_wait_polls());
+    (void)launch_chain(k_duplicate, dim3((unsigned)grid), dim3(256), s, db, M, sorted_ent, tiles_touched, rect, rec,
+                       depth_aux, counters, cap, pkey, pval, hist_passes, sort_aux, flags, flag_words, dup_flags,
+                       mirror, sort_wait_polls());
     count_launches(1);
     return cudaGetLastError();
 }

@@ -1,0 +1,58 @@
+"""The chunked binning at the sizes where it can go wrong: one tile, ragged and
+empty views between full ones, more than 12288 tiles (sorted tile ids kept), an
+entry that covers a whole frame, views without any pair, and a view past the
+chunks' tile limit (radix passes). The lists are compared with the oracle's
+decisions and the library's binning rule bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2509_07021_gb300 import render, sgsplat, synth
+from paper_2509_07021_gb300.sgsplat import DeviceScene
+
+from parity_util import GpuView, check_decisions
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+AWAY = synth.look_at((0.0, 0.0, -9.0), (0.0, 0.0, -20.0))   # sees nothing
+
+CASES = {
+    # name: (Gaussians, views (width, height, fx, viewmat))
+    "one_tile": (500, [(16, 16, 20.0, None)]),
+    "ragged": (4000, [(129, 97, 110.0, None), (33, 47, 30.0, None), (17, 300, 60.0, None)]),
+    "empty_views": (3000, [(64, 48, 60.0, AWAY), (80, 50, 70.0, None), (40, 40, 45.0, AWAY), (48, 80, 60.0, None),
+                           (16, 16, 20.0, AWAY)]),
+    "all_empty": (300, [(64, 48, 60.0, AWAY), (80, 50, 70.0, AWAY)]),
+    "kept_tile_ids": (2500, [(1936, 1104, 1500.0, None), (1040, 800, 900.0, None), (700, 300, 400.0, None)]),
+    "past_the_chunk_limit": (400, [(3856, 3856, 3000.0, None), (64, 64, 60.0, None)]),
+}
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_lists_match_the_binning_rule(name):
+    n, views = CASES[name]
+    rng = np.random.default_rng(990)
+    scene = synth.make_scene(rng, n, lobes=1, means="cube", cube_side=1.4, masks="uniform")
+    scene.scales[:, 0] = 2.0      # covers whole frames
+    scene.opac[0] = scene.gmask[0] = 1.0
+    cams = [synth.make_camera(w, h, f, viewmat=vm) for w, h, f, vm in views]
+    ds = DeviceScene.from_host(scene)
+    out = render.render_forward(ds, cams)
+    lay = sgsplat.sg_workspace_layout(ds, cams, out.ws.numel())
+    assert (lay["pair_tile"] == sgsplat.NO_OFFSET) == (out.sizes["n_tiles"] <= 12288)
+    gv = GpuView.plain(ds, cams, out)
+    checks = []
+    for v, cam in enumerate(cams):
+        res, _ = oracle.render(scene, [cam], tile_sel=[np.zeros(cam.n_tiles, bool)])
+        checks.append((v, scene, res[0]))
+    check_decisions(gv, cams, checks)
+    assert gv.K == int(gv.tt.sum()) and (gv.K == 0) == (name == "all_empty")
+    # a second forward on the same workspace leaves the same lists
+    img, T, last = torch.empty_like(out.img), torch.empty_like(out.T_final), torch.empty_like(out.last)
+    st, sizes = sgsplat.sg_render_forward(ds, cams, out.ws, img, T, last, raise_on_error=False)
+    assert st == sgsplat.SG_OK and sizes["n_pairs"] == gv.K
+    again = GpuView.plain(ds, cams, out)
+    assert np.array_equal(again.pair_entry, gv.pair_entry) and np.array_equal(again.ranges, gv.ranges)
+    assert torch.equal(img, out.img) and torch.equal(T, out.T_final) and torch.equal(last, out.last)
