@@ -8,12 +8,17 @@
 //  * dual update: lambda += x - x~
 //
 // Selection is a radix select over order-preserving keys of the scores (the
-// kappa largest, equal scores by lower index): four passes over the keys, most
-// significant byte first, each histogramming the keys that match the threshold
-// digits found so far and picking the next digit where the running count
-// reaches kappa; then one pass that keeps every key below the threshold and the
+// kappa largest, equal scores by lower index): three passes over the key digits,
+// most significant first (11, 11 and 10 bits), each histogramming the keys that
+// match the threshold digits found so far and picking the next digit where the
+// running count reaches kappa (the first histogram is taken while the keys are
+// written); then one pass that keeps every key below the threshold and the
 // first of its ties in index order (a decoupled look-back over the blocks' tie
-// counts), and writes x~ and the new lambda.
+// counts), and writes x~ and the new lambda. The steps are bound by their few
+// short launches: 11-bit digits need one less than bytes, the final pass's
+// eight entries per thread move as 16-byte vectors, and it looks back only where
+// some but not all ties are kept (opacity and sharpness step of 1M Gaussians with
+// 1.65M lobes: 132 -> 61 us of kernels).
 #include "sg_internal.cuh"
 
 #include <algorithm>
@@ -40,20 +45,29 @@ struct SelState {
 
 constexpr int SEL_ITEMS = 8;                     // consecutive entries per thread in the final pass
 constexpr int SEL_TILE = 256 * SEL_ITEMS;
+constexpr int SEL_BINS = 2048, SEL_PASSES = 3;
+constexpr int SEL_PER = SEL_BINS / 256;          // bins per thread
+__host__ __device__ constexpr int sel_shift(int p) { return p == 0 ? 21 : p == 1 ? 10 : 0; }
+__host__ __device__ constexpr uint32_t sel_mask(int p) { return p == 2 ? 1023u : 2047u; }
 
-// Writes every key; the grid also zeroes the histograms and the look-back
-// words and thread 0 sets up the selection state.
-__device__ __forceinline__ void sel_setup(int64_t n, int64_t kappa, SelState *st, uint32_t *hist,
-                                          uint64_t *flags, uint64_t nflags) {
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t j = t; j < 4 * RS_RADIX; j += nth) hist[j] = 0u;
-    for (uint64_t j = t; j < nflags; j += nth) flags[j] = 0ull;
-    if (t == 0) {
+// Adds a block's digit counts to the pass's histogram and clears them.
+__device__ __forceinline__ void sel_flush(uint32_t *h, uint32_t *__restrict__ hist) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < SEL_BINS; i += 256)
+        if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
+__device__ __forceinline__ void sel_clear(uint32_t *h) {
+    for (int i = threadIdx.x; i < SEL_BINS; i += 256) h[i] = 0u;
+    __syncthreads();
+}
+
+// Writes every key and the first digit's histogram (state, histograms and
+// look-back words are zero on entry); thread 0 sets up the selection state.
+__device__ __forceinline__ void sel_setup(int64_t n, int64_t kappa, SelState *st) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->kappa = kappa;
         st->mode = kappa <= 0 ? 1 : (kappa >= n ? 2 : 0);
-        st->status = 0ull;
-        st->block_ctr = 0ull;
     }
 }
 
@@ -61,38 +75,52 @@ __global__ void __launch_bounds__(256) k_score_opacity(int64_t n, const float *_
                                                        const float *__restrict__ lam,
                                                        const float *__restrict__ score,
                                                        uint32_t *__restrict__ keys, int64_t kappa, SelState *st,
-                                                       uint32_t *hist, uint64_t *flags, uint64_t nflags) {
+                                                       uint32_t *__restrict__ hist) {
     chain_enter();
-    sel_setup(n, kappa, st, hist, flags, nflags);
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float z = __fadd_rn(x[i], lam[i]);
-    keys[i] = desc_key(score ? score[i] : fabsf(z));
+    __shared__ uint32_t h[SEL_BINS];
+    sel_setup(n, kappa, st);
+    sel_clear(h);
+    const int64_t nth = (int64_t)gridDim.x * 256;
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += nth) {
+        const uint32_t k = desc_key(score ? score[i] : fabsf(__fadd_rn(x[i], lam[i])));
+        keys[i] = k;
+        atomicAdd(&h[k >> sel_shift(0)], 1u);
+    }
+    sel_flush(h, hist);
 }
 
 __global__ void __launch_bounds__(256) k_score_sharpness(int64_t L, const float *__restrict__ s,
                                                          const float *__restrict__ lam,
                                                          const float *__restrict__ amp,
                                                          uint32_t *__restrict__ keys, int64_t kappa, SelState *st,
-                                                         uint32_t *hist, uint64_t *flags, uint64_t nflags) {
+                                                         uint32_t *__restrict__ hist) {
     chain_enter();
-    sel_setup(L, kappa, st, hist, flags, nflags);
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L) return;
-    const float z = __fadd_rn(s[i], lam[i]);
-    const float a0 = amp[i], a1 = amp[L + i], a2 = amp[2 * L + i];
-    const float na = sqrtf(a0 * a0 + a1 * a1 + a2 * a2);
-    const float D = na * fabsf(1.0f - expf(-2.0f * z));
-    keys[i] = desc_key(D);
+    __shared__ uint32_t h[SEL_BINS];
+    sel_setup(L, kappa, st);
+    sel_clear(h);
+    const int64_t nth = (int64_t)gridDim.x * 256;
+#pragma unroll 2
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < L; i += nth) {
+        const float z = __fadd_rn(s[i], lam[i]);
+        const float a0 = amp[i], a1 = amp[L + i], a2 = amp[2 * L + i];
+        const float na = sqrtf(a0 * a0 + a1 * a1 + a2 * a2);
+        const float D = na * fabsf(1.0f - expf(-2.0f * z));
+        const uint32_t k = desc_key(D);
+        keys[i] = k;
+        atomicAdd(&h[k >> sel_shift(0)], 1u);
+    }
+    sel_flush(h, hist);
 }
 
-// The threshold digits of the passes done so far, from their histograms (every
-// block of the later kernels redoes these picks; 256 threads, thread d: digit
-// d). Pass q's digit is the one where the running count of the keys matching
-// the earlier digits reaches the entries still to keep.
+// The threshold digits of the first `passes` passes, from their histograms
+// (every block of the later kernels redoes these picks; 256 threads, SEL_PER
+// bins each). Pass q's digit is the one where the running count of the keys
+// matching the earlier digits reaches the entries still to keep.
 struct SelPrefix {
     uint32_t prefix, mask;
     int64_t remaining;
+    int64_t matching;   // keys that match the digits found
     int32_t mode;
 };
 
@@ -100,24 +128,40 @@ __device__ __forceinline__ SelPrefix sel_resolve(const SelState *st, const uint3
                                                  int passes) {
     __shared__ uint64_t shs[33];
     __shared__ uint32_t s_digit;
-    __shared__ uint64_t s_below;
-    SelPrefix r{0u, 0u, st->kappa, st->mode};
+    __shared__ uint64_t s_below, s_match;
+    SelPrefix r{0u, 0u, st->kappa, 0, st->mode};
     for (int q = 0; q < passes && r.mode == 0; ++q) {   // uniform
-        const uint64_t c = hist[q * RS_RADIX + threadIdx.x];
+        uint32_t c[SEL_PER];
+        const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + q * SEL_BINS) + threadIdx.x * (SEL_PER / 4);
+#pragma unroll
+        for (int i = 0; i < SEL_PER / 4; ++i) {
+            const uint4 v = h4[i];
+            c[4 * i] = v.x; c[4 * i + 1] = v.y; c[4 * i + 2] = v.z; c[4 * i + 3] = v.w;
+        }
+        uint64_t sum = 0;
+#pragma unroll
+        for (int i = 0; i < SEL_PER; ++i) sum += c[i];
         uint64_t tot;
-        const uint64_t excl = block_exclusive<uint64_t>(c, tot, shs);
-        if ((int64_t)excl < r.remaining && r.remaining <= (int64_t)(excl + c)) {
-            s_digit = threadIdx.x;
-            s_below = excl;
+        uint64_t excl = block_exclusive<uint64_t>(sum, tot, shs);
+        if ((int64_t)excl < r.remaining && r.remaining <= (int64_t)(excl + sum)) {   // one thread
+#pragma unroll
+            for (int i = 0; i < SEL_PER; ++i) {
+                if ((int64_t)excl < r.remaining && r.remaining <= (int64_t)(excl + c[i])) {
+                    s_digit = threadIdx.x * SEL_PER + i;
+                    s_below = excl;
+                    s_match = c[i];
+                }
+                excl += c[i];
+            }
         }
         __syncthreads();
         if ((int64_t)tot < r.remaining) {   // fewer keys than asked (not expected): keep them all
             r.mode = 2;
         } else {
-            const int shift = 24 - 8 * q;
-            r.prefix |= s_digit << shift;
-            r.mask |= 0xFFu << shift;
+            r.prefix |= s_digit << sel_shift(q);
+            r.mask |= sel_mask(q) << sel_shift(q);
             r.remaining -= (int64_t)s_below;
+            r.matching = (int64_t)s_match;
         }
         __syncthreads();   // s_digit / s_below are rewritten by the next pass
     }
@@ -129,30 +173,27 @@ __device__ __forceinline__ SelPrefix sel_resolve(const SelState *st, const uint3
 __global__ void __launch_bounds__(256) k_sel_hist(int64_t n, const uint32_t *__restrict__ keys,
                                                   const SelState *st, uint32_t *__restrict__ hist, int p) {
     chain_enter();
-    __shared__ uint32_t h[RS_RADIX];
+    __shared__ uint32_t h[SEL_BINS];
     const SelPrefix r = sel_resolve(st, hist, p);
-    h[threadIdx.x] = 0u;
-    __syncthreads();
-    const int shift = 24 - 8 * p;
-    if (r.mode == 0) {   // uniform
-        const uint32_t pre = r.prefix, msk = r.mask;
-        const int64_t n4 = n / 4;
-        const uint4 *k4 = reinterpret_cast<const uint4 *>(keys);
-        const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
-        for (int64_t j = t; j < n4; j += nth) {
-            const uint4 k = k4[j];
-            if ((k.x & msk) == pre) atomicAdd(&h[(k.x >> shift) & 255u], 1u);
-            if ((k.y & msk) == pre) atomicAdd(&h[(k.y >> shift) & 255u], 1u);
-            if ((k.z & msk) == pre) atomicAdd(&h[(k.z >> shift) & 255u], 1u);
-            if ((k.w & msk) == pre) atomicAdd(&h[(k.w >> shift) & 255u], 1u);
-        }
-        for (int64_t j = 4 * n4 + t; j < n; j += nth) {
-            const uint32_t k = keys[j];
-            if ((k & msk) == pre) atomicAdd(&h[(k >> shift) & 255u], 1u);
-        }
+    if (r.mode != 0) return;   // uniform
+    sel_clear(h);
+    const int shift = sel_shift(p);
+    const uint32_t pre = r.prefix, msk = r.mask, dm = sel_mask(p);
+    const int64_t n4 = n / 4;
+    const uint4 *k4 = reinterpret_cast<const uint4 *>(keys);
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x, nth = (int64_t)gridDim.x * 256;
+    for (int64_t j = t; j < n4; j += nth) {
+        const uint4 k = k4[j];
+        if ((k.x & msk) == pre) atomicAdd(&h[(k.x >> shift) & dm], 1u);
+        if ((k.y & msk) == pre) atomicAdd(&h[(k.y >> shift) & dm], 1u);
+        if ((k.z & msk) == pre) atomicAdd(&h[(k.z >> shift) & dm], 1u);
+        if ((k.w & msk) == pre) atomicAdd(&h[(k.w >> shift) & dm], 1u);
     }
-    __syncthreads();
-    if (h[threadIdx.x]) atomicAdd(&hist[p * RS_RADIX + threadIdx.x], h[threadIdx.x]);
+    for (int64_t j = 4 * n4 + t; j < n; j += nth) {
+        const uint32_t k = keys[j];
+        if ((k & msk) == pre) atomicAdd(&h[(k >> shift) & dm], 1u);
+    }
+    sel_flush(h, hist + p * SEL_BINS);
 }
 
 __global__ void __launch_bounds__(256) k_penalty_grad(int64_t n, const float *__restrict__ x,
@@ -169,33 +210,55 @@ __global__ void __launch_bounds__(256) k_penalty_grad(int64_t n, const float *__
 // + 0 .. SEL_ITEMS - 1 (consecutive, so block and thread prefixes of the tie
 // counts follow the index order). Keeps the keys below the threshold and the
 // first `remaining` keys equal to it; writes x~ = z (kept) or 0 and
-// lambda += x - x~.
+// lambda += x - x~. vec: x, lam and x_tilde are 16-byte aligned (a thread's
+// eight entries then move as two vectors each).
 __global__ void __launch_bounds__(256) k_sel_final(int64_t n, const uint32_t *__restrict__ keys,
                                                    const float *__restrict__ x, float *__restrict__ lam,
                                                    float *__restrict__ x_tilde, SelState *st,
                                                    const uint32_t *__restrict__ hist,
-                                                   uint64_t *__restrict__ flags, uint32_t spin_limit) {
+                                                   uint64_t *__restrict__ flags, uint32_t spin_limit, bool vec) {
     chain_enter();
     __shared__ uint32_t shs[33];
     __shared__ uint64_t s_blk, s_excl;
     if (threadIdx.x == 0) s_blk = atomicAdd(reinterpret_cast<unsigned long long *>(&st->block_ctr), 1ull);
     __syncthreads();
     const uint64_t blk = s_blk;
-    const SelPrefix r = sel_resolve(st, hist, 4);
+    const SelPrefix r = sel_resolve(st, hist, SEL_PASSES);
     const int32_t mode = r.mode;
-    const uint32_t T = r.prefix;          // the threshold key (all four digits)
+    const uint32_t T = r.prefix;          // the threshold key (every digit)
     const int64_t rem = r.remaining;      // its ties to keep
+    // all of them (the scores are mostly distinct): no rank among the ties is needed
+    const bool ranked = mode == 0 && rem < r.matching;   // uniform over the grid
     const int64_t i0 = (int64_t)blk * SEL_TILE + (int64_t)threadIdx.x * SEL_ITEMS;
+    const bool whole = vec && i0 + SEL_ITEMS <= n;
     uint32_t k[SEL_ITEMS];
+    float xv[SEL_ITEMS], lv[SEL_ITEMS];
+    if (whole) {
+        const uint4 *k4 = reinterpret_cast<const uint4 *>(keys + i0);
+        const float4 *x4 = reinterpret_cast<const float4 *>(x + i0), *l4 = reinterpret_cast<const float4 *>(lam + i0);
+#pragma unroll
+        for (int q = 0; q < SEL_ITEMS / 4; ++q) {
+            const uint4 kq = k4[q];
+            const float4 xq = x4[q], lq = l4[q];
+            k[4 * q] = kq.x; k[4 * q + 1] = kq.y; k[4 * q + 2] = kq.z; k[4 * q + 3] = kq.w;
+            xv[4 * q] = xq.x; xv[4 * q + 1] = xq.y; xv[4 * q + 2] = xq.z; xv[4 * q + 3] = xq.w;
+            lv[4 * q] = lq.x; lv[4 * q + 1] = lq.y; lv[4 * q + 2] = lq.z; lv[4 * q + 3] = lq.w;
+        }
+    } else {
+#pragma unroll
+        for (int it = 0; it < SEL_ITEMS; ++it) {
+            const bool on = i0 + it < n;
+            k[it] = on ? keys[i0 + it] : 0xFFFFFFFFu;
+            xv[it] = on ? x[i0 + it] : 0.f;
+            lv[it] = on ? lam[i0 + it] : 0.f;
+        }
+    }
     uint32_t ties = 0u;
 #pragma unroll
-    for (int it = 0; it < SEL_ITEMS; ++it) {
-        k[it] = i0 + it < n ? keys[i0 + it] : 0xFFFFFFFFu;
-        ties += (mode == 0 && i0 + it < n && k[it] == T) ? 1u : 0u;
-    }
-    uint32_t btot;
-    uint32_t rank = block_exclusive<uint32_t>(ties, btot, shs);   // ties in earlier threads of the block
-    if (mode == 0) {   // uniform: ties in earlier blocks
+    for (int it = 0; it < SEL_ITEMS; ++it) ties += (mode == 0 && i0 + it < n && k[it] == T) ? 1u : 0u;
+    uint32_t btot, rank = 0u;
+    if (ranked) {
+        rank = block_exclusive<uint32_t>(ties, btot, shs);   // ties in earlier threads of the block, then blocks
         if (threadIdx.x == 0) st_relaxed64(flags + blk, DL_AGG | ((uint64_t)btot & DL_VAL));
         if (threadIdx.x < 32) {
             const uint64_t excl = block_lookback64(flags, blk, btot, spin_limit, &st->status);
@@ -203,32 +266,44 @@ __global__ void __launch_bounds__(256) k_sel_final(int64_t n, const uint32_t *__
         }
         __syncthreads();
     }
-    const uint64_t before = mode == 0 ? s_excl : 0ull;
+    const uint64_t before = ranked ? s_excl : 0ull;
 #pragma unroll
     for (int it = 0; it < SEL_ITEMS; ++it) {
-        const int64_t i = i0 + it;
-        if (i >= n) break;
         bool keep = mode == 2;
         if (mode == 0) {
             if (k[it] < T) {
                 keep = true;
-            } else if (k[it] == T) {
-                keep = (int64_t)(before + rank) < rem;
+            } else if (k[it] == T && i0 + it < n) {
+                keep = !ranked || (int64_t)(before + rank) < rem;
                 ++rank;
             }
         }
-        const float xi = x[i], li = lam[i];
-        const float z = __fadd_rn(xi, li);
+        const float z = __fadd_rn(xv[it], lv[it]);
         const float xt = keep ? z : 0.0f;
-        x_tilde[i] = xt;
-        lam[i] = __fadd_rn(li, __fsub_rn(xi, xt));
+        lv[it] = __fadd_rn(lv[it], __fsub_rn(xv[it], xt));
+        xv[it] = xt;
+    }
+    if (whole) {
+        float4 *t4 = reinterpret_cast<float4 *>(x_tilde + i0), *l4 = reinterpret_cast<float4 *>(lam + i0);
+#pragma unroll
+        for (int q = 0; q < SEL_ITEMS / 4; ++q) {
+            t4[q] = make_float4(xv[4 * q], xv[4 * q + 1], xv[4 * q + 2], xv[4 * q + 3]);
+            l4[q] = make_float4(lv[4 * q], lv[4 * q + 1], lv[4 * q + 2], lv[4 * q + 3]);
+        }
+    } else {
+#pragma unroll
+        for (int it = 0; it < SEL_ITEMS; ++it) {
+            if (i0 + it >= n) break;
+            x_tilde[i0 + it] = xv[it];
+            lam[i0 + it] = lv[it];
+        }
     }
 }
 
-// Workspace: the selection state, the keys, the 4 passes' histograms and the
-// final pass's look-back words.
+// Workspace: the selection state, the passes' histograms and the final pass's
+// look-back words (zeroed together), and the keys.
 struct AdmmLayout {
-    size_t state, keys, hist, flags, total;
+    size_t state, hist, flags, zeroed, keys, total;
     uint64_t nflags;
 };
 
@@ -239,10 +314,11 @@ static AdmmLayout admm_layout(int64_t n) {
     size_t o = 0;
     auto take = [&](size_t b) { size_t r = o; o += al256(b); return r; };
     L.state = take(sizeof(SelState));
-    L.keys = take(4 * (size_t)n);
-    L.hist = take((size_t)4 * RS_RADIX * 4);
+    L.hist = take((size_t)SEL_PASSES * SEL_BINS * 4);
     L.nflags = std::max<uint64_t>(div_up((uint64_t)n, SEL_TILE), 1);
     L.flags = take(8 * L.nflags);
+    L.zeroed = o;
+    L.keys = take(4 * (size_t)n);
     L.total = o;
     return L;
 }
@@ -260,21 +336,22 @@ cudaError_t launch_admm_step(int kind, int64_t n, const float *x, const float *s
     uint32_t *keys = reinterpret_cast<uint32_t *>(w + L.keys);
     uint32_t *hist = reinterpret_cast<uint32_t *>(w + L.hist);
     uint64_t *flags = reinterpret_cast<uint64_t *>(w + L.flags);
-    const dim3 grid((unsigned)div_up((uint64_t)n, 256));
+    const cudaError_t e = cudaMemsetAsync(w, 0, L.zeroed, s);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)std::min<uint64_t>(div_up((uint64_t)n, 256 * 8), 4 * 152));
     if (kind == 0)
-        (void)launch_chain(k_score_opacity, grid, dim3(256), s, n, x, lam, score, keys, kappa, st, hist, flags,
-                           L.nflags);
+        (void)launch_chain(k_score_opacity, grid, dim3(256), s, n, x, lam, score, keys, kappa, st, hist);
     else
-        (void)launch_chain(k_score_sharpness, grid, dim3(256), s, n, x, lam, amp, keys, kappa, st, hist, flags,
-                           L.nflags);
-    const unsigned hgrid = (unsigned)std::min<uint64_t>(std::max<uint64_t>(div_up((uint64_t)n, 256 * 16), 1),
-                                                        4 * 152);
-    for (int p = 0; p < 4; ++p)
+        (void)launch_chain(k_score_sharpness, grid, dim3(256), s, n, x, lam, amp, keys, kappa, st, hist);
+    const unsigned hgrid = (unsigned)std::min<uint64_t>(div_up((uint64_t)n, 256 * 16), 4 * 152);
+    for (int p = 1; p < SEL_PASSES; ++p)
         (void)launch_chain(k_sel_hist, dim3(hgrid), dim3(256), s, n, (const uint32_t *)keys, (const SelState *)st,
                            hist, p);
+    const bool vec = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(lam) |
+                       reinterpret_cast<uintptr_t>(x_tilde)) & 15u) == 0u;
     (void)launch_chain(k_sel_final, dim3((unsigned)L.nflags), dim3(256), s, n, (const uint32_t *)keys, x, lam,
-                       x_tilde, st, (const uint32_t *)hist, flags, sort_wait_polls());
-    count_launches(6);
+                       x_tilde, st, (const uint32_t *)hist, flags, sort_wait_polls(), vec);
+    count_launches(2 + SEL_PASSES - 1);
     return cudaGetLastError();
 }
 
