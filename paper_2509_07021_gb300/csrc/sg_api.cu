@@ -1043,9 +1043,11 @@ int sg_postprocess_plan(const sg_scene *in, float tau_opacity, float tau_sharpne
     g_err[0] = '\0';
     int st = post_check(in, ws, ws_bytes);
     if (st != SG_OK) return st;
-    uint64_t totals[2] = {0, 0};
+    uint64_t totals[3] = {0, 0, 0};   // Gaussians, lobes, device status
     SG_CUDA(launch_post_plan(*in, tau_opacity, tau_sharpness, ws, totals, static_cast<cudaStream_t>(stream)),
             "post-processing plan");
+    if (totals[2] != (uint64_t)SG_OK)
+        return fail(SG_ERR_TIMEOUT, "the plan's bounded device wait expired (workspace unspecified)");
     if (n_out) *n_out = (int64_t)totals[0];
     if (l_out) *l_out = (int64_t)totals[1];
     return SG_OK;
@@ -1064,7 +1066,7 @@ int sg_postprocess_apply(const sg_scene *in, float tau_opacity, float tau_sharpn
     }
     if (out->n_lobes > 0 && (!out->axis || !out->sharp || !out->amp || !out->lmask))
         return fail(SG_ERR_INVALID_ARG, "an output lobe array is NULL");
-    SG_CUDA(launch_post_apply(*in, tau_opacity, tau_sharpness, ws, *out, out->n, out->n_lobes,
+    SG_CUDA(launch_post_apply(*in, tau_sharpness, ws, *out, out->n, out->n_lobes,
                               static_cast<cudaStream_t>(stream)),
             "post-processing apply");
     return SG_OK;

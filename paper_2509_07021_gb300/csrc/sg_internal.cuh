@@ -88,7 +88,6 @@ constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = SG_RS_ITEMS;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;   // 3072 keys per block
 constexpr int RS_RADIX = 256;
-constexpr int SCAN_TILE = 4096;
 
 // Byte offsets of every workspace buffer (host computed, identical for the
 // forward and the backward of one call).
@@ -368,15 +367,6 @@ cudaError_t launch_preprocess_backward(const Batch &hb, const Batch *db,
                                        const uint32_t *tiles_touched, const uint8_t *clamp, const float *dg,
                                        uint64_t M, cudaStream_t s);
 
-// Exclusive scan of `in` (or of tiles_touched[idx[i]] when idx != null) into
-// `out`, total written to *total. n items (host known), or min(n, *n_dev) when
-// n_dev is given. mirror (nullable, host memory mapped into the device): also
-// receives the total and *status_src in its first two words.
-cudaError_t launch_scan(const uint32_t *in, const uint32_t *gather_idx, uint32_t *out,
-                        uint64_t n, uint64_t *block_sums, uint64_t *total, cudaStream_t s,
-                        const uint64_t *n_dev = nullptr, uint64_t *mirror = nullptr,
-                        const uint64_t *status_src = nullptr);
-
 constexpr size_t SORT_AUX_BYTES = 16384;
 // Most keys one sort takes (its look-back words carry 30-bit counts).
 constexpr uint64_t SORT_MAX_KEYS = (1ull << 30) - 1;
@@ -529,11 +519,12 @@ cudaError_t launch_admm_step(int kind, int64_t n, const float *x, const float *s
 cudaError_t launch_penalty_grad(int64_t n, const float *x, const float *x_tilde, const float *lam, float delta,
                                 float *grad, cudaStream_t s);
 
-// Post-processing (Sec. 3.3.3): plan (flags, scans, totals read back) and apply.
+// Post-processing (Sec. 3.3.3): plan (positions; totals and the device status
+// read back into totals_host[3]) and apply.
 size_t post_workspace_bytes(int64_t n);
 cudaError_t launch_post_plan(const sg_scene &sc, float tau_o, float tau_s, void *ws, uint64_t *totals_host,
                              cudaStream_t s);
-cudaError_t launch_post_apply(const sg_scene &sc, float tau_o, float tau_s, const void *ws, const sg_scene &out,
+cudaError_t launch_post_apply(const sg_scene &sc, float tau_s, const void *ws, const sg_scene &out,
                               int64_t n_out, int64_t l_out, cudaStream_t s);
 
 // Resident blocks per SM x SMs for the persistent blend of this shape.

@@ -1,5 +1,5 @@
-// Binning: exclusive scan, stable LSD radix sort of u32 (key, value) pairs,
-// duplicateWithKeys and per-tile ranges.
+// Binning: stable LSD radix sort of u32 (key, value) pairs, duplicateWithKeys,
+// the chunked binning and per-tile ranges.
 //
 // The (tile, depth) ordering of the paper's tile-depth-Gaussian key table
 // (Sec. 1, rendering VRAM; the 3DGS binning it inherits) is the order of an
@@ -20,124 +20,6 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return (1u << (threadIdx.x & 31)) - 1u;
 }
 
-
-// ---------------------------------------------------------------------------
-// exclusive scan: reduce -> spine -> downsweep
-// ---------------------------------------------------------------------------
-// With idx, in[idx[i]]; an index outside in's n_in items reads 0. (Indices
-// come from a sort whose bounded wait may have given up, leaving stale words
-// in its output: the gather stays inside the array whatever they hold.)
-__device__ __forceinline__ uint32_t scan_load(const uint32_t *in, const uint32_t *idx, uint64_t i, uint64_t n_in) {
-    if (!idx) return in[i];
-    const uint32_t e = idx[i];
-    return e < n_in ? in[e] : 0u;
-}
-
-__global__ void __launch_bounds__(256) k_scan_reduce(const uint32_t *__restrict__ in,
-                                                     const uint32_t *__restrict__ idx, uint64_t n_in, uint64_t n,
-                                                     const uint64_t *__restrict__ n_dev,
-                                                     uint64_t *__restrict__ sums) {
-    __shared__ uint64_t sh[33];
-    if (n_dev) n = min(n, *n_dev);
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
-    uint64_t acc = 0;
-#pragma unroll 4
-    for (int i = 0; i < SCAN_TILE / 256; ++i) {
-        const uint64_t j = base + (uint64_t)i * 256 + threadIdx.x;
-        if (j < n) acc += scan_load(in, idx, j, n_in);
-    }
-    uint64_t tot;
-    block_exclusive<uint64_t>(acc, tot, sh);
-    if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-// mirror (nullable; host memory mapped into the device): receives the total
-// and *status_src, so the host can read both without a copy in the stream.
-__global__ void __launch_bounds__(1024) k_scan_spine(uint64_t *__restrict__ sums, uint64_t nb,
-                                                     uint64_t *__restrict__ total, uint64_t *mirror,
-                                                     const uint64_t *status_src) {
-    __shared__ uint64_t sh[33];
-    const uint64_t per = div_up(nb, 1024);
-    const uint64_t lo = threadIdx.x * per, hi = min(nb, lo + per);
-    uint64_t acc = 0;
-    for (uint64_t i = lo; i < hi; ++i) acc += sums[i];
-    uint64_t tot;
-    uint64_t run = block_exclusive<uint64_t>(acc, tot, sh);
-    for (uint64_t i = lo; i < hi; ++i) {
-        const uint64_t v = sums[i];
-        sums[i] = run;
-        run += v;
-    }
-    if (threadIdx.x == 0 && total) *total = tot;
-    if (threadIdx.x == 0 && mirror) {
-        mirror[0] = tot;
-        mirror[1] = status_src ? *status_src : 0;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_scan_down(const uint32_t *__restrict__ in,
-                                                   const uint32_t *__restrict__ idx, uint64_t n_in, uint64_t n,
-                                                   const uint64_t *__restrict__ n_dev,
-                                                   const uint64_t *__restrict__ sums,
-                                                   uint32_t *__restrict__ out) {
-    if (n_dev) n = min(n, *n_dev);
-    // each thread owns 16 consecutive items, staged through shared memory
-    __shared__ uint32_t buf[SCAN_TILE + SCAN_TILE / 32];
-    __shared__ uint64_t sh[33];
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
-#pragma unroll 4
-    for (int i = 0; i < SCAN_TILE / 256; ++i) {
-        const int p = i * 256 + threadIdx.x;
-        const uint64_t j = base + p;
-        buf[p + (p >> 5)] = j < n ? scan_load(in, idx, j, n_in) : 0u;
-    }
-    __syncthreads();
-    uint32_t loc[16];
-    uint64_t acc = 0;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int p = threadIdx.x * 16 + k;
-        loc[k] = buf[p + (p >> 5)];
-        acc += loc[k];
-    }
-    uint64_t tot;
-    uint64_t run = block_exclusive<uint64_t>(acc, tot, sh) + sums[blockIdx.x];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int p = threadIdx.x * 16 + k;
-        buf[p + (p >> 5)] = (uint32_t)run;
-        run += loc[k];
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int i = 0; i < SCAN_TILE / 256; ++i) {
-        const int p = i * 256 + threadIdx.x;
-        const uint64_t j = base + p;
-        if (j < n) out[j] = buf[p + (p >> 5)];
-    }
-}
-
-cudaError_t launch_scan(const uint32_t *in, const uint32_t *gather_idx, uint32_t *out, uint64_t n,
-                        uint64_t *block_sums, uint64_t *total, cudaStream_t s, const uint64_t *n_dev,
-                        uint64_t *mirror, const uint64_t *status_src) {
-    const uint64_t nb = div_up(n, SCAN_TILE);
-    if (nb == 0) {
-        if (mirror) {   // the spine alone writes the zero total
-            k_scan_spine<<<1, 1024, 0, s>>>(block_sums, 0, total, mirror, status_src);
-            count_launches(1);
-            return cudaGetLastError();
-        }
-        if (total) return cudaMemsetAsync(total, 0, sizeof(uint64_t), s);
-        return cudaSuccess;
-    }
-    k_scan_reduce<<<(unsigned)nb, 256, 0, s>>>(in, gather_idx, n, n, n_dev, block_sums);
-    count_launches(1);
-    k_scan_spine<<<1, 1024, 0, s>>>(block_sums, nb, total, mirror, status_src);
-    count_launches(1);
-    k_scan_down<<<(unsigned)nb, 256, 0, s>>>(in, gather_idx, n, n, n_dev, block_sums, out);
-    count_launches(1);
-    return cudaGetLastError();
-}
 
 // ---------------------------------------------------------------------------
 // stable LSD radix sort, 8-bit digits, RS_TILE keys per block, one sweep per pass
