@@ -141,7 +141,7 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
     std::memset(&b, 0, sizeof(Batch));
     b.n_views = n_views;
     b.n_scenes = n_scenes;
-    uint64_t bwd_blk = 0;
+    uint64_t bwd_blk = 0, runs = 0;
     for (int s = 0; s < n_scenes; ++s) {
         const sg_scene &sc = scenes[s];
         if (sc.n < 0 || sc.n > (int64_t)INT32_MAX - PRE_THREADS)
@@ -183,6 +183,8 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
         d.dtype_geom = sc.dtype_geom; d.dtype_lobe = sc.dtype_lobe; d.dtype_sharp = sc.dtype_sharp;
         d.blk_off = (uint32_t)bwd_blk;
         bwd_blk += div_up((uint64_t)sc.n, PRE_THREADS);
+        d.run_off = (uint32_t)runs;
+        runs += div_up((uint64_t)sc.n, PRE_RUN);
     }
     uint64_t tiles = 0, groups = 0, pix = 0, ent = 0;
     for (int v = 0; v < n_views; ++v) {
@@ -208,6 +210,10 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
         d.near_plane = c.near_plane;
         d.bg[0] = c.bg[0]; d.bg[1] = c.bg[1]; d.bg[2] = c.bg[2];
         d.W = c.width; d.H = c.height;
+        // one rounded operation per step, as the decision recipe states them
+        const float tanx = (0.5f * (float)c.width) / c.fx, tany = (0.5f * (float)c.height) / c.fy;
+        d.limx = 1.3f * tanx;
+        d.limy = 1.3f * tany;
         d.tiles_x = (c.width + TILE - 1) / TILE;
         d.tiles_y = (c.height + TILE - 1) / TILE;
         d.scene = s;
@@ -229,6 +235,7 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
     b.n_groups = (uint32_t)groups;
     b.n_entries = ent;
     b.scene_blocks = (uint32_t)bwd_blk;
+    b.scene_runs = (uint32_t)runs;
     uint32_t per_scene[SG_MAX_SCENES] = {};
     b.max_views_per_scene = 0;
     for (int v = 0; v < n_views; ++v) {
@@ -327,7 +334,7 @@ uint64_t capacity_for(const Batch &b, size_t ws_bytes) {
     return lo;
 }
 
-// Backward scratch: batch table, counters and the [9][M] 2D gradients (the
+// Backward scratch: batch table, counters and the [M][9] 2D gradients (the
 // persistent backward takes its tile order from the forward's workspace).
 struct BwdLayout {
     size_t batch, counters, dg, total;
@@ -1094,7 +1101,7 @@ int sg_forward_status(const void *ws, uint64_t *n_pairs, int32_t *status, void *
 namespace {
 
 // Scratch of sg_render_backward_noalloc: batch table, counters and the
-// [9][M] per-entry 2D-gradient accumulators. Every device that loads the
+// [M][9] per-entry 2D-gradient accumulators. Every device that loads the
 // library holds it until the process exits.
 __device__ __align__(256) unsigned char g_noalloc_scratch[SG_NOALLOC_SCRATCH_BYTES];
 

@@ -455,11 +455,12 @@ cudaError_t launch_blend_forward(const Batch *db, uint32_t n_tiles, const uint2 
 // ---------------------------------------------------------------------------
 // K7 blend backward
 // ---------------------------------------------------------------------------
-// Sums 9 per-lane values over the warp and adds them to dg[k*M + e] (value k
-// scaled by sc[k]). Recursive halving: 4 + 2 + 1 shuffles leave each group of
-// four lanes with one of the first eight sums, two more finish it; the ninth
-// value takes a plain butterfly. Eight lanes issue their atomics together.
-__device__ __forceinline__ void warp_sum9_atomic(const float v[9], float *dg, uint64_t M, uint32_t e) {
+// Sums 9 per-lane values over the warp and adds them to the entry's nine
+// consecutive sums at dg9. Recursive halving: 4 + 2 + 1 shuffles leave each
+// group of four lanes with one of the first eight sums, two more finish it; the
+// ninth value takes a plain butterfly. Nine lanes issue one atomic together, on
+// two sectors.
+__device__ __forceinline__ void warp_sum9_atomic(const float v[9], float *dg9) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool h1 = lane & 16, h2 = lane & 8, h3 = lane & 4;
@@ -483,11 +484,8 @@ __device__ __forceinline__ void warp_sum9_atomic(const float v[9], float *dg, ui
     float d = v[8];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(FULL, d, o);
-    if ((lane & 3) == 0) {
-        const int idx = (h1 ? 4 : 0) + (h2 ? 2 : 0) + (h3 ? 1 : 0);
-        atomicAdd(dg + (uint64_t)idx * M + e, c);
-    }
-    if (lane == 1) atomicAdd(dg + 8 * M + e, d);
+    // sum i (i < 8) is in lanes 4 i .. 4 i + 3, the ninth in every lane: lane 1 adds it
+    if ((lane & 3) == 0 || lane == 1) atomicAdd(dg9 + (lane == 1 ? 8 : lane >> 2), lane == 1 ? d : c);
 }
 
 // Adds one pixel's share of one blended pair to v (in dg order) and steps the
@@ -537,7 +535,7 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                                                const float *__restrict__ T_final,
                                                const int32_t *__restrict__ last,
                                                const float *__restrict__ d_img, float *__restrict__ dg,
-                                               uint64_t M, uint32_t &ne, bool lists_ok, int nb) {
+                                               uint32_t &ne, bool lists_ok, int nb) {
     constexpr int NT = BLEND_THREADS / P;
     int tx, ty;
     const ViewDesc *vw;
@@ -658,7 +656,7 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
             }
             // the moments are linear in dP: the conic factors and 1/o' are applied
             // once per entry by the preprocess adjoint, after the sum over tiles
-            if (__any_sync(0xffffffffu, any)) warp_sum9_atomic(v, dg, M, sm.id[k]);
+            if (__any_sync(0xffffffffu, any)) warp_sum9_atomic(v, dg + 9 * (uint64_t)sm.id[k]);
         }
     }
 }
@@ -683,7 +681,7 @@ k_blend_bwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
     const bool lists_ok = *status != (uint64_t)SG_ERR_TIMEOUT;
     if (!PERSIST) {
         blend_bwd_tile<P, COUNT>(b, blockIdx.x, sm, smax, spx, slot_last, ranges, pval, rec, T_final, last,
-                                 d_img, dg, M, ne, lists_ok, nb);
+                                 d_img, dg, ne, lists_ok, nb);
     } else {
         for (;;) {
             if (threadIdx.x == 0) s_item = atomicAdd(queue, 1u);
@@ -692,7 +690,7 @@ k_blend_bwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
             __syncthreads();
             if (item >= n_tiles) break;
             blend_bwd_tile<P, COUNT>(b, tile_order ? tile_order[item] : item, sm, smax, spx, slot_last, ranges,
-                                     pval, rec, T_final, last, d_img, dg, M, ne, lists_ok, nb);
+                                     pval, rec, T_final, last, d_img, dg, ne, lists_ok, nb);
         }
     }
     if (COUNT) add_evals(ne, evals);

@@ -15,6 +15,7 @@ namespace sgk {
 constexpr int TILE = SG_TILE;             // 16x16 pixel tiles
 constexpr int BLEND_THREADS = TILE * TILE;
 constexpr int PRE_THREADS = 256;
+constexpr int PRE_RUN = 512;    // scene Gaussians per block of the several-view preprocess kernels
 
 // Per-view camera and packing offsets. Built on the host, copied into the
 // workspace by k_setup so that kernels take a single pointer.
@@ -29,6 +30,7 @@ struct ViewDesc {
     int32_t n;            // Gaussians of that scene
     uint32_t tile_off;    // first global tile id of the view
     uint32_t grp_off;     // first group of 32 tiles of the view (the binning's scan)
+    float limx, limy;     // guard band: 1.3 tan(fov / 2) per axis
     uint32_t pad0;
     uint64_t pix_off;     // first pixel of the view in T_final / last (img: x3)
     uint64_t ent_off;     // first (view, Gaussian) entry of the view
@@ -45,7 +47,8 @@ struct SceneDesc {
     sg_grads grads;
     int64_t n, n_lobes;
     int32_t dtype_geom, dtype_lobe, dtype_sharp, color_model;
-    uint32_t blk_off;     // first block of the scene in the per-Gaussian preprocess grids
+    uint32_t blk_off;     // first block of the scene in the per-Gaussian grids (PRE_THREADS a block)
+    uint32_t run_off;     // and in the several-view grids (PRE_RUN a block)
 };
 
 struct Batch {
@@ -54,6 +57,8 @@ struct Batch {
     uint32_t scene_blocks;   // blocks of 256 scene Gaussians over all scenes
     uint32_t max_views_per_scene;
     uint32_t n_groups;       // groups of 32 tiles over all views
+    uint32_t scene_runs;     // blocks of PRE_RUN scene Gaussians over all scenes
+    uint32_t pad0;
     uint64_t n_entries;
     ViewDesc view[SG_MAX_VIEWS];
     SceneDesc scene[SG_MAX_SCENES];

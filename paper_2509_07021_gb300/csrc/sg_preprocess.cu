@@ -128,9 +128,7 @@ __device__ __forceinline__ void project_view(const ViewDesc &vw, float px, float
         }
 
     const float fx = vw.fx, fy = vw.fy;
-    const float tanx = fdv(fm(0.5f, (float)vw.W), fx);
-    const float tany = fdv(fm(0.5f, (float)vw.H), fy);
-    const float limx = fm(1.3f, tanx), limy = fm(1.3f, tany);
+    const float limx = vw.limx, limy = vw.limy;
     g.ux = fdv(g.tx, g.tz);
     g.uy = fdv(g.ty, g.tz);
     g.ccx = fm(fminf(limx, fmaxf(-limx, g.ux)), g.tz);
@@ -165,10 +163,11 @@ __device__ __forceinline__ void project_view(const ViewDesc &vw, float px, float
     g.rf = ceilf(fm(3.f, fsq(lam1)));
     g.x = fs(fa(fm(fx, g.ux), vw.cx), 0.5f);
     g.y = fs(fa(fm(fy, g.uy), vw.cy), 0.5f);
-    g.x0 = clamp_tile(floorf(fdv(fs(g.x, g.rf), 16.f)), vw.tiles_x);
-    g.x1 = clamp_tile(floorf(fdv(fa(fa(g.x, g.rf), 15.f), 16.f)), vw.tiles_x);
-    g.y0 = clamp_tile(floorf(fdv(fs(g.y, g.rf), 16.f)), vw.tiles_y);
-    g.y1 = clamp_tile(floorf(fdv(fa(fa(g.y, g.rf), 15.f), 16.f)), vw.tiles_y);
+    // (dividing by 16 and multiplying by 1/16 round alike)
+    g.x0 = clamp_tile(floorf(fm(fs(g.x, g.rf), 0.0625f)), vw.tiles_x);
+    g.x1 = clamp_tile(floorf(fm(fa(fa(g.x, g.rf), 15.f), 0.0625f)), vw.tiles_x);
+    g.y0 = clamp_tile(floorf(fm(fs(g.y, g.rf), 0.0625f)), vw.tiles_y);
+    g.y1 = clamp_tile(floorf(fm(fa(fa(g.y, g.rf), 15.f), 0.0625f)), vw.tiles_y);
     const bool area_ok = (g.x1 > g.x0) && (g.y1 > g.y0);
     g.op = fm(gmask, opac);
     const bool op_ok = g.op >= (1.0f / 255.0f);
@@ -469,25 +468,21 @@ __device__ __forceinline__ uint32_t preprocess_entry(const ViewDesc &vw, const S
     return touched;
 }
 
-// One thread per scene Gaussian: its parameters are read once and projected
-// into every view of the call that shows its scene. ONE_VIEW: no scene has
-// more than one view, so the walk stops at the first (the parameters need not
-// stay live across views). Each block also adds its pairs and its entries with
-// a pair to the view's totals (view_pairs, view_visible), which the binning
-// cuts its chunks by: a warp reduction per view, then one atomic per block.
-template <int DG, int DL, int DS, int CM, bool ONE_VIEW>
-__global__ void __launch_bounds__(PRE_THREADS, ONE_VIEW ? 1 : CM == SG_COLOR_SH3 ? 2 : 3)
+// No scene of the call has more than one view: one thread per scene Gaussian.
+// Each block also adds its pairs and its entries with a pair to the view's
+// totals (view_pairs, view_visible), which the binning cuts its chunks by: a
+// warp reduction, then one atomic per block.
+template <int DG, int DL, int DS, int CM>
+__global__ void __launch_bounds__(PRE_THREADS)
 k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
-             uint2 *__restrict__ rect, uint32_t *__restrict__ dkey,
-             uint8_t *__restrict__ clamp, unsigned long long *__restrict__ view_pairs,
-             uint32_t *__restrict__ view_visible) {
+             uint2 *__restrict__ rect, uint32_t *__restrict__ dkey, uint8_t *__restrict__ clamp,
+             unsigned long long *__restrict__ view_pairs, uint32_t *__restrict__ view_visible) {
     chain_enter();
-    constexpr int NV = ONE_VIEW ? 1 : SG_MAX_VIEWS;
-    __shared__ uint32_t s_pairs[NV], s_vis[NV];
+    __shared__ uint32_t s_pairs, s_vis;
     const Batch &b = *bp;
     const int si = find_block_scene(b, blockIdx.x);
     const SceneDesc &sc = b.scene[si];
-    for (int v = threadIdx.x; v < NV; v += PRE_THREADS) s_pairs[v] = s_vis[v] = 0u;
+    if (threadIdx.x == 0) s_pairs = s_vis = 0u;
     __syncthreads();
     const int64_t gt = (int64_t)(blockIdx.x - sc.blk_off) * PRE_THREADS + threadIdx.x;
     const bool on = gt < sc.n;
@@ -499,7 +494,6 @@ k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__re
     load_colour_base<CM>(sc, g, cb);
     Geo3 g3;
     geo3_recipe(s0, s1, s2, q0, q1, q2, q3, g3);
-    int mine = 0;   // ONE_VIEW: the scene's view
     for (int v = 0; v < b.n_views; ++v) {
         const ViewDesc &vw = b.view[v];
         if (vw.scene != si) continue;
@@ -510,18 +504,104 @@ k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__re
         const uint32_t pairs = __reduce_add_sync(0xffffffffu, touched);
         const uint32_t vis = (uint32_t)__popc(__ballot_sync(0xffffffffu, touched != 0u));
         if ((threadIdx.x & 31) == 0 && vis) {
-            atomicAdd(&s_pairs[ONE_VIEW ? 0 : v], pairs);
-            atomicAdd(&s_vis[ONE_VIEW ? 0 : v], vis);
+            atomicAdd(&s_pairs, pairs);
+            atomicAdd(&s_vis, vis);
         }
-        mine = v;
-        if (ONE_VIEW) break;
+        __syncthreads();
+        if (threadIdx.x == 0 && s_vis) {
+            atomicAdd(view_pairs + v, (unsigned long long)s_pairs);
+            atomicAdd(view_visible + v, s_vis);
+        }
+        return;   // the scene's only view
+    }
+}
+
+// Scene of block `blk` of the several-view grids.
+__device__ __forceinline__ int find_run_scene(const Batch &b, uint32_t blk) {
+    int lo = 0, hi = b.n_scenes - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (b.scene[mid].run_off <= blk) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Appends the threads with `take` to the block's queue (in any order): item i
+// of the block's run of PRE_RUN Gaussians.
+__device__ __forceinline__ void queue_push(bool take, uint32_t i, uint16_t *queue, uint32_t *count) {
+    const uint32_t m = __ballot_sync(0xffffffffu, take);
+    uint32_t at = 0;
+    if ((threadIdx.x & 31) == 0 && m) at = atomicAdd(count, (uint32_t)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (take) queue[at + (uint32_t)__popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = (uint16_t)i;
+}
+
+// Scenes seen from several views: a block takes PRE_RUN Gaussians. Those whose
+// opacity alone culls them in every view (o' < 1/255: pruned or nearly so) only get
+// their empty entries; the others are queued, so that full warps project
+// them into the views. Parameters are read once for all views.
+template <int DG, int DL, int DS, int CM>
+__global__ void __launch_bounds__(PRE_THREADS, CM == SG_COLOR_SH3 ? 2 : 3)
+k_preprocess_views(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
+                   uint2 *__restrict__ rect, uint32_t *__restrict__ dkey, uint8_t *__restrict__ clamp,
+                   unsigned long long *__restrict__ view_pairs, uint32_t *__restrict__ view_visible) {
+    chain_enter();
+    __shared__ uint32_t s_pairs[SG_MAX_VIEWS], s_vis[SG_MAX_VIEWS], s_n;
+    __shared__ uint16_t s_queue[PRE_RUN];
+    const Batch &b = *bp;
+    const int si = find_run_scene(b, blockIdx.x);
+    const SceneDesc &sc = b.scene[si];
+    for (int v = threadIdx.x; v < SG_MAX_VIEWS; v += PRE_THREADS) s_pairs[v] = s_vis[v] = 0u;
+    if (threadIdx.x == 0) s_n = 0u;
+    __syncthreads();
+    const int64_t g0 = (int64_t)(blockIdx.x - sc.run_off) * PRE_RUN;
+    for (uint32_t i = threadIdx.x; i < PRE_RUN; i += PRE_THREADS) {
+        const int64_t g = g0 + i;
+        const bool on = g < sc.n;
+        const bool live = on && fm(__ldg(sc.gmask + g), ldp<DG>(sc.opac, g)) >= (1.0f / 255.0f);
+        if (on && !live) {
+            for (int v = 0; v < b.n_views; ++v) {
+                if (b.view[v].scene != si) continue;
+                const uint64_t e = b.view[v].ent_off + (uint64_t)g;
+                tiles_touched[e] = 0u;
+                rect[e] = make_uint2(0u, 0u);
+                dkey[e] = SORT_DROP_KEY;
+            }
+        }
+        queue_push(live, i, s_queue, &s_n);
     }
     __syncthreads();
-    for (int v = threadIdx.x; v < (ONE_VIEW ? 1 : b.n_views); v += PRE_THREADS)
+    const uint32_t n = s_n;
+    for (uint32_t q = threadIdx.x; (q & ~31u) < n; q += PRE_THREADS) {   // uniform across the warp
+        const bool on = q < n;
+        const int64_t g = g0 + s_queue[on ? q : n - 1];
+        float px, py, pz, s0, s1, s2, q0, q1, q2, q3, o;
+        load_geo<DG>(sc, g, px, py, pz, s0, s1, s2, q0, q1, q2, q3, o);
+        const float gm = __ldg(sc.gmask + g);
+        ColourBase cb;
+        load_colour_base<CM>(sc, g, cb);
+        Geo3 g3;
+        geo3_recipe(s0, s1, s2, q0, q1, q2, q3, g3);
+        for (int v = 0; v < b.n_views; ++v) {
+            const ViewDesc &vw = b.view[v];
+            if (vw.scene != si) continue;
+            uint32_t touched = 0u;
+            if (on)
+                touched = preprocess_entry<DL, DS, CM>(vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g,
+                                                       rec, tiles_touched, rect, dkey, clamp);
+            const uint32_t pairs = __reduce_add_sync(0xffffffffu, touched);
+            const uint32_t vis = (uint32_t)__popc(__ballot_sync(0xffffffffu, touched != 0u));
+            if ((threadIdx.x & 31) == 0 && vis) {
+                atomicAdd(&s_pairs[v], pairs);
+                atomicAdd(&s_vis[v], vis);
+            }
+        }
+    }
+    __syncthreads();
+    for (int v = threadIdx.x; v < b.n_views; v += PRE_THREADS)
         if (s_vis[v]) {
-            const int view = ONE_VIEW ? mine : v;
-            atomicAdd(view_pairs + view, (unsigned long long)s_pairs[v]);
-            atomicAdd(view_visible + view, s_vis[v]);
+            atomicAdd(view_pairs + v, (unsigned long long)s_pairs[v]);
+            atomicAdd(view_visible + v, s_vis[v]);
         }
 }
 
@@ -531,11 +611,11 @@ static cudaError_t launch_pre_t(const Batch &hb, const Batch *db, Rec *rec, uint
                                 uint32_t *vv, cudaStream_t s) {
     if (hb.scene_blocks == 0) return cudaSuccess;   // one block per 256 scene Gaussians
     if (hb.max_views_per_scene <= 1)
-        (void)launch_chain(k_preprocess<DG, DL, DS, CM, true>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db,
-                           rec, tt, rect, dkey, clamp, vp, vv);
+        (void)launch_chain(k_preprocess<DG, DL, DS, CM>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db, rec, tt,
+                           rect, dkey, clamp, vp, vv);
     else
-        (void)launch_chain(k_preprocess<DG, DL, DS, CM, false>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db,
-                           rec, tt, rect, dkey, clamp, vp, vv);
+        (void)launch_chain(k_preprocess_views<DG, DL, DS, CM>, dim3(hb.scene_runs), dim3(PRE_THREADS), s, db, rec, tt,
+                           rect, dkey, clamp, vp, vv);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -569,57 +649,122 @@ cudaError_t launch_preprocess(const Batch &hb, const Batch *db, Rec *rec, uint32
 // ---------------------------------------------------------------------------
 // K8 preprocess backward
 // ---------------------------------------------------------------------------
-// dg layout: planar [9][M] per entry: the blend adjoint's sums of dG dx, dG dy,
-// dG dx^2, dG dx dy, dG dy^2 (dG = dL/dalpha G), then dL/do', dL/dr, dL/dg, dL/db.
+// dg layout: [M][9] per entry: the blend
+// adjoint's sums of dP dx, dP dy, dP dx^2, dP dx dy, dP dy^2, dP, dL/dr, dL/dg, dL/db.
 // Resident blocks per SM requested for the preprocess adjoint (it is bound by
 // the latency of its parameter loads, so occupancy matters more than registers).
 #ifndef SG_PRE_BWD_MIN_BLOCKS
 #define SG_PRE_BWD_MIN_BLOCKS 3
 #endif
 
-template <int DG, int DL, int DS, int CM>
-__global__ void __launch_bounds__(PRE_THREADS, SG_PRE_BWD_MIN_BLOCKS)
-k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tiles_touched,
-                 const uint8_t *__restrict__ clamp, const float *__restrict__ dg, uint64_t M) {
-    chain_enter();
-    const Batch &b = *bp;
-    const int si = find_block_scene(b, blockIdx.x);
-    const SceneDesc &sc = b.scene[si];
-    const int64_t g = (int64_t)(blockIdx.x - sc.blk_off) * PRE_THREADS + threadIdx.x;
-    if (g >= sc.n) return;
+// Gradients of a Gaussian that no view of the call shows.
+template <int CM>
+__device__ __forceinline__ void zero_gradients(const SceneDesc &sc, int64_t g) {
+    const int64_t n = sc.n, L = sc.n_lobes;
+    const sg_grads &gr = sc.grads;
+    if (CM == SG_COLOR_SH3) {
+        if (gr.sh)
+            for (int k = 0; k < 48; ++k) gr.sh[(int64_t)k * n + g] = 0.f;
+    } else {
+        const int hi = min(__ldg(sc.lobe_off + g + 1), (int)L), lo = max(0, min(__ldg(sc.lobe_off + g), hi));
+        for (int k = lo; k < hi; ++k) {
+            if (gr.amp) { gr.amp[k] = 0.f; gr.amp[L + k] = 0.f; gr.amp[2 * L + k] = 0.f; }
+            if (gr.axis) { gr.axis[k] = 0.f; gr.axis[L + k] = 0.f; gr.axis[2 * L + k] = 0.f; }
+            if (gr.sharp) gr.sharp[k] = 0.f;
+            if (gr.lmask) gr.lmask[k] = 0.f;
+        }
+    }
+    if (gr.means) gr.means[g] = gr.means[n + g] = gr.means[2 * n + g] = 0.f;
+    if (gr.scales) gr.scales[g] = gr.scales[n + g] = gr.scales[2 * n + g] = 0.f;
+    if (gr.quats) gr.quats[g] = gr.quats[n + g] = gr.quats[2 * n + g] = gr.quats[3 * n + g] = 0.f;
+    if (gr.opac) gr.opac[g] = 0.f;
+    if (gr.gmask) gr.gmask[g] = 0.f;
+    if (gr.c0) gr.c0[g] = gr.c0[n + g] = gr.c0[2 * n + g] = 0.f;
+}
+
+// One lobe's share of a view's colour adjoint: adds its gradients (axis, amp,
+// sharp, lmask) to d and dL/dv to dv. (vx, vy, vz): unit view direction, gc:
+// upstream colour gradient.
+struct LobeGrad {
+    float ax[3], amp[3], s, m;
+};
+template <int DL, int DS>
+__device__ __forceinline__ void lobe_adjoint(const LobeChunk<DL, DS> &lc, int u, float vx, float vy, float vz,
+                                             const float gc[3], LobeGrad &d, float &dvx, float &dvy, float &dvz) {
+    const float ax = lc.ax[u], ay = lc.ay[u], az = lc.az[u];
+    const float na = sqrtf(ax * ax + ay * ay + az * az);
+    const float ia = 1.0f / na;
+    const float mx = ax * ia, my = ay * ia, mz = az * ia;
+    const float dot = mx * vx + my * vy + mz * vz;
+    const float sh = lc.sh[u];
+    const float ex = expf(sh * (dot - 1.0f));
+    const float m = lc.m[u];
+    const float ga = lc.a0[u] * gc[0] + lc.a1[u] * gc[1] + lc.a2[u] * gc[2];
+    const float de = m * ga;
+    const float dd = de * ex * sh;                                     // dL/d(mu_hat . v)
+    const float gmx = dd * vx, gmy = dd * vy, gmz = dd * vz;           // dL/dmu_hat
+    const float pr = mx * gmx + my * gmy + mz * gmz;
+    dvx += dd * mx; dvy += dd * my; dvz += dd * mz;
+    d.amp[0] += m * ex * gc[0]; d.amp[1] += m * ex * gc[1]; d.amp[2] += m * ex * gc[2];
+    d.ax[0] += (gmx - mx * pr) * ia; d.ax[1] += (gmy - my * pr) * ia; d.ax[2] += (gmz - mz * pr) * ia;
+    d.s += de * ex * (dot - 1.0f);
+    d.m += ex * ga;
+}
+
+__device__ __forceinline__ void write_lobe(const sg_grads &gr, int64_t L, int k, const LobeGrad &d) {
+    if (gr.amp) { gr.amp[k] = d.amp[0]; gr.amp[L + k] = d.amp[1]; gr.amp[2 * L + k] = d.amp[2]; }
+    if (gr.axis) { gr.axis[k] = d.ax[0]; gr.axis[L + k] = d.ax[1]; gr.axis[2 * L + k] = d.ax[2]; }
+    if (gr.sharp) gr.sharp[k] = d.s;
+    if (gr.lmask) gr.lmask[k] = d.m;
+}
+
+// Gaussian g of scene si: sums its views' adjoints and writes its gradients
+// (on false: a lane past the scene's end that only takes part in the warp's
+// barrier). ONE_VIEW: the call has one view, whose nine sums of this Gaussian
+// are on their way to dgs (shared memory); else they are read from dg. With
+// several views the lobes follow the views' geometry, two lobes at a time over
+// all views: their sums stay in registers and are written once.
+template <int DG, int DL, int DS, int CM, bool ONE_VIEW>
+__device__ __forceinline__ void adjoint_gaussian(const Batch &b, const SceneDesc &sc, int si, int64_t g, bool on,
+                                                 const uint32_t *__restrict__ tiles_touched,
+                                                 const uint8_t *__restrict__ clamp, const float *__restrict__ dg,
+                                                 const float *dgs) {
     const int64_t n = sc.n, L = sc.n_lobes;
 
     float px, py, pz, s0, s1, s2, q0, q1, q2, q3, o;
     load_geo<DG>(sc, g, px, py, pz, s0, s1, s2, q0, q1, q2, q3, o);
     const float gm = __ldg(sc.gmask + g);
     const bool sh_mode = CM == SG_COLOR_SH3;
-    const int hi = sh_mode ? 0 : min(__ldg(sc.lobe_off + g + 1), (int)L);
-    const int lo = sh_mode ? 0 : max(0, min(__ldg(sc.lobe_off + g), hi));
+    const int hi = sh_mode || !on ? 0 : min(__ldg(sc.lobe_off + g + 1), (int)L);
+    const int lo = sh_mode || !on ? 0 : max(0, min(__ldg(sc.lobe_off + g), hi));
 
     float d_mean[3] = {0.f, 0.f, 0.f}, d_scale[3] = {0.f, 0.f, 0.f}, d_q[4] = {0.f, 0.f, 0.f, 0.f};
     float d_opac = 0.f, d_gmask = 0.f, d_c0[3] = {0.f, 0.f, 0.f};
     bool first = true;   // first visible view writes lobe gradients, later views add
-    const bool multi_view = b.n_views > 1;
+    constexpr bool multi_view = !ONE_VIEW;
     Geo3 g3;
     geo3_recipe(s0, s1, s2, q0, q1, q2, q3, g3);
     float dS[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
 
-    // With several views, the views whose entry of this Gaussian reaches a tile
-    // are found first, 32 at a time, with independent loads (one memory round
-    // trip instead of one per view); the others need no gradient work.
+    // The views whose entry of this Gaussian reaches a tile, 32 views at a time,
+    // found with independent loads (one memory round trip instead of one per
+    // view); with one view, the view's tile test follows the eager loads below.
+    auto live_views = [&](int v0) {
+        uint32_t m = 0u;
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) {
+            const int v = v0 + i;
+            if (v < b.n_views && b.view[v].scene == si && tiles_touched[b.view[v].ent_off + (uint64_t)g] != 0u)
+                m |= 1u << i;
+        }
+        return m;
+    };
+    uint32_t live0 = 0u;   // of the first 32 views
     for (int v0 = 0; v0 < b.n_views; v0 += 32) {
-        // one view: view 0 when it sees this Gaussian's scene (its tile test
-        // follows the eager loads below)
         uint32_t live = b.view[0].scene == si ? 1u : 0u;
         if (multi_view) {
-            live = 0u;
-#pragma unroll 8
-            for (int i = 0; i < 32; ++i) {
-                const int v = v0 + i;
-                if (v < b.n_views && b.view[v].scene == si &&
-                    tiles_touched[b.view[v].ent_off + (uint64_t)g] != 0u)
-                    live |= 1u << i;
-            }
+            live = live_views(v0);
+            if (v0 == 0) live0 = live;
         }
         while (live) {
             const int v = v0 + __ffs(live) - 1;
@@ -631,10 +776,14 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
             const uint32_t tte = multi_view ? 1u : tiles_touched[e];
             // moments of dP = dL/dpower = dL/dalpha o' G over the entry's pixels
             // (dx, dy = pixel - centre); gop = sum dP = o' dL/do'.
-            const float mdx = dg[e], mdy = dg[M + e], mdxx = dg[2 * M + e], mdxy = dg[3 * M + e],
-                        mdyy = dg[4 * M + e], gop = dg[5 * M + e];
-            const float grgb[3] = {dg[6 * M + e], dg[7 * M + e], dg[8 * M + e]};
             const uint32_t cl = clamp[e];
+            if (ONE_VIEW) {   // uniform: the staged sums are in
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+            }
+            const float *m9 = ONE_VIEW ? dgs : dg + 9 * e;
+            const float mdx = m9[0], mdy = m9[1], mdxx = m9[2], mdxy = m9[3], mdyy = m9[4], gop = m9[5];
+            const float grgb[3] = {m9[6], m9[7], m9[8]};
             if (tte == 0u) continue;
             // the forward's clamp max(c, 0) per channel, read back from its bits
             const float gc[3] = {(cl & 1u) ? 0.f : grgb[0], (cl & 2u) ? 0.f : grgb[1], (cl & 4u) ? 0.f : grgb[2]};
@@ -659,7 +808,7 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
                 }
                 sh3_grad_acc(vx, vy, vz, w, dvx, dvy, dvz);
                 float *gsh = sc.grads.sh;
-                if (gsh) {
+                if (gsh && on) {
 #pragma unroll
                     for (int ch = 0; ch < 3; ++ch)
 #pragma unroll
@@ -674,45 +823,16 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
                 d_c0[1] += gc[1];
                 d_c0[2] += gc[2];
             }
-            for (int k0 = lo; k0 < hi; k0 += LOBE_CHUNK) {
-                LobeChunk<DL, DS> lc;
-                lc.load(sc, k0, hi);
+            if (ONE_VIEW) {
+                for (int k0 = lo; k0 < hi; k0 += LOBE_CHUNK) {
+                    LobeChunk<DL, DS> lc;
+                    lc.load(sc, k0, hi);
 #pragma unroll
-                for (int u = 0; u < LOBE_CHUNK; ++u) {
-                    const int k = k0 + u;
-                    if (k >= hi) break;
-                    const float ax = lc.ax[u], ay = lc.ay[u], az = lc.az[u];
-                    const float na = sqrtf(ax * ax + ay * ay + az * az);
-                    const float ia = 1.0f / na;
-                    const float mx = ax * ia, my = ay * ia, mz = az * ia;
-                    const float dot = mx * vx + my * vy + mz * vz;
-                    const float sh = lc.sh[u];
-                    const float ex = expf(sh * (dot - 1.0f));
-                    const float m = lc.m[u];
-                    const float a0 = lc.a0[u], a1 = lc.a1[u], a2 = lc.a2[u];
-                    const float ga = a0 * gc[0] + a1 * gc[1] + a2 * gc[2];
-                    const float de = m * ga;
-                    const float dd = de * ex * sh;                 // dL/d(mu_hat . v)
-                    const float gmx = dd * vx, gmy = dd * vy, gmz = dd * vz;   // dL/dmu_hat
-                    const float pr = mx * gmx + my * gmy + mz * gmz;
-                    dvx += dd * mx; dvy += dd * my; dvz += dd * mz;
-                    float ga_out[3] = {m * ex * gc[0], m * ex * gc[1], m * ex * gc[2]};
-                    float gax[3] = {(gmx - mx * pr) * ia, (gmy - my * pr) * ia, (gmz - mz * pr) * ia};
-                    const float gs = de * ex * (dot - 1.0f);
-                    const float gml = ex * ga;
-                    const sg_grads &gr = sc.grads;
-                    if (first) {
-                        if (gr.amp) { gr.amp[k] = ga_out[0]; gr.amp[L + k] = ga_out[1]; gr.amp[2 * L + k] = ga_out[2]; }
-                        if (gr.axis) { gr.axis[k] = gax[0]; gr.axis[L + k] = gax[1]; gr.axis[2 * L + k] = gax[2]; }
-                        if (gr.sharp) gr.sharp[k] = gs;
-                        if (gr.lmask) gr.lmask[k] = gml;
-                    } else {
-                        if (gr.amp) {
-                            gr.amp[k] += ga_out[0]; gr.amp[L + k] += ga_out[1]; gr.amp[2 * L + k] += ga_out[2];
-                        }
-                        if (gr.axis) { gr.axis[k] += gax[0]; gr.axis[L + k] += gax[1]; gr.axis[2 * L + k] += gax[2]; }
-                        if (gr.sharp) gr.sharp[k] += gs;
-                        if (gr.lmask) gr.lmask[k] += gml;
+                    for (int u = 0; u < LOBE_CHUNK; ++u) {
+                        if (k0 + u >= hi) break;
+                        LobeGrad d{};
+                        lobe_adjoint(lc, u, vx, vy, vz, gc, d, dvx, dvy, dvz);
+                        write_lobe(sc.grads, L, k0 + u, d);
                     }
                 }
             }
@@ -790,8 +910,7 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
             const float itz2 = itz * itz;
             dtz += -(vw.fx * dJ00 + vw.fy * dJ11) * itz2;
             {
-                const float limx = 1.3f * (0.5f * (float)vw.W / vw.fx);
-                const float limy = 1.3f * (0.5f * (float)vw.H / vw.fy);
+                const float limx = vw.limx, limy = vw.limy;
                 const bool inx = G.ux >= -limx && G.ux <= limx;
                 const bool iny = G.uy >= -limy && G.uy <= limy;
                 // J02 = -fx ccx / tz^2, ccx = clamp(tx/tz) tz
@@ -808,6 +927,39 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
         }
     }
 
+    if (!on) return;
+    if (!ONE_VIEW && !first) {
+        for (int k0 = lo; k0 < hi; k0 += LOBE_CHUNK) {
+            LobeChunk<DL, DS> lc;
+            lc.load(sc, k0, hi);
+            LobeGrad d[LOBE_CHUNK] = {};
+            for (int v0 = 0; v0 < b.n_views; v0 += 32) {
+                uint32_t live = v0 == 0 ? live0 : live_views(v0);
+                while (live) {
+                    const ViewDesc &vw = b.view[v0 + __ffs(live) - 1];
+                    live &= live - 1u;
+                    const uint64_t e = vw.ent_off + (uint64_t)g;
+                    const float *m9 = dg + 9 * e;
+                    const uint32_t cl = clamp[e];
+                    const float gc[3] = {(cl & 1u) ? 0.f : m9[6], (cl & 2u) ? 0.f : m9[7], (cl & 4u) ? 0.f : m9[8]};
+                    float vx = px - vw.campos[0], vy = py - vw.campos[1], vz = pz - vw.campos[2];
+                    const float idn = 1.0f / sqrtf(vx * vx + vy * vy + vz * vz);
+                    vx *= idn; vy *= idn; vz *= idn;
+                    float dvx = 0.f, dvy = 0.f, dvz = 0.f;
+#pragma unroll
+                    for (int u = 0; u < LOBE_CHUNK; ++u)   // the last chunk may be short
+                        if (k0 + u < hi) lobe_adjoint(lc, u, vx, vy, vz, gc, d[u], dvx, dvy, dvz);
+                    const float pr = vx * dvx + vy * dvy + vz * dvz;
+                    d_mean[0] += (dvx - vx * pr) * idn;
+                    d_mean[1] += (dvy - vy * pr) * idn;
+                    d_mean[2] += (dvz - vz * pr) * idn;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < LOBE_CHUNK; ++u)
+                if (k0 + u < hi) write_lobe(sc.grads, L, k0 + u, d[u]);
+        }
+    }
     const sg_grads &gr = sc.grads;
     // Sigma_3D = M M^T, M = R diag(s): scale and (unit, then raw) quaternion
     if (!first) {
@@ -840,16 +992,9 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
         d_q[2] = (gyq - y * pr) * g3.invq;
         d_q[3] = (gzq - z * pr) * g3.invq;
     }
-    if (first && sh_mode && gr.sh) {   // not visible in any view: SH gradients are zero
-        for (int k = 0; k < 48; ++k) gr.sh[(int64_t)k * n + g] = 0.f;
-    }
-    if (first) {   // not visible in any view: lobe gradients are zero
-        for (int k = lo; k < hi; ++k) {
-            if (gr.amp) { gr.amp[k] = 0.f; gr.amp[L + k] = 0.f; gr.amp[2 * L + k] = 0.f; }
-            if (gr.axis) { gr.axis[k] = 0.f; gr.axis[L + k] = 0.f; gr.axis[2 * L + k] = 0.f; }
-            if (gr.sharp) gr.sharp[k] = 0.f;
-            if (gr.lmask) gr.lmask[k] = 0.f;
-        }
+    if (first) {   // not visible in any view
+        zero_gradients<CM>(sc, g);
+        return;
     }
     if (gr.means) { gr.means[g] = d_mean[0]; gr.means[n + g] = d_mean[1]; gr.means[2 * n + g] = d_mean[2]; }
     if (gr.scales) { gr.scales[g] = d_scale[0]; gr.scales[n + g] = d_scale[1]; gr.scales[2 * n + g] = d_scale[2]; }
@@ -861,11 +1006,83 @@ k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tile
     if (gr.c0) { gr.c0[g] = d_c0[0]; gr.c0[n + g] = d_c0[1]; gr.c0[2 * n + g] = d_c0[2]; }
 }
 
+// One view in the call: one thread per scene Gaussian. A warp's sums, a
+// contiguous piece of dg, are copied to its piece of shared memory
+// asynchronously while its parameters load (a stride of nine words has no bank
+// conflicts).
+template <int DG, int DL, int DS, int CM>
+__global__ void __launch_bounds__(PRE_THREADS, SG_PRE_BWD_MIN_BLOCKS)
+k_preprocess_bwd(const Batch *__restrict__ bp, const uint32_t *__restrict__ tiles_touched,
+                 const uint8_t *__restrict__ clamp, const float *__restrict__ dg, uint64_t M) {
+    chain_enter();
+    __shared__ float s_dg[9 * PRE_THREADS];
+    const Batch &b = *bp;
+    const int si = find_block_scene(b, blockIdx.x);
+    const SceneDesc &sc = b.scene[si];
+    const int64_t g = (int64_t)(blockIdx.x - sc.blk_off) * PRE_THREADS + threadIdx.x;
+    const uint32_t lane = threadIdx.x & 31;
+    if (g - lane >= sc.n) return;   // uniform across the warp
+    float *sw = s_dg + 9 * (threadIdx.x - lane);
+    if (b.view[0].scene == si) {   // uniform
+        const uint64_t w0 = 9 * (b.view[0].ent_off + (uint64_t)(g - lane));
+#pragma unroll
+        for (uint32_t k = 0; k < 9; ++k) {
+            const uint32_t i = 32u * k + lane;
+            if (w0 + i < 9 * M)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(sw + i)),
+                             "l"(dg + w0 + i)
+                             : "memory");
+        }
+    }
+    const int64_t last = sc.n - 1;
+    adjoint_gaussian<DG, DL, DS, CM, true>(b, sc, si, g < sc.n ? g : last, g < sc.n, tiles_touched, clamp, dg,
+                                           sw + 9 * (g < sc.n ? lane : (uint32_t)(last - (g - lane))));
+}
+
+// Several views: a block takes PRE_RUN Gaussians. Those with no tile in any view
+// of their scene get zero gradients; the others are queued, so that full warps
+// run their adjoints.
+template <int DG, int DL, int DS, int CM>
+__global__ void __launch_bounds__(PRE_THREADS, SG_PRE_BWD_MIN_BLOCKS)
+k_preprocess_bwd_views(const Batch *__restrict__ bp, const uint32_t *__restrict__ tiles_touched,
+                       const uint8_t *__restrict__ clamp, const float *__restrict__ dg, uint64_t M) {
+    chain_enter();
+    __shared__ uint32_t s_n;
+    __shared__ uint16_t s_queue[PRE_RUN];
+    const Batch &b = *bp;
+    const int si = find_run_scene(b, blockIdx.x);
+    const SceneDesc &sc = b.scene[si];
+    if (threadIdx.x == 0) s_n = 0u;
+    __syncthreads();
+    const int64_t g0 = (int64_t)(blockIdx.x - sc.run_off) * PRE_RUN;
+    for (uint32_t i = threadIdx.x; i < PRE_RUN; i += PRE_THREADS) {
+        const int64_t g = g0 + i;
+        const bool on = g < sc.n;
+        uint32_t any = 0u;
+        if (on) {
+#pragma unroll 8
+            for (int v = 0; v < b.n_views; ++v)
+                if (b.view[v].scene == si) any |= tiles_touched[b.view[v].ent_off + (uint64_t)g];
+        }
+        if (on && any == 0u) zero_gradients<CM>(sc, g);
+        queue_push(on && any != 0u, i, s_queue, &s_n);
+    }
+    __syncthreads();
+    const uint32_t n = s_n;
+    for (uint32_t q = threadIdx.x; q < n; q += PRE_THREADS)
+        adjoint_gaussian<DG, DL, DS, CM, false>(b, sc, si, g0 + s_queue[q], true, tiles_touched, clamp, dg, nullptr);
+}
+
 template <int DG, int DL, int DS, int CM = SG_COLOR_SG>
 static cudaError_t launch_bwd_t(const Batch &hb, const Batch *db, const uint32_t *tt, const uint8_t *clamp,
                                 const float *dg, uint64_t M, cudaStream_t s) {
     if (hb.scene_blocks == 0) return cudaSuccess;
-    (void)launch_chain(k_preprocess_bwd<DG, DL, DS, CM>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db, tt, clamp, dg, M);
+    if (hb.n_views == 1)
+        (void)launch_chain(k_preprocess_bwd<DG, DL, DS, CM>, dim3(hb.scene_blocks), dim3(PRE_THREADS), s, db, tt, clamp,
+                           dg, M);
+    else
+        (void)launch_chain(k_preprocess_bwd_views<DG, DL, DS, CM>, dim3(hb.scene_runs), dim3(PRE_THREADS), s, db, tt,
+                           clamp, dg, M);
     count_launches(1);
     return cudaGetLastError();
 }

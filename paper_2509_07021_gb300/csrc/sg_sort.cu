@@ -24,8 +24,9 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
 // ---------------------------------------------------------------------------
 // stable LSD radix sort, 8-bit digits, RS_TILE keys per block, one sweep per pass
 // ---------------------------------------------------------------------------
-// One kernel histograms every digit position at once (and clears the look-back
-// flags of every pass; for the radix tile sort the duplicate does both). Each pass is then a single kernel: blocks take key
+// One kernel histograms every digit position at once and clears the look-back
+// flags of every pass (for the radix tile sort the duplicate does both). Each
+// pass is then a single kernel: blocks take key
 // tiles in order from an atomic counter, rank their keys stably (warp
 // match_any + per-warp digit counters), scan the pass's digit histogram for
 // the digit bases, publish their digit counts, and get their offsets among
