@@ -81,3 +81,20 @@ def test_opacity_step_ties_across_blocks(kappa):
     torch.cuda.synchronize()
     np.testing.assert_array_equal(ot_d.cpu().numpy(), ot_ref)
     np.testing.assert_array_equal(lam_d.cpu().numpy(), lam_ref)
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+@pytest.mark.parametrize("n,kappa", [(5000, 1234), (2049, 2048)])
+def test_opacity_step_on_unaligned_vectors(n, kappa, offset):
+    """Vectors that start off a 16-byte boundary take the final pass's scalar path."""
+    rng = np.random.default_rng(n + offset)
+    o, lam = rng.random(n).astype(np.float32), rng.normal(0, 0.2, n).astype(np.float32)
+    ot_ref, lam_ref, _ = admm.opacity_step(o, lam, kappa, None)
+    buf = torch.zeros(3, n + offset, device="cuda")
+    x, lam_d, ot = (buf[i, offset:] for i in range(3))
+    x.copy_(_t(o))
+    lam_d.copy_(_t(lam))
+    sgsplat.sg_admm_opacity_step(x, lam_d, ot, kappa)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(ot.cpu().numpy(), ot_ref)
+    np.testing.assert_array_equal(lam_d.cpu().numpy(), lam_ref)

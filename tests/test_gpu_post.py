@@ -44,3 +44,20 @@ def test_postprocessed_scene_renders():
     out = render.render_forward(ds, [synth.make_camera(64, 64, 80.0)])
     torch.cuda.synchronize()
     assert torch.isfinite(out.img).all() and out.sizes["n_pairs"] > 0
+
+
+@pytest.mark.parametrize("n,lobes", [(700, 4), (513, 7), (256, 2)])
+def test_many_lobes_per_block(n, lobes):
+    """A block's lobes fill several of the apply's shared-memory tiles, with kept
+    and removed ones on both sides of each edge."""
+    rng = np.random.default_rng(n)
+    scene = synth.make_scene(rng, n, lobes=lobes, masks="uniform")
+    scene.sharp[::2] = rng.uniform(0.0, 2.0, scene.sharp[::2].size).astype(np.float32)
+    out = sgsplat.sg_postprocess(DeviceScene.from_host(scene), 0.1, 1.0)
+    torch.cuda.synchronize()
+    gid, lid, off, c0 = post.postprocess(scene, 0.1, 1.0)
+    np.testing.assert_array_equal(out.lobe_off.cpu().numpy(), off)
+    for k in ("axis", "amp"):
+        np.testing.assert_array_equal(getattr(out, k).cpu().numpy(), getattr(scene, k)[:, lid])
+    np.testing.assert_array_equal(out.sharp.cpu().numpy(), scene.sharp[lid])
+    np.testing.assert_allclose(out.c0.cpu().numpy(), c0, rtol=2e-6, atol=2e-6)
