@@ -488,10 +488,24 @@ __device__ __forceinline__ void warp_sum9_atomic(const float v[9], float *dg9) {
     if ((lane & 3) == 0 || lane == 1) atomicAdd(dg9 + (lane == 1 ? 8 : lane >> 2), lane == 1 ? d : c);
 }
 
-// Adds one pixel's share of one blended pair to v (in dg order) and steps the
-// pixel's T and Sg back over the pair.
-__device__ __forceinline__ void bwd_adjoint(const PairEval &p, float dy, const float4 &r, float bl,
-                                            float &T, float &Sg, float g0, float g1, float g2, float v[9]) {
+// A thread's sums over its pixels for one entry. Its pixels lie in NC columns
+// (slot j in column j % NC), so dx takes only NC values: the moments in dx are formed
+// once per entry from the columns' sums of dP and dP dy. The kernel is bound by
+// instruction issue and nearly every evaluated slot has a blended lane, so the four
+// operations fewer per blended pixel count: 650 -> 614 us at 1M Gaussians,
+// 1920x1080; 9.67 -> 9.17 ms at 6M in 16 views.
+template <int NC>
+struct AdjSums {
+    float a[NC], b[NC], c;   // per column: sum dP, sum dP dy; all: sum dP dy^2
+    float r[3];              // sum w dL/drgb
+};
+
+// Adds one pixel's share of one blended pair (column h) and steps the pixel's
+// T and Sg back over the pair. dy2 = dy^2.
+template <int NC>
+__device__ __forceinline__ void bwd_adjoint(const PairEval &p, float dy, float dy2, const float4 &r, float bl,
+                                            float &T, float &Sg, float g0, float g1, float g2, int h,
+                                            AdjSums<NC> &v) {
     const float oma = __fsub_rn(1.f, p.alpha);
     const float ro = rcp_approx(oma);
     const float Ti = T * ro;
@@ -500,19 +514,15 @@ __device__ __forceinline__ void bwd_adjoint(const PairEval &p, float dy, const f
     const float dal = Ti * cg - Sg * ro;
     Sg = fmaf(cg, w, Sg);
     T = Ti;
-    v[6] = fmaf(w, g0, v[6]);
-    v[7] = fmaf(w, g1, v[7]);
-    v[8] = fmaf(w, g2, v[8]);
+    v.r[0] = fmaf(w, g0, v.r[0]);
+    v.r[1] = fmaf(w, g1, v.r[1]);
+    v.r[2] = fmaf(w, g2, v.r[2]);
     // dP = dL/dpower = dL/dalpha o' G, none where the 0.99 clamp is active
     // (dL/do' = dP / o': the division is applied once per Gaussian)
     const float dP = p.ag > ALPHA_MAX ? 0.f : dal * p.ag;
-    v[5] += dP;
-    const float hx = dP * p.dx, hy = dP * dy;
-    v[0] += hx;                          // sum dP dx
-    v[1] += hy;                          // sum dP dy
-    v[2] = fmaf(hx, p.dx, v[2]);         // sum dP dx^2
-    v[3] = fmaf(hx, dy, v[3]);           // sum dP dx dy
-    v[4] = fmaf(hy, dy, v[4]);           // sum dP dy^2
+    v.a[h] += dP;
+    v.b[h] = fmaf(dP, dy, v.b[h]);
+    v.c = fmaf(dP, dy2, v.c);
 }
 
 // Per pixel the walk runs back from the pixel's last blended pair, recovering
@@ -619,9 +629,7 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
             if ((msk & ((1u << P) - 1u)) == 0u) continue;   // warp-uniform
             const float4 q = sm.q[k], r = sm.r[k];
             const float bl = __uint_as_float(cm.x);
-            float v[9];
-#pragma unroll
-            for (int i = 0; i < 9; ++i) v[i] = 0.f;
+            AdjSums<row_slots<P>()> v{};
             bool any = false;
             constexpr int RS = row_slots<P>();
 #pragma unroll
@@ -635,6 +643,7 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                 slot_pixel<P>(j0, cx, cy);
                 RowEval row;
                 eval_row((float)(ty * TILE + cy), q, r, row);
+                const float dy2 = row.dy * row.dy;
                 // both pixels of the row first, with no branch between them
                 PairEval pe[RS];
                 bool ok[RS];
@@ -642,7 +651,8 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                 for (int hh = 0; hh < RS; ++hh) {
                     slot_pixel<P>(j0 + hh, cx, cy);
                     eval_pixel((float)(tx * TILE + cx), q, row, pe[hh]);
-                    const bool live = ((bits >> hh) & 1u) && pos < __float_as_int(pg[hh].w);
+                    // (where the mask's bit is clear the pixels fail one of the two tests)
+                    const bool live = pos < __float_as_int(pg[hh].w);
                     if (COUNT) ne += live ? 1u : 0u;
                     ok[hh] = live && pair_kept(pe[hh]);
                 }
@@ -651,12 +661,26 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                     const int j = j0 + hh;
                     if (!ok[hh]) continue;
                     any = true;
-                    bwd_adjoint(pe[hh], row.dy, r, bl, T[j], Sg[j], pg[hh].x, pg[hh].y, pg[hh].z, v);
+                    bwd_adjoint(pe[hh], row.dy, dy2, r, bl, T[j], Sg[j], pg[hh].x, pg[hh].y, pg[hh].z, hh, v);
                 }
             }
             // the moments are linear in dP: the conic factors and 1/o' are applied
             // once per entry by the preprocess adjoint, after the sum over tiles
-            if (__any_sync(0xffffffffu, any)) warp_sum9_atomic(v, dg + 9 * (uint64_t)sm.id[k]);
+            if (__any_sync(0xffffffffu, any)) {
+                float m[9] = {0.f, 0.f, 0.f, 0.f, v.c, 0.f, v.r[0], v.r[1], v.r[2]};   // in dg order
+#pragma unroll
+                for (int h = 0; h < RS; ++h) {
+                    int cx, cy;
+                    slot_pixel<P>(h, cx, cy);
+                    const float dx = __fsub_rn((float)(tx * TILE + cx), q.x);
+                    m[0] = fmaf(v.a[h], dx, m[0]);
+                    m[1] += v.b[h];
+                    m[2] = fmaf(v.a[h] * dx, dx, m[2]);
+                    m[3] = fmaf(v.b[h], dx, m[3]);
+                    m[5] += v.a[h];
+                }
+                warp_sum9_atomic(m, dg + 9 * (uint64_t)sm.id[k]);
+            }
         }
     }
 }
