@@ -440,7 +440,7 @@ struct BinArgs {
     uint64_t *counters;
     BinTab *tab;
     uint32_t *poff;                  // scratch, M words: first pair of each entry of the order
-    uint64_t *flags;                 // zeroed, one word per BIN_BLOCK entries: look-back
+    uint64_t *flags;                 // zeroed, a word per 256 entries (at most that many used): look-back
     uint16_t *pkey;                  // depth-ordered pairs: tile inside the view
     uint32_t *pval;                  //   and entry
     uint32_t *matrix;                // max_chunks x row words
@@ -451,7 +451,7 @@ struct BinArgs {
     uint32_t *okeys;                 // nullable: their global tile ids
     uint64_t *mirror;                // nullable host words: [0] pairs, [1] status
 };
-constexpr int BIN_ITEMS = 8, BIN_BLOCK = 256 * BIN_ITEMS;   // entries per thread and block of the chunk cutter
+constexpr int BIN_CUT_THREADS = 1024, BIN_ITEMS = 8;   // the chunk cutter's most threads, entries per thread
 cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s);   // chunks and their pairs
 cudaError_t launch_bin_place(const BinArgs &a, cudaStream_t s);   // scan and placement
 

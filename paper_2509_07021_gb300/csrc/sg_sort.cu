@@ -119,13 +119,14 @@ __global__ void __launch_bounds__(RS_THREADS) k_os_hist(const uint32_t *__restri
     }
 }
 
-// three resident blocks per SM (80 registers a thread)
+// three resident blocks per SM (80 registers a thread); GROUPED: see the look-back
+template <bool GROUPED>
 __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const uint64_t *__restrict__ n_dev, uint64_t max_n, int pass, int shift,
     uint32_t mask, bool drop, uint32_t *__restrict__ flags, SortAux *aux, uint2 *__restrict__ ranges,
     uint64_t n_ranges, uint32_t spin_limit, const uint64_t *__restrict__ skip_status,
-    const Batch *__restrict__ view_of) {
+    const Batch *__restrict__ view_of, uint32_t *__restrict__ groups) {
     chain_enter();
     constexpr int NW = RS_THREADS / 32;
     __shared__ uint32_t s_ent[SG_MAX_VIEWS];   // view pass: the views' first entries
@@ -203,37 +204,72 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
     // publish this tile's count, then look back for the exclusive prefix
     uint32_t *my = flags + (uint64_t)t * RS_RADIX + d;
     st_relaxed(my, LB_AGG | run);
-    // Look back LB_WINDOW predecessors per step (independent loads in flight):
-    // add counts until the nearest tile that carries its inclusive prefix;
-    // a tile not yet published stops the step and is re-read.
     uint32_t excl = 0u;
     uint32_t spins = 0;
-    for (int64_t p = (int64_t)t - 1; p >= 0;) {
-        uint32_t fv[LB_WINDOW];
+    if (GROUPED) {
+        // A short sort: its tiles all start together, so none finds an inclusive
+        // prefix near by and each would add up every count before its own, 16 a step.
+        // Instead each group of 16 tiles adds its counts up in one word per digit
+        // (5 bits of tiles, 27 of keys), and a tile adds the words of the groups before
+        // its own and the counts of its group: two steps up to 256 tiles (549k of
+        // 1M keys: 17 -> 12 us a pass).
+        const uint32_t g = t / LB_WINDOW;
+        atomicAdd(groups + (uint64_t)g * RS_RADIX + d, (1u << 27) + run);
+        for (uint32_t q0 = 0; q0 <= g; q0 += LB_WINDOW) {   // windows of groups; the last step: the tile's own group
+            const bool own = q0 + LB_WINDOW > g;
+            for (int part = 0; part < (own ? 2 : 1); ++part) {
+                const uint32_t first = part ? g * LB_WINDOW : q0, last = part ? t : min(g, q0 + LB_WINDOW);
+                const uint32_t *src = part ? flags : groups;
+                for (;;) {
+                    uint32_t fv[LB_WINDOW], sum = 0u;
 #pragma unroll
-        for (int i = 0; i < LB_WINDOW; ++i)
-            fv[i] = (p - i >= 0) ? ld_relaxed(flags + (uint64_t)(p - i) * RS_RADIX + d) : LB_INC;
-        int used = 0;
-        bool found = false, stalled = false;
+                    for (uint32_t i = 0; i < LB_WINDOW; ++i)
+                        fv[i] = first + i < last ? ld_relaxed(src + (uint64_t)(first + i) * RS_RADIX + d) : 0u;
+                    bool ready = true;
 #pragma unroll
-        for (int i = 0; i < LB_WINDOW; ++i) {
-            if (found || stalled) continue;
-            if ((fv[i] & ~LB_VAL) == 0u) { stalled = true; continue; }
-            excl += fv[i] & LB_VAL;
-            ++used;
-            if (fv[i] & LB_INC) found = true;
-        }
-        if (found) break;
-        p -= used;
-        if (stalled) {
-            if (++spins >= spin_limit) {
-                atomicExch(&aux->status, (uint32_t)SG_ERR_TIMEOUT);
-                break;
+                    for (uint32_t i = 0; i < LB_WINDOW; ++i) {
+                        if (first + i >= last) continue;
+                        ready = ready && (part ? (fv[i] & ~LB_VAL) != 0u : (fv[i] >> 27) == (uint32_t)LB_WINDOW);
+                        sum += part ? fv[i] & LB_VAL : fv[i] & ((1u << 27) - 1u);
+                    }
+                    if (!ready && ++spins < spin_limit) {
+                        __nanosleep(32);
+                        continue;
+                    }
+                    if (!ready) atomicExch(&aux->status, (uint32_t)SG_ERR_TIMEOUT);
+                    excl += sum;
+                    break;
+                }
             }
-            __nanosleep(32);
         }
+    } else {
+        for (int64_t p = (int64_t)t - 1; p >= 0;) {
+            uint32_t fv[LB_WINDOW];
+#pragma unroll
+            for (int i = 0; i < LB_WINDOW; ++i)
+                fv[i] = (p - i >= 0) ? ld_relaxed(flags + (uint64_t)(p - i) * RS_RADIX + d) : LB_INC;
+            int used = 0;
+            bool found = false, stalled = false;
+#pragma unroll
+            for (int i = 0; i < LB_WINDOW; ++i) {
+                if (found || stalled) continue;
+                if ((fv[i] & ~LB_VAL) == 0u) { stalled = true; continue; }
+                excl += fv[i] & LB_VAL;
+                ++used;
+                if (fv[i] & LB_INC) found = true;
+            }
+            if (found) break;
+            p -= used;
+            if (stalled) {
+                if (++spins >= spin_limit) {
+                    atomicExch(&aux->status, (uint32_t)SG_ERR_TIMEOUT);
+                    break;
+                }
+                __nanosleep(32);
+            }
+        }
+        st_relaxed(my, LB_INC | ((excl + run) & LB_VAL));
     }
-    st_relaxed(my, LB_INC | ((excl + run) & LB_VAL));
     uint32_t tot, all;
     const uint32_t ds = block_exclusive<uint32_t>(run, tot, shs);
     // global start of digit d in this pass: keys of smaller digits (all tiles) + earlier tiles
@@ -276,7 +312,10 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
 
 int radix_passes(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
 
-uint64_t sort_flag_words(uint64_t max_n, int passes) { return div_up(max_n, RS_TILE) * RS_RADIX * (uint64_t)passes; }
+uint64_t sort_flag_words(uint64_t max_n, int passes) {
+    const uint64_t tiles = div_up(max_n, RS_TILE);   // a word per tile and digit, and per group of tiles
+    return (tiles + div_up(tiles, LB_WINDOW)) * RS_RADIX * (uint64_t)passes;
+}
 
 // Buckets by list length on a log scale with 8 buckets per octave (exponent and
 // the 3 bits below the leading one), longest bucket first; inside a bucket the
@@ -325,23 +364,141 @@ __global__ void __launch_bounds__(256) k_os_finish(const SortAux *aux, uint64_t 
     if (h[threadIdx.x]) atomicAdd(&bucket_counts[threadIdx.x], h[threadIdx.x]);
 }
 
+// Opts a kernel into `bytes` of dynamic shared memory on the current device
+// (beside a few KB of static; 48 KB in all need no opting in).
+template <typename K>
+static cudaError_t allow_smem(K kernel, size_t bytes) {
+    if (bytes <= 32 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// The whole depth sort of at most 1024 ITEMS keys in one block: the same stable
+// digit passes with the keys in registers between them and shared memory for the
+// scatter, no look-back and one launch instead of five or six, which is what bounds the
+// short sorts (1000 keys: 38 -> 14 us). Warp w holds the positions
+// [32 ITEMS w, 32 ITEMS (w + 1)).
+constexpr uint32_t DS_MAX = 8192;
+template <int ITEMS>
+__global__ void __launch_bounds__(1024) k_depth_small(const uint32_t *__restrict__ keys, uint32_t M,
+                                                      uint32_t *__restrict__ vout, SortAux *aux,
+                                                      const Batch *__restrict__ b, int passes) {
+    chain_enter();
+    extern __shared__ uint32_t ds_smem[];
+    uint32_t *sk = ds_smem, *sv = sk + 1024 * ITEMS, *cnt = sv + 1024 * ITEMS;   // cnt[32][RS_RADIX]
+    __shared__ uint32_t dstart[RS_RADIX], shs[33], s_ent[SG_MAX_VIEWS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t p0 = (uint32_t)(warp * 32 * ITEMS + lane);
+    if (passes > VIEW_PASS && (int)threadIdx.x < b->n_views) s_ent[threadIdx.x] = (uint32_t)b->view[threadIdx.x].ent_off;
+    uint32_t k[ITEMS], v[ITEMS], r[ITEMS], meta[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        v[i] = p0 + 32u * i;
+        k[i] = v[i] < M ? keys[v[i]] : SORT_DROP_KEY;
+    }
+    uint32_t n = M;
+    for (int p = 0; p < passes; ++p) {   // uniform
+        for (int i = threadIdx.x; i < 32 * RS_RADIX; i += 1024) cnt[i] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const bool ok = p0 + 32u * i < n && (p > 0 || k[i] != SORT_DROP_KEY);   // pass 0 drops
+            uint32_t d = 0x100u;
+            if (ok && p < VIEW_PASS) d = (k[i] >> (8 * p)) & 255u;
+            if (ok && p == VIEW_PASS) {
+                int lo = 0, hi = b->n_views - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (s_ent[mid] <= v[i]) lo = mid; else hi = mid - 1;
+                }
+                d = (uint32_t)lo;
+            }
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t below = peers & lanemask_lt();
+            r[i] = (ok && below == 0u) ? atomicAdd(&cnt[warp * RS_RADIX + d], (uint32_t)__popc(peers)) : 0u;
+            meta[i] = (uint32_t)(__ffs(peers) - 1) | (uint32_t)__popc(below) << 5 | d << 16;
+            __syncwarp();
+        }
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            r[i] = __shfl_sync(0xffffffffu, r[i], (int)(meta[i] & 31u)) + ((meta[i] >> 5) & 63u);
+        __syncthreads();
+        uint32_t run = 0u;
+        if (threadIdx.x < RS_RADIX) {
+#pragma unroll 8
+            for (int w = 0; w < 32; ++w) {
+                const uint32_t c = cnt[w * RS_RADIX + threadIdx.x];
+                cnt[w * RS_RADIX + threadIdx.x] = run;
+                run += c;
+            }
+        }
+        uint32_t kept;
+        const uint32_t ds = block_exclusive<uint32_t>(run, kept, shs);
+        if (threadIdx.x < RS_RADIX) dstart[threadIdx.x] = ds;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const uint32_t d = meta[i] >> 16;
+            if (d < RS_RADIX) {
+                const uint32_t pos = dstart[d] + cnt[warp * RS_RADIX + d] + r[i];
+                sk[pos] = k[i];
+                sv[pos] = v[i];
+            }
+        }
+        __syncthreads();
+        n = kept;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (p0 + 32u * i < n) {
+                k[i] = sk[p0 + 32u * i];
+                v[i] = sv[p0 + 32u * i];
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (p0 + 32u * i < n) vout[p0 + 32u * i] = v[i];
+    if (threadIdx.x == 0) aux->kept = n;
+}
+
+template <int ITEMS>
+static cudaError_t depth_small(const Batch *db, const uint32_t *keys, uint32_t M, uint32_t *vout, SortAux *aux,
+                               int passes, cudaStream_t s) {
+    const size_t smem = (size_t)(2 * 1024 * ITEMS + 32 * RS_RADIX) * 4;
+    const cudaError_t e = allow_smem(k_depth_small<ITEMS>, smem);
+    if (e != cudaSuccess) return e;
+    (void)launch_chain_smem(k_depth_small<ITEMS>, dim3(1), dim3(1024), smem, s, keys, M, vout, aux, db, passes);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
                               const uint64_t *n_dev, uint64_t max_n, uint32_t *hist, SortAux *aux, cudaStream_t s) {
     const uint32_t nblocks = (uint32_t)div_up(max_n, RS_TILE);
     if (nblocks == 0) return cudaSuccess;
     if (max_n > SORT_MAX_KEYS) return cudaErrorInvalidValue;   // counts must fit the look-back word
     const int passes = n_views > 1 ? 5 : 4;
-    const uint64_t pass_words = (uint64_t)nblocks * RS_RADIX;
+    if (max_n <= DS_MAX) {
+        uint32_t *out = n_views > 1 ? v1 : v0;
+        const uint32_t M = (uint32_t)max_n;
+        return M <= 2048 ? depth_small<2>(db, k0, M, out, aux, passes, s)
+                         : M <= 4096 ? depth_small<4>(db, k0, M, out, aux, passes, s)
+                                     : depth_small<8>(db, k0, M, out, aux, passes, s);
+    }
+    // Grouped look-back where the kept keys' tiles may all be resident at once
+    // (three per SM) or not far more; beyond, inclusive prefixes are found near by.
+    const bool grouped = nblocks <= 8u * 3u * 152u;
+    const uint64_t pass_words = sort_flag_words(max_n, 1);
     const unsigned hgrid = nblocks < 4u * 152u ? nblocks : 4u * 152u;
     (void)launch_chain(k_os_hist, dim3(hgrid), dim3(RS_THREADS), s, (const uint32_t *)k0, n_dev, max_n, aux, hist,
                        pass_words * passes);
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
     for (int p = 0; p < passes; ++p) {
         // pass 0 leaves SORT_DROP_KEY out and later passes see only the kept keys
-        (void)launch_chain(k_os_pass, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki,
-                           p > 0 ? (const uint32_t *)vi : (const uint32_t *)nullptr, ko, vo, p > 0 ? (const uint64_t *)&aux->kept : n_dev, max_n, p, 8 * p, 255u, p == 0,
+        (void)launch_chain(grouped ? k_os_pass<true> : k_os_pass<false>, dim3(nblocks), dim3(RS_THREADS), s,
+                           (const uint32_t *)ki, p > 0 ? (const uint32_t *)vi : (const uint32_t *)nullptr, ko, vo,
+                           p > 0 ? (const uint64_t *)&aux->kept : n_dev, max_n, p, 8 * p, 255u, p == 0,
                            hist + pass_words * p, aux, (uint2 *)nullptr, (uint64_t)0, sort_wait_polls(),
-                           (const uint64_t *)nullptr, p == VIEW_PASS ? db : (const Batch *)nullptr);
+                           (const uint64_t *)nullptr, p == VIEW_PASS ? db : (const Batch *)nullptr,
+                           hist + pass_words * p + (uint64_t)nblocks * RS_RADIX);
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
@@ -356,15 +513,16 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
     const uint32_t nblocks = (uint32_t)div_up(max_n, RS_TILE);
     const int passes = nblocks ? radix_passes(bits) : 0;
     if (max_n > SORT_MAX_KEYS) return cudaErrorInvalidValue;
-    const uint64_t pass_words = (uint64_t)nblocks * RS_RADIX;
+    const uint64_t pass_words = sort_flag_words(max_n, 1);
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
         const uint32_t mask = (1u << std::min(8, bits - shift)) - 1u;
-        (void)launch_chain(k_os_pass, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki, (const uint32_t *)vi,
+        (void)launch_chain(k_os_pass<false>, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki, (const uint32_t *)vi,
                            ko, vo, (const uint64_t *)(counters + CNT_WRITTEN), max_n, p, shift, mask, false,
                            hist + pass_words * p, aux, p == passes - 1 ? ranges : (uint2 *)nullptr, n_ranges,
-                           sort_wait_polls(), (const uint64_t *)(counters + CNT_STATUS), (const Batch *)nullptr);
+                           sort_wait_polls(), (const uint64_t *)(counters + CNT_STATUS), (const Batch *)nullptr,
+                           (uint32_t *)nullptr);
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
@@ -417,7 +575,7 @@ __device__ __forceinline__ uint32_t bin_view_of_chunk(const BinTab &tab, int n_v
     return (uint32_t)lo;
 }
 
-// Blocks take BIN_BLOCK entries of the depth order at a time, in order, from a
+// Blocks take BIN_ITEMS entries per thread of the depth order at a time, in order, from a
 // ticket. An entry costs its pairs plus BIN_ENTRY_COST (the emitting and the
 // placing warp spend time on both), so entry j's cost starts at
 // X = its first pair + BIN_ENTRY_COST j. A chunk of view v starts at the first
@@ -425,7 +583,7 @@ __device__ __forceinline__ uint32_t bin_view_of_chunk(const BinTab &tab, int n_v
 // views before it): entry j marks the chunks whose threshold lies in
 // (X, X + its cost] with the start j + 1. Every block recomputes the views' tables
 // from preprocess's totals; block 0 publishes them.
-__global__ void __launch_bounds__(256) k_bin_cut(BinArgs a, uint32_t spin_limit) {
+__global__ void __launch_bounds__(BIN_CUT_THREADS) k_bin_cut(BinArgs a, uint32_t spin_limit) {
     chain_wait();
     __shared__ unsigned long long s_out0;
     __shared__ uint64_t shs64[33];
@@ -493,9 +651,10 @@ __global__ void __launch_bounds__(256) k_bin_cut(BinArgs a, uint32_t spin_limit)
             s_blk = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long *>(a.counters + CNT_DUP_BLOCK), 1ull);
         __syncthreads();
         const uint32_t blk = s_blk;
-        if ((uint64_t)blk * BIN_BLOCK >= V) return;   // uniform
+        const uint64_t e0 = (uint64_t)blk * blockDim.x * BIN_ITEMS;   // the block's first entry
+        if (e0 >= V) return;   // uniform
         // BIN_ITEMS consecutive entries per thread
-        const uint64_t j0 = (uint64_t)blk * BIN_BLOCK + (uint64_t)BIN_ITEMS * tid;
+        const uint64_t j0 = e0 + (uint64_t)(BIN_ITEMS * tid);
         uint32_t e[BIN_ITEMS], n[BIN_ITEMS], sum = 0;
 #pragma unroll
         for (int i = 0; i < BIN_ITEMS; i += 4) {   // the order's array is 256-byte aligned
@@ -809,13 +968,6 @@ __global__ void __launch_bounds__(256) k_bin_keys(const uint2 *__restrict__ rang
     }
 }
 
-// Opts a kernel into `bytes` of dynamic shared memory on the current device.
-template <typename K>
-static cudaError_t allow_smem(K kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
     if (a.n_tiles == 0 || a.row == 0 || a.row > BIN_MAX_ROW || a.max_chunks <= (uint32_t)a.n_views ||
         a.max_chunks > BIN_MAX_CHUNKS || a.cap > SORT_MAX_KEYS)
@@ -823,10 +975,14 @@ cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
     const size_t smem = (size_t)a.row * 4;
     const cudaError_t e = allow_smem(k_bin_emit, smem);
     if (e != cudaSuccess) return e;
+    // larger blocks shorten the look-back over many entries (1M: 20 -> 14 us) but
+    // cost the short ones 2 us
+    const unsigned cut_threads = a.M > (1u << 19) ? BIN_CUT_THREADS : 256;
     // one block at least: it publishes the zero total of a call without entries;
     // how many of the M entries are in the order is only known on the device
-    const uint64_t cut = std::min<uint64_t>(std::max<uint64_t>(div_up(a.M, BIN_BLOCK), 1), 4 * 152);
-    (void)launch_chain(k_bin_cut, dim3((unsigned)cut), dim3(256), s, a, sort_wait_polls());
+    const uint64_t cut = std::min<uint64_t>(std::max<uint64_t>(div_up(a.M, cut_threads * BIN_ITEMS), 1),
+                                            2 * 152 * (1024 / cut_threads));
+    (void)launch_chain(k_bin_cut, dim3((unsigned)cut), dim3(cut_threads), s, a, sort_wait_polls());
     (void)launch_chain_smem(k_bin_emit, dim3(a.max_chunks), dim3(256), smem, s, a);
     count_launches(2);
     return cudaGetLastError();

@@ -56,3 +56,27 @@ def test_lists_match_the_binning_rule(name):
     again = GpuView.plain(ds, cams, out)
     assert np.array_equal(again.pair_entry, gv.pair_entry) and np.array_equal(again.ranges, gv.ranges)
     assert torch.equal(img, out.img) and torch.equal(T, out.T_final) and torch.equal(last, out.last)
+
+
+@pytest.mark.parametrize("n,views", [(1, 1), (2048, 1), (2049, 1), (2048, 2), (2049, 2), (8192, 1), (4096, 2), (8193, 1),
+                                     (4097, 2), (60_000, 1), (30_000, 3)])
+def test_depth_order_at_the_kernels_edges(n, views):
+    """One block sorts up to 8192 entries (2, 4 or 8 keys a thread), the digit
+    passes the larger ones; with several views the order is by view first. Every
+    tile list must hold its entries by (depth bits, entry), each entry in as
+    many lists as it reaches tiles. Equal depths are planted."""
+    rng = np.random.default_rng(n + views)
+    scene = synth.make_scene(rng, n, lobes=0, means="cube", cube_side=1.4, masks="uniform")
+    scene.means[2, n // 3:n // 2] = 4.0
+    cams = [synth.make_camera(200 + 16 * v, 120, 150.0) for v in range(views)]
+    ds = DeviceScene.from_host(scene)
+    out = render.render_forward(ds, cams)
+    gv = GpuView.plain(ds, cams, out)
+    assert gv.K == int(gv.tt.sum())
+    np.testing.assert_array_equal(np.bincount(gv.pair_entry, minlength=n * views), gv.tt)
+    depth = gv.rec[gv.pair_entry, 11].view(np.uint32).astype(np.int64)
+    key = (gv.pair_tile * 2**32 + depth) * 1.0   # exact below 2^53: tiles here are few
+    same = np.diff(gv.pair_tile) == 0
+    assert np.all(np.diff(gv.pair_tile) >= 0) and np.all(np.diff(key)[same] >= 0)
+    tie = same & (np.diff(depth) == 0)
+    assert np.all(np.diff(gv.pair_entry)[tie] > 0)
