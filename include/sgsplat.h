@@ -237,7 +237,10 @@ int sg_profile_set_stages(uint32_t stage_mask);
  * launch of resident blocks that take (view, tile) items from a work counter,
  * tiles ordered by descending list length, instead of one block per tile.
  * sg_set_tuning(NULL) restores the defaults: both blends persistent, the
- * forward with 4 pixels per thread, the backward with 8, 64-Gaussian batches.
+ * forward with 4 pixels per thread, the backward with 8, 64-Gaussian batches
+ * (batch 0). While a blend's fields hold these defaults, the call's tile count
+ * picks its pixels per thread (fewer for fewer tiles); a batch size other
+ * than 0 pins the given shape.
  */
 typedef struct sg_tuning {
     int32_t fwd_pixels_per_thread;

@@ -63,7 +63,7 @@ def search(measure, candidates=CANDIDATES, persistent=(0, 1)):
     timings = {}
     for p, q in [(p, q) for q in persistent for p in candidates]:
         timings[(p, q)] = measure(fwd_pixels_per_thread=p, bwd_pixels_per_thread=p, fwd_persistent=q,
-                                  bwd_persistent=q, fwd_batch=0, bwd_batch=0)
+                                  bwd_persistent=q, fwd_batch=64, bwd_batch=64)
     best_f = min(timings, key=lambda k: timings[k]["blend_fwd"])
     best_b = min(timings, key=lambda k: timings[k]["blend_bwd"])
     batch_ms = {}

@@ -102,7 +102,8 @@ struct StageTimer {
 };
 
 // Process-wide kernel shape choices (sg_set_tuning); defaults from measurement
-// (1M Gaussians at 1920x1080: both blends persistent, 4 and 8 pixels per thread).
+// (1M Gaussians at 1920x1080: both blends persistent, 4 and 8 pixels per thread;
+// with fewer tiles the defaults stand for the tile count's choice, auto_pixels).
 constexpr sg_tuning kDefaultTuning = {4, 8, 1, 1, 0, 0, 0, {0}};
 constexpr int kDefaultBatch = 64;
 sg_tuning &tuning() {
@@ -353,15 +354,35 @@ BwdLayout bwd_layout(const Batch &b) {
 
 size_t bwd_bytes(const Batch &b) { return bwd_layout(b).total; }
 
-// Blend shape of this call: pixels per thread from the tuning, and for the
-// persistent form the resident grid, the work counter and the tile order.
-int blend_shape(bool backward, const uint32_t *order, uint32_t *queue, BlendShape &sh) {
+// Pixels per thread while the tuning holds the defaults: with few tiles a
+// warp's walk of its list is the critical path, so a tile is given to more
+// warps; with many, fewer warps per tile issue less in all. The lines lie where the
+// measured times cross (us, forward / backward, 1, 2, 4, 8 pixels per thread):
+//    494 tiles (32k pairs)    27/61    36/84    56/105   78/157
+//   2500 tiles (116k pairs)   29/88    40/99    61/118   85/179
+//   3600 tiles (877k pairs)  134/580  133/393  197/334  278/544
+//   8160 tiles (2.7M pairs)  325/1448 313/945  307/756  384/615
+// (resident blocks: the forward keeps 2432 tiles of 4 pixels per thread in
+// flight, the backward 3648 of 8).
+int auto_pixels(bool backward, uint64_t n_tiles) {
+    if (backward) return n_tiles <= 2560 ? 1 : n_tiles <= 3072 ? 2 : n_tiles <= 5632 ? 4 : 8;
+    return n_tiles <= 3600 ? 1 : n_tiles <= 7680 ? 2 : 4;
+}
+
+// Blend shape of this call: pixels per thread from the tuning (from the tile
+// count while it holds the defaults), and for the persistent form the resident
+// grid, the work counter and the tile order.
+int blend_shape(bool backward, uint64_t n_tiles, const uint32_t *order, uint32_t *queue, BlendShape &sh) {
     const sg_tuning &t = tuning();
     sh.pixels_per_thread = backward ? t.bwd_pixels_per_thread : t.fwd_pixels_per_thread;
     sh.persistent = (backward ? t.bwd_persistent : t.fwd_persistent) != 0;
+    const int nb = backward ? t.bwd_batch : t.fwd_batch;
+    const sg_tuning &d = kDefaultTuning;
+    if (nb == 0 && sh.persistent &&
+        sh.pixels_per_thread == (backward ? d.bwd_pixels_per_thread : d.fwd_pixels_per_thread))
+        sh.pixels_per_thread = auto_pixels(backward, n_tiles);
     sh.tile_order = sh.persistent ? order : nullptr;
     sh.queue = queue;
-    const int nb = backward ? t.bwd_batch : t.fwd_batch;
     sh.batch = nb ? nb : kDefaultBatch;
     sh.grid = sh.persistent ? blend_persistent_grid(backward, sh.pixels_per_thread, sh.batch) : 0;
     if (sh.persistent && sh.grid <= 0)
@@ -577,7 +598,7 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
         counting ? reinterpret_cast<unsigned long long *>(counters + CNT_EVALS) : nullptr;
     if (counting) SG_CUDA(cudaMemsetAsync(evals, 0, 8, stream), "clear counter");
     BlendShape shape{};
-    st = blend_shape(false, reinterpret_cast<uint32_t *>(w + L.order),
+    st = blend_shape(false, b.n_tiles, reinterpret_cast<uint32_t *>(w + L.order),
                      reinterpret_cast<uint32_t *>(counters + CNT_QUEUE), shape);
     if (st != SG_OK) return st;
     shape.status = counters + CNT_STATUS;
@@ -664,7 +685,7 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
         counting ? reinterpret_cast<unsigned long long *>(counters + CNT_EVALS) : nullptr;
     BlendShape shape{};
     // the forward's tile order (longest lists first)
-    st = blend_shape(true, reinterpret_cast<const uint32_t *>(w + L.order),
+    st = blend_shape(true, b.n_tiles, reinterpret_cast<const uint32_t *>(w + L.order),
                      reinterpret_cast<uint32_t *>(counters + CNT_QUEUE), shape);
     if (st != SG_OK) return st;
     shape.status = reinterpret_cast<const uint64_t *>(w + L.counters) + CNT_STATUS;   // the forward's
@@ -870,6 +891,7 @@ int sg_autotune(const sg_scene *scene, const sg_camera *cams, int n_views, void 
         sg_tuning t = saved;
         t.fwd_pixels_per_thread = t.bwd_pixels_per_thread = 1 << (c >> 1);
         t.fwd_persistent = t.bwd_persistent = c & 1;
+        t.fwd_batch = t.bwd_batch = kDefaultBatch;   // the candidate itself, not the tile count's choice
         tuning() = t;
         float tf = 0.f, tb = 0.f;
         for (int r = 0; r <= reps && st == SG_OK; ++r) {

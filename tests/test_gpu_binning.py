@@ -80,3 +80,28 @@ def test_depth_order_at_the_kernels_edges(n, views):
     assert np.all(np.diff(gv.pair_tile) >= 0) and np.all(np.diff(key)[same] >= 0)
     tie = same & (np.diff(depth) == 0)
     assert np.all(np.diff(gv.pair_entry)[tie] > 0)
+
+
+@pytest.mark.parametrize("w,h", [(640, 640), (1024, 640), (1040, 640), (960, 960), (976, 960), (1408, 1024), (1424, 1024),
+                                 (1920, 1024), (1936, 1024)])
+def test_default_shape_at_its_tile_counts(w, h):
+    """The tile count picks the default blends' pixels per thread; on both sides of
+    every line the outputs are those of a pinned shape (bit exact forward, the
+    backward's atomics in another order)."""
+    rng = np.random.default_rng(5)
+    scene = synth.make_scene(rng, 3000, lobes=1, means="cube", cube_side=3.0, masks="uniform")
+    cam = synth.make_camera(w, h, 1.2 * w)
+    ds = DeviceScene.from_host(scene)
+    d = torch.randn(1, 3, h, w, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    out = render.render_forward(ds, [cam])
+    g = render.render_backward(ds, [cam], out, d)
+    old = sgsplat.sg_get_tuning()
+    sgsplat.sg_set_tuning(4, 8, 1, 1, fwd_batch=64, bwd_batch=64)
+    try:
+        ref = render.render_forward(ds, [cam])
+        gr = render.render_backward(ds, [cam], ref, d)
+    finally:
+        sgsplat.sg_set_tuning(**old)
+    assert torch.equal(out.img, ref.img) and torch.equal(out.T_final, ref.T_final) and torch.equal(out.last, ref.last)
+    for k in gr:
+        assert torch.linalg.norm(g[k] - gr[k]) <= 2e-5 * torch.linalg.norm(gr[k]) + 1e-12, k
