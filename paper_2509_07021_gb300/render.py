@@ -53,17 +53,19 @@ def render_forward(scene: DeviceScene, cams, stream=None, importance=None) -> Fo
     if hint is None:
         hint = 8 * scene.n * len(cams)
 
+    packed = _sg.pack(scene, cams)
+
     def call(ws):
         if importance is None:
-            return _sg.sg_render_forward(scene, cams, ws, img, T, last, stream, raise_on_error=False)
+            return _sg.sg_render_forward(scene, cams, ws, img, T, last, stream, raise_on_error=False, packed=packed)
         return _sg.sg_render_forward_importance(scene, cams, ws, img, T, last, importance, stream,
-                                                raise_on_error=False)
+                                                raise_on_error=False, packed=packed)
 
-    sizes = _sg.sg_workspace_query(scene, cams, int(hint * PAIR_HEADROOM) + 1024)
+    sizes = _sg.sg_workspace_query(scene, cams, int(hint * PAIR_HEADROOM) + 1024, packed)
     ws = torch.empty(sizes["ws_bytes"], dtype=torch.uint8, device=device)
     st, out = call(ws)
     if st == _sg.SG_ERR_CAPACITY:
-        sizes = _sg.sg_workspace_query(scene, cams, int(out["n_pairs"] * PAIR_HEADROOM) + 1024)
+        sizes = _sg.sg_workspace_query(scene, cams, int(out["n_pairs"] * PAIR_HEADROOM) + 1024, packed)
         ws = torch.empty(sizes["ws_bytes"], dtype=torch.uint8, device=device)
         st, out = call(ws)
     if st != _sg.SG_OK:

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 
 import numpy as np
@@ -270,44 +271,40 @@ class DeviceScene:
         return cls(dtype_geom=dg, dtype_lobe=dl, dtype_sharp=ds, **kw)
 
     def struct(self):
-        s = sg_scene()
-        s.n = self.n
-        s.n_lobes = self.n_lobes
-        s.dtype_geom, s.dtype_lobe, s.dtype_sharp = self.dtype_geom, self.dtype_lobe, self.dtype_sharp
-        s.color_model = self.color_model
-        for k in self.FLOAT_FIELDS + ("lobe_off",):
-            t = getattr(self, k)
-            setattr(s, k, t.data_ptr() if t.numel() else None)
-        s.sh = self.sh.data_ptr() if self.sh is not None and self.sh.numel() else None
-        return s
+        # packed in one go: field by field, ctypes takes as long as several kernel launches
+        ptr = [0 if t is None else t.data_ptr() for t in (   # (0 for an empty tensor)
+            self.means, self.scales, self.quats, self.opac, self.gmask, self.c0, self.lobe_off, self.axis,
+            self.sharp, self.amp, self.lmask, self.sh)]
+        return sg_scene.from_buffer_copy(_SCENE.pack(self.n, self.n_lobes, self.dtype_geom, self.dtype_lobe,
+                                                     self.dtype_sharp, self.color_model, *ptr))
+
+
+_SCENE = struct.Struct("=2q4i12Q")
+_CAMERA = struct.Struct("=2i4f12f4f")
+assert _SCENE.size == ctypes.sizeof(sg_scene) and _CAMERA.size == ctypes.sizeof(sg_camera)
+
+
+def _pack_camera(cam):
+    vm = np.asarray(cam.viewmat, np.float32).reshape(12)
+    bg = np.asarray(cam.bg, np.float32).reshape(3)
+    return _CAMERA.pack(int(cam.width), int(cam.height), cam.fx, cam.fy, cam.cx, cam.cy, *vm.tolist(), cam.near,
+                        *bg.tolist())
 
 
 def camera_struct(cam):
-    c = sg_camera()
-    c.width, c.height = int(cam.width), int(cam.height)
-    c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    vm = np.asarray(cam.viewmat, np.float32).reshape(12)
-    for i in range(12):
-        c.viewmat[i] = float(vm[i])
-    c.near_plane = float(cam.near)
-    bg = np.asarray(cam.bg, np.float32).reshape(3)
-    for i in range(3):
-        c.bg[i] = float(bg[i])
-    return c
+    return sg_camera.from_buffer_copy(_pack_camera(cam))
 
 
 def camera_array(cams):
-    arr = (sg_camera * len(cams))()
-    for i, cam in enumerate(cams):
-        arr[i] = camera_struct(cam)
-    return arr
+    return (sg_camera * len(cams)).from_buffer_copy(b"".join([_pack_camera(c) for c in cams]))
 
 
 def grads_struct(grads: dict):
     g = sg_grads()
     for k, _ in sg_grads._fields_:
         t = grads.get(k)
-        setattr(g, k, t.data_ptr() if (t is not None and t.numel()) else None)
+        if t is not None:
+            setattr(g, k, t.data_ptr())   # (0 for an empty tensor)
     return g
 
 
@@ -323,9 +320,15 @@ def sg_last_error() -> str:
     return lib().sg_last_error().decode()
 
 
-def sg_workspace_query(scene: DeviceScene, cams, pair_capacity: int) -> dict:
-    s = scene.struct()
-    c = camera_array(cams)
+def pack(scene: DeviceScene, cams):
+    """(scene struct, camera array) of a call. The plain entry points take it as
+    `packed`, so that a caller that makes several of them on one scene and its
+    cameras packs once."""
+    return scene.struct(), camera_array(cams)
+
+
+def sg_workspace_query(scene: DeviceScene, cams, pair_capacity: int, packed=None) -> dict:
+    s, c = packed or pack(scene, cams)
     out = sg_sizes()
     _check(lib().sg_workspace_query(ctypes.byref(s), c, len(cams), int(pair_capacity),
                                     ctypes.byref(out)))
@@ -348,11 +351,10 @@ def sg_workspace_layout(scene: DeviceScene, cams, ws_bytes: int) -> dict:
 
 
 def sg_render_forward(scene: DeviceScene, cams, ws: torch.Tensor, img, T_final, last,
-                      stream=None, raise_on_error=True):
+                      stream=None, raise_on_error=True, packed=None):
     """Returns (status, sizes dict). Raises SGError on failure unless
     raise_on_error is False (then the status is returned)."""
-    s = scene.struct()
-    c = camera_array(cams)
+    s, c = packed or pack(scene, cams)
     out = sg_sizes()
     st = lib().sg_render_forward(ctypes.byref(s), c, len(cams), _ptr(ws), ws.numel(), _ptr(img),
                                  _ptr(T_final), _ptr(last), ctypes.byref(out),
@@ -503,9 +505,8 @@ def sg_render_batched_forward(scenes, cams, view_scene, ws, img, T_final, last, 
 
 
 def sg_render_forward_importance(scene: DeviceScene, cams, ws, img, T_final, last, importance,
-                                 stream=None, raise_on_error=True):
-    s = scene.struct()
-    c = camera_array(cams)
+                                 stream=None, raise_on_error=True, packed=None):
+    s, c = packed or pack(scene, cams)
     out = sg_sizes()
     st = lib().sg_render_forward_importance(ctypes.byref(s), c, len(cams), _ptr(ws), ws.numel(),
                                             _ptr(img), _ptr(T_final), _ptr(last), _ptr(importance),
