@@ -395,9 +395,61 @@ __device__ __forceinline__ void load_colour_base(const SceneDesc &sc, int64_t g,
     cb.lo = max(0, min(__ldg(sc.lobe_off + g), cb.hi));
 }
 
-// Returns the entry's tiles_touched.
-template <int DL, int DS, int CM>
-__device__ __forceinline__ uint32_t preprocess_entry(const ViewDesc &vw, const SceneDesc &sc, int64_t g, float px,
+// Tiles reached by the entries of the warp's lanes (rows: a lane's tile rows from
+// y0, none for a lane without a visible entry). The work items are (lane, row), 32 at a time:
+// lane by lane, a warp would take as long as its tallest rectangle (about 8 rows
+// against 1.8 on average over all lanes; 1M Gaussians: 75 -> 66 us).
+__device__ __forceinline__ uint32_t count_tiles(const TileReach &R, int x0, int x1, int y0, uint32_t rows) {
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t inc = warp_inclusive(rows), exc = inc - rows;
+    const uint32_t n_rows = __shfl_sync(FULL, inc, 31), owners = __ballot_sync(FULL, rows != 0u);
+    const uint32_t x01 = (uint32_t)x0 | (uint32_t)x1 << 16;
+    uint32_t touched = 0u;
+    for (uint32_t base = 0; base < n_rows; base += 32u) {   // uniform
+        // the item's owner: the last lane with rows that starts at or before it
+        const bool own = rows != 0u;
+        const uint32_t before = __ballot_sync(FULL, own && exc < base);
+        const uint32_t heads = __reduce_or_sync(FULL, own && exc >= base && exc < base + 32u ? 1u << (exc - base) : 0u);
+        const int rank = __popc(before) + __popc(heads & (0xffffffffu >> (31 - lane)));   // from 1
+        // the rank-th owner lane
+        uint32_t m = owners;
+        int src = 0, left = rank;
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+            const int c = __popc(m & ((1u << w) - 1u));
+            if (left > c) { left -= c; m >>= w; src += w; }
+        }
+        src &= 31;
+        TileReach S;
+        S.x = __shfl_sync(FULL, R.x, src);
+        S.y = __shfl_sync(FULL, R.y, src);
+        S.B = __shfl_sync(FULL, R.B, src);
+        S.det = __shfl_sync(FULL, R.det, src);
+        S.At = __shfl_sync(FULL, R.At, src);
+        S.ymax = __shfl_sync(FULL, R.ymax, src);
+        S.m = __shfl_sync(FULL, R.m, src);
+        S.invA = __shfl_sync(FULL, R.invA, src);
+        S.mode = __shfl_sync(FULL, R.mode, src);
+        const uint32_t sx = __shfl_sync(FULL, x01, src), s0 = __shfl_sync(FULL, exc, src);
+        const int sy = __shfl_sync(FULL, y0, src);
+        int c0 = 0, c1 = 0;
+        if (base + lane < n_rows)
+            tile_reach_row(S, sy + (int)(base + lane - s0), (int)(sx & 0xFFFFu), (int)(sx >> 16), c0, c1);
+        // back to the owners: the runs of [exc, exc + rows) within this window
+        const uint32_t rinc = warp_inclusive((uint32_t)(c1 - c0));
+        const int hi = (int)min(max(inc, base) - base, 32u) - 1, lo = (int)min(max(exc, base) - base, 32u) - 1;
+        const uint32_t a = __shfl_sync(FULL, rinc, hi & 31), z = __shfl_sync(FULL, rinc, lo & 31);
+        if (own) touched += (hi >= 0 ? a : 0u) - (lo >= 0 ? z : 0u);
+    }
+    return touched;
+}
+
+// Returns the entry's tiles_touched. SPREAD: all lanes of the warp call it together
+// (on false: a lane without a Gaussian) and share the tile rows; else each lane
+// walks its own rows.
+template <int DL, int DS, int CM, bool SPREAD>
+__device__ __forceinline__ uint32_t preprocess_entry(bool on,const ViewDesc &vw, const SceneDesc &sc, int64_t g, float px,
                                                  float py, float pz, const Geo3 &g3, float o, float gm,
                                                  const ColourBase &cb, uint64_t e,
                                                  Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
@@ -405,10 +457,21 @@ __device__ __forceinline__ uint32_t preprocess_entry(const ViewDesc &vw, const S
                                                  uint32_t *__restrict__ dkey, uint8_t *__restrict__ clamp) {
     Geo G;
     project_view(vw, px, py, pz, g3, o, gm, G);
-    if (!G.visible) {
-        tiles_touched[e] = 0u;
-        rect[e] = make_uint2(0u, 0u);
-        dkey[e] = SORT_DROP_KEY;
+    const bool vis = on && G.visible;
+    // tiles of the rectangle that the alpha >= 1/255 ellipse reaches
+    const float reach_t = tile_reach_threshold(G.op);
+    uint32_t touched = 0u;
+    if (SPREAD) {
+        TileReach R;
+        tile_reach_init(G.x, G.y, G.conA, G.conB, G.conC, reach_t, R);
+        touched = count_tiles(R, G.x0, G.x1, G.y0, vis ? (uint32_t)(G.y1 - G.y0) : 0u);
+    }
+    if (!vis) {
+        if (on) {
+            tiles_touched[e] = 0u;
+            rect[e] = make_uint2(0u, 0u);
+            dkey[e] = SORT_DROP_KEY;
+        }
         return 0u;
     }
 
@@ -447,20 +510,19 @@ __device__ __forceinline__ uint32_t preprocess_entry(const ViewDesc &vw, const S
     }
     // channels clamped by max(c, 0) (not c >= 0, NaN included): the backward reads these bits
     clamp[e] = (uint8_t)((cr >= 0.f ? 0u : 1u) | (cg >= 0.f ? 0u : 2u) | (cbl >= 0.f ? 0u : 4u));
-    const float reach_t = tile_reach_threshold(G.op);
     Rec r;
     r.a = make_float4(G.x, G.y, G.conA, G.conB);
     r.b = make_float4(G.conC, reach_t, G.op, fmaxf(cr, 0.f));
     r.c = make_float4(fmaxf(cg, 0.f), fmaxf(cbl, 0.f), G.rf, G.tz);
     rec[e] = r;
-    // tiles of the rectangle that the alpha >= 1/255 ellipse reaches
-    TileReach R;
-    tile_reach_init(G.x, G.y, G.conA, G.conB, G.conC, reach_t, R);
-    uint32_t touched = 0u;
-    for (int ty = G.y0; ty < G.y1; ++ty) {
-        int c0, c1;
-        tile_reach_row(R, ty, G.x0, G.x1, c0, c1);
-        touched += (uint32_t)(c1 - c0);
+    if (!SPREAD) {
+        TileReach R;
+        tile_reach_init(G.x, G.y, G.conA, G.conB, G.conC, reach_t, R);
+        for (int ty = G.y0; ty < G.y1; ++ty) {
+            int c0, c1;
+            tile_reach_row(R, ty, G.x0, G.x1, c0, c1);
+            touched += (uint32_t)(c1 - c0);
+        }
     }
     tiles_touched[e] = touched;
     rect[e] = make_uint2((uint32_t)G.x0 | ((uint32_t)G.x1 << 16), (uint32_t)G.y0 | ((uint32_t)G.y1 << 16));
@@ -473,7 +535,7 @@ __device__ __forceinline__ uint32_t preprocess_entry(const ViewDesc &vw, const S
 // totals (view_pairs, view_visible), which the binning cuts its chunks by: a
 // warp reduction, then one atomic per block.
 template <int DG, int DL, int DS, int CM>
-__global__ void __launch_bounds__(PRE_THREADS)
+__global__ void __launch_bounds__(PRE_THREADS, CM == SG_COLOR_SH3 ? 3 : 4)
 k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
              uint2 *__restrict__ rect, uint32_t *__restrict__ dkey, uint8_t *__restrict__ clamp,
              unsigned long long *__restrict__ view_pairs, uint32_t *__restrict__ view_visible) {
@@ -497,9 +559,8 @@ k_preprocess(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t *__re
     for (int v = 0; v < b.n_views; ++v) {
         const ViewDesc &vw = b.view[v];
         if (vw.scene != si) continue;
-        uint32_t touched = 0u;
-        if (on)
-            touched = preprocess_entry<DL, DS, CM>(vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g, rec,
+        const uint32_t touched =
+            preprocess_entry<DL, DS, CM, true>(on, vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g, rec,
                                                    tiles_touched, rect, dkey, clamp);
         const uint32_t pairs = __reduce_add_sync(0xffffffffu, touched);
         const uint32_t vis = (uint32_t)__popc(__ballot_sync(0xffffffffu, touched != 0u));
@@ -585,9 +646,9 @@ k_preprocess_views(const Batch *__restrict__ bp, Rec *__restrict__ rec, uint32_t
         for (int v = 0; v < b.n_views; ++v) {
             const ViewDesc &vw = b.view[v];
             if (vw.scene != si) continue;
-            uint32_t touched = 0u;
-            if (on)
-                touched = preprocess_entry<DL, DS, CM>(vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g,
+            // (its queued lanes are mostly visible: sharing the rows measured 8 % slower)
+            const uint32_t touched =
+                preprocess_entry<DL, DS, CM, false>(on, vw, sc, g, px, py, pz, g3, o, gm, cb, vw.ent_off + (uint64_t)g,
                                                        rec, tiles_touched, rect, dkey, clamp);
             const uint32_t pairs = __reduce_add_sync(0xffffffffu, touched);
             const uint32_t vis = (uint32_t)__popc(__ballot_sync(0xffffffffu, touched != 0u));
