@@ -255,15 +255,19 @@ __device__ __forceinline__ void blend_fwd_tile(const Batch &b, uint32_t tile, St
     const float x0 = (float)(tx * TILE), y0 = (float)(ty * TILE);
     // Importance: each thread leaves its share of Sum alpha T (over its pixels) for
     // entry k of the batch in part[thread][k]; after the block's next barrier,
-    // thread k sums column k, zeroes it and adds the total to the Gaussian's
-    // score with one atomic (no warp collective per list entry).
+    // lane k of each warp sums its warp's rows of column k (NB = 32), zeroes them and adds
+    // the total to the Gaussian's score with one atomic (no warp collective per
+    // list entry).
     int pending = 0;   // entries of the last batch whose partials are not yet summed
     auto flush = [&]() {
-        for (int k = threadIdx.x; k < pending; k += NT) {
+        const int k = threadIdx.x & 31;
+        if (k < pending) {
+            float *row = part + (threadIdx.x & ~31u) * PS + k;
             float sum = 0.f;
-            for (int t = 0; t < NT; ++t) {
-                sum += part[t * PS + k];
-                part[t * PS + k] = 0.f;
+#pragma unroll 8
+            for (int t = 0; t < 32; ++t) {
+                sum += row[t * PS];
+                row[t * PS] = 0.f;
             }
             // only an entry of this view's scene (a stale id from another view is left out)
             const uint32_t li = sm.id[k] - (uint32_t)vw->ent_off;
@@ -271,6 +275,7 @@ __device__ __forceinline__ void blend_fwd_tile(const Batch &b, uint32_t tile, St
         }
         pending = 0;
     };
+    static_assert(!IMP || NB == 32, "one lane per entry in the importance flush");
     for (int base = 0; base < n; base += NB) {
         bool all = true;
 #pragma unroll
