@@ -43,14 +43,14 @@ __global__ void __launch_bounds__(256) k_post_count(const sg_scene sc, float tau
 // lobes in one 64-bit word (31 bits each; both totals are below 2^31) and finds
 // its offsets by a decoupled look-back: one launch instead of a three-kernel
 // scan for each. The block holding the last Gaussian writes the totals.
-constexpr int POST_ITEMS = 8, POST_BLOCK = 256 * POST_ITEMS;
+constexpr int POST_ITEMS = 8, POST_THREADS = 1024, POST_BLOCK = POST_THREADS * POST_ITEMS;
 struct PostState {
     uint64_t totals[2];   // Gaussians, lobes
     uint64_t status;      // SG_ERR_TIMEOUT when a block gave up its bounded wait
     uint64_t block_ctr;
 };
 
-__global__ void __launch_bounds__(256) k_post_scan(int64_t n, uint32_t *__restrict__ gidx, uint32_t *__restrict__ loff,
+__global__ void __launch_bounds__(POST_THREADS) k_post_scan(int64_t n, uint32_t *__restrict__ gidx, uint32_t *__restrict__ loff,
                                                    PostState *__restrict__ st, uint64_t *__restrict__ flags,
                                                    uint32_t spin_limit) {
     __shared__ uint64_t shs[33];
@@ -261,7 +261,7 @@ cudaError_t launch_post_plan(const sg_scene &sc, float tau_o, float tau_s, void 
     if (sc.n > 0) {
         uint32_t *gidx = reinterpret_cast<uint32_t *>(w + L.gidx);
         k_post_count<<<(unsigned)div_up((uint64_t)sc.n, 256), 256, 0, s>>>(sc, tau_o, tau_s, gidx);
-        k_post_scan<<<(unsigned)div_up((uint64_t)sc.n, POST_BLOCK), 256, 0, s>>>(
+        k_post_scan<<<(unsigned)div_up((uint64_t)sc.n, POST_BLOCK), POST_THREADS, 0, s>>>(
             sc.n, gidx, reinterpret_cast<uint32_t *>(w + L.loff), st, reinterpret_cast<uint64_t *>(w + L.flags),
             sort_wait_polls());
         count_launches(2);
