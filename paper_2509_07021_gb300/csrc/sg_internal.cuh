@@ -416,7 +416,7 @@ constexpr uint32_t BIN_MAX_ROW = 56 * 1024;
 constexpr uint32_t BIN_MIN_CHUNK = 256;
 // An entry's share of a chunk's cost besides its pairs (one each).
 constexpr uint32_t BIN_ENTRY_COST = 1;
-constexpr uint32_t BIN_MAX_CHUNKS = 6 * 152;
+constexpr uint32_t BIN_MAX_CHUNKS = 5 * 152;
 // Per-call tables of the binning (workspace; view_pairs zeroed by the setup kernel).
 struct BinTab {
     unsigned long long view_pairs[SG_MAX_VIEWS];   // pairs of each view (preprocess)

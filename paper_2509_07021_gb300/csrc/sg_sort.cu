@@ -551,18 +551,21 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
 // look-back followed by chunks of 8192 pairs or, past 12288 tiles, three radix
 // passes): 32k pairs 82 -> 31 us, 116k 91 -> 41, 3.9M 162 -> 129, 5.4M 195 -> 168,
 // 11.8M over four views 450 -> 348, 252M over 16 views 10.5 -> 6.4 ms. The
-// placement is bound by its warps' serial rounds (~400 cycles each, six warps
+// placement is bound by its warps' serial rounds (~400 cycles each, five warps
 // per SM) up to some 20M pairs, beyond by its scattered 4-byte stores.
 uint32_t bin_rows(uint64_t cap, uint32_t row) {
     // Resident placing blocks, each holding one row of cursors in shared memory:
-    // six one-warp blocks per SM, five below 1M pairs (a smaller matrix).
-    const uint32_t want = cap > (1u << 20) ? 6u : 5u;
+    // five one-warp blocks per SM, four below 1M pairs (a smaller matrix). More
+    // place no faster and cost the matrix's scan (4 / 5 / 6 per SM: emission, scan and
+    // placement 155 / 151 / 164 us at 5.4M pairs, 125 / 122 / 129 at 3.9M).
+    const uint32_t want = cap > (1u << 20) ? 5u : 4u;
     return 152u * std::max(std::min(want, (227u * 1024u) / (row * 4u + 1024u)), 1u);
 }
 
 uint32_t bin_chunks(uint64_t cap, uint32_t row) {
     // Past 16M pairs the chunks' open output sectors (chunks x tiles x 32 bytes,
-    // over every view) no longer fit L2: four per SM place faster than six.
+    // over every view) no longer fit L2: four per SM place faster (252M pairs:
+    // eight 5.0 ms, four 3.8).
     return std::min(bin_rows(cap, row), cap > (16u << 20) ? 4u * 152u : BIN_MAX_CHUNKS);
 }
 
