@@ -339,26 +339,22 @@ def gpu_errors_vs_oracle(scene, cam, d_img, storages=("f32", "f16_bf16s"), n_til
 def stage_rooflines(stages_ms, counts, evals, hbm_gbs):
     """Achieved fraction of roofline for every stage: algorithmic bytes (HBM
     stages) or flops (blend) per step over the stage's event time per step.
-    counts: N Gaussians, L lobes, M entries, V entries with pairs, K pairs, T tiles;
-    counting: the tile sort counted (cap: the pair capacity, which sets its chunks)."""
+    counts: N Gaussians, L lobes, M entries, V entries with pairs, K pairs, T tiles of the one
+    view (the binning's chunks hold a counter per tile, five chunks per SM)."""
     N, L, M, V, K, T = (counts[k] for k in ("N", "L", "M", "V", "K", "T"))
+    C = min(SM_COUNT * max(1, min(5, 232448 // (4 * T + 1024))), 1 + K // 256)
     by = {
-        "preprocess": 64 * N + 32 * L + 69 * M,                 # params in; record, tt, rect, clamp, key, value out
-        "depth_sort": 4 * M + 8 * M + 8 * V + 3 * 16 * V,       # histogram, pass 0 (drops), passes 1-3
-        "pair_offsets": 12 * V,                                 # sorted id + tt in, offset out
-        "duplicate": 64 * V + 8 * K,                            # id, tt, rect, record in; pairs out
-        "tile_sort": 4 * K + 2 * 16 * K + 8 * T,                # histogram, two passes, tile ranges
+        "preprocess": 64 * N + 32 * L + 65 * M,                 # params in; record, tt, rect, clamp, key out
+        "depth_sort": 4 * M + 4 * M + 8 * V + 3 * 16 * V,       # histogram, pass 0 (drops), passes 1-3
+        # chunk cutter: id, tt in, first pair out; pairs: id, first pair, rect, record in, 16-bit
+        # tiles and entries out, the [C][T] count matrix out
+        "duplicate": 12 * V + 40 * V + 6 * K + 4 * C * T,
+        # matrix read and rewritten by the scan, read by the placing; pairs in, entries out; ranges
+        "tile_sort": 12 * C * T + 6 * K + 4 * K + 8 * T,
         "tile_ranges": 12 * T,                                  # persistent tile order: ranges in, order out
         "bwd_clear": 36 * M,
         "preprocess_bwd": 64 * N + 32 * L + 41 * M + 60 * N + 32 * L,
     }
-    if counts.get("counting"):
-        # chunks of the counting tile sort (at most 608, 8192 pairs of capacity each)
-        C = min(608, max(1, -(-int(counts["cap"]) // 8192)))
-        by["duplicate"] = 64 * V + 6 * K                        # 16-bit tile keys
-        # keys read twice, entries read and written; the [C][T] count matrix written,
-        # read and rewritten by the scan, read by the placing; tile ranges
-        by["tile_sort"] = 4 * K + 8 * K + 16 * C * T + 8 * T
     out = {}
     for k, ms in stages_ms.items():
         if ms <= 0:
@@ -544,8 +540,7 @@ def run_ours(args, world, rank, local):
     M = out.sizes["n_entries"]
     tt = out.ws[lay["tiles_touched"]:lay["tiles_touched"] + 4 * M].view(torch.int32)
     counts = {"N": scene.n, "L": scene.n_lobes, "M": M, "V": int((tt != 0).sum().item()),
-              "K": n_pairs, "T": cam.n_tiles, "cap": out.sizes["pair_capacity"],
-              "counting": lay["pair_tile"] == 2**64 - 1}
+              "K": n_pairs, "T": cam.n_tiles}
     hbm_peak = 6800.0
     try:
         hbm_peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"])
