@@ -278,8 +278,12 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
     L.clamp = take(M);
     L.dup_flags = take(div_up(M, 256) * 8 + 8);   // look-back words of the chunk cutter / the duplicate
     L.ranges = take(T * 8);
-    L.order = take(T * 4);   // tile order of the persistent blends (forward and backward)
-    L.order_scratch = take(TILE_ORDER_WORDS * 4);
+    L.order = take(T * 4);   // tile order of the persistent blends (by list length)
+    // the forward's tile order: its counts and cursors; the backward's: its counts,
+    // then each tile's place (see TileOrder)
+    L.order_scratch = take((TILE_ORDER_WORDS + TB_BUCKETS) * 4);
+    L.walk = L.order_scratch + TILE_ORDER_WORDS * 4;
+    take(walk_ordered(T) ? 4 * T : 0);
     L.bin = take(sizeof(BinTab));
     L.scan_words = take(8 * (1 + (uint64_t)b.n_groups));
     L.fixed_end = o;
@@ -335,10 +339,11 @@ uint64_t capacity_for(const Batch &b, size_t ws_bytes) {
     return lo;
 }
 
-// Backward scratch: batch table, counters and the [M][9] 2D gradients (the
-// persistent backward takes its tile order from the forward's workspace).
+// Backward scratch: batch table, counters, the [M][9] 2D gradients and the
+// persistent backward's own tile order (where walk_ordered; elsewhere it takes the
+// forward's).
 struct BwdLayout {
-    size_t batch, counters, dg, total;
+    size_t batch, counters, dg, order, total;
 };
 
 BwdLayout bwd_layout(const Batch &b) {
@@ -348,6 +353,7 @@ BwdLayout bwd_layout(const Batch &b) {
     L.batch = take(sizeof(Batch));
     L.counters = take(CNT_N * sizeof(uint64_t));
     L.dg = take(9 * b.n_entries * sizeof(float));
+    L.order = take(walk_ordered(b.n_tiles) ? 4 * (size_t)b.n_tiles : 0);
     L.total = o;
     return L;
 }
@@ -507,7 +513,7 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
         };
         zero(aux_depth, sizeof(SortAux) / 4);
         zero(dup_flags, 2 * div_up(M, 256));
-        zero(w + L.order_scratch, TILE_ORDER_WORDS);
+        zero(w + L.order_scratch, TILE_ORDER_WORDS + TB_BUCKETS);
         zero(tab, sizeof(tab->view_pairs) / 4);
         if (L.chunked) {
             zero(w + L.scan_words, 2 * (1 + (uint64_t)b.n_groups));
@@ -602,6 +608,7 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
                      reinterpret_cast<uint32_t *>(counters + CNT_QUEUE), shape);
     if (st != SG_OK) return st;
     shape.status = counters + CNT_STATUS;
+    if (walk_ordered(b.n_tiles)) shape.walk_counts = reinterpret_cast<uint32_t *>(w + L.walk);
     shape.importance = want_importance && !counting;
     if (shape.importance)
         for (int s = 0; s < n_scenes; ++s)
@@ -684,9 +691,19 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     unsigned long long *evals =
         counting ? reinterpret_cast<unsigned long long *>(counters + CNT_EVALS) : nullptr;
     BlendShape shape{};
-    // the forward's tile order (longest lists first)
-    st = blend_shape(true, b.n_tiles, reinterpret_cast<const uint32_t *>(w + L.order),
+    // Tiles by the forward's largest last position: the walk's length, where the list's
+    // is only its bound (a list's tail lies behind stopped pixels). With two or three
+    // tiles per resident warp the last ones to start decide when the kernel ends.
+    TileOrder walk;
+    if (walk_ordered(b.n_tiles)) {
+        walk.counts = reinterpret_cast<const uint32_t *>(w + L.walk);
+        walk.place = walk.counts + TB_BUCKETS;
+        walk.order = reinterpret_cast<uint32_t *>(bw + BL.order);
+        walk.n = b.n_tiles;
+    }
+    st = blend_shape(true, b.n_tiles, walk.n ? walk.order : reinterpret_cast<const uint32_t *>(w + L.order),
                      reinterpret_cast<uint32_t *>(counters + CNT_QUEUE), shape);
+    if (!shape.persistent) walk = TileOrder();
     if (st != SG_OK) return st;
     shape.status = reinterpret_cast<const uint64_t *>(w + L.counters) + CNT_STATUS;   // the forward's
     {
@@ -695,7 +712,7 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
         ZeroRegions z;
         z.ptr[0] = reinterpret_cast<uint32_t *>(dg);
         z.words[0] = 9 * M;
-        SG_CUDA(launch_setup(b, db, counters, stream, z), "setup");
+        SG_CUDA(launch_setup(b, db, counters, stream, z, walk), "setup");
     }
     {
         StageTimer t(ST_BLEND_BWD, stream);

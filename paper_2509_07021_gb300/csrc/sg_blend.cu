@@ -218,8 +218,9 @@ enum : int { FWD_PLAIN = 0, FWD_COUNT = 1, FWD_IMPORTANCE = 2 };
 // lists_ok false: a sort's bounded wait gave up in this forward (its lists may
 // hold stale words): every tile renders as an empty list. (On a capacity
 // overflow the tile sort does not run and every range stays empty.)
+// Returns the largest last position of the thread's pixels.
 template <int P, int MODE, int NB>
-__device__ __forceinline__ void blend_fwd_tile(const Batch &b, uint32_t tile, StagedN<NB> &sm,
+__device__ __forceinline__ int blend_fwd_tile(const Batch &b, uint32_t tile, StagedN<NB> &sm,
                                                const uint2 *__restrict__ ranges,
                                                const uint32_t *__restrict__ pval,
                                                const Rec *__restrict__ rec, float *__restrict__ img,
@@ -348,6 +349,7 @@ __device__ __forceinline__ void blend_fwd_tile(const Batch &b, uint32_t tile, St
     }
     const uint64_t HW = (uint64_t)vw->W * (uint64_t)vw->H;
     float *im = img + 3 * vw->pix_off;
+    int walk = 0;
 #pragma unroll
     for (int j = 0; j < P; ++j) {
         const int px = (int)fpx[j], py = (int)fpy[j];
@@ -359,40 +361,78 @@ __device__ __forceinline__ void blend_fwd_tile(const Batch &b, uint32_t tile, St
             T_final[vw->pix_off + pix] = T[j];
             last[vw->pix_off + pix] = lastc[j];
         }
+        walk = max(walk, lastc[j]);
     }
+    return walk;
+}
+
+// Files the tile under its walk length (the largest last position of its pixels) for the
+// backward's order: its warps combine theirs in shared memory, and the last to arrive
+// takes the tile's rank in its bucket. *s_walk and *s_arrived are zero before and after;
+// a barrier lies between a block's tiles.
+template <int NW>
+__device__ __forceinline__ void tile_done(int walk, uint32_t tile, uint32_t *s_walk, uint32_t *s_arrived,
+                                          uint32_t *counts) {
+    if (counts == nullptr) return;
+    walk = __reduce_max_sync(0xffffffffu, walk);
+    if ((threadIdx.x & 31) != 0) return;
+    uint32_t len = (uint32_t)walk;
+    if (NW > 1) {
+        atomicMax(s_walk, len);
+        __threadfence_block();
+        if (atomicAdd(s_arrived, 1u) != NW - 1) return;
+        len = atomicExch(s_walk, 0u);
+        *s_arrived = 0u;
+    }
+    const uint32_t bucket = len_bucket(len);
+    counts[TB_BUCKETS + tile] = bucket << 24 | atomicAdd(&counts[bucket], 1u);
 }
 
 // Persistent form: resident blocks pull tiles from a work counter in the
 // given order (longest lists first); otherwise one block per tile.
+// The 4-pixel plain form asks for 16 blocks per SM (64 registers): without the bound it
+// takes 72 and 14 blocks (297 -> 308 us at 3.9M pairs, 1920x1080; 5.26 -> 5.54 ms
+// over 16 views), with 18 it spills (333 us). The others keep the compiler's choice: a
+// bound of one block raises the 1-pixel form from 40 to 67 registers (130 -> 176 us).
 template <int P, int MODE, bool PERSIST, int NB>
-__global__ void __launch_bounds__(BLEND_THREADS / P)
+__global__ void __launch_bounds__(BLEND_THREADS / P, P == 4 && MODE == FWD_PLAIN ? 16 : 0)
 k_blend_fwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
             const uint32_t *__restrict__ pval, const Rec *__restrict__ rec,
             float *__restrict__ img, float *__restrict__ T_final, int32_t *__restrict__ last,
             const uint32_t *__restrict__ tile_order, uint32_t *__restrict__ queue, uint32_t n_tiles,
-            unsigned long long *__restrict__ evals, const uint64_t *__restrict__ status) {
+            unsigned long long *__restrict__ evals, const uint64_t *__restrict__ status,
+            uint32_t *__restrict__ walk_counts) {
     chain_enter();
     __shared__ StagedN<NB> sm;
     __shared__ float part[MODE == FWD_IMPORTANCE ? (BLEND_THREADS / P) * (NB + 1) : 1];
-    __shared__ uint32_t s_item;
+    constexpr int NW = BLEND_THREADS / P / 32;
+    __shared__ uint32_t s_item, s_tile, s_walk, s_arrived;
     const Batch &b = *bp;
     uint32_t ne = 0;
+    if (threadIdx.x == 0) s_walk = s_arrived = 0u;
+    if (!PERSIST) __syncthreads();   // (the persistent loop starts with one)
     const bool lists_ok = *status != (uint64_t)SG_ERR_TIMEOUT;
     if (MODE == FWD_IMPORTANCE) {
         for (int i = threadIdx.x; i < (BLEND_THREADS / P) * (NB + 1); i += BLEND_THREADS / P) part[i] = 0.f;
         __syncthreads();
     }
     if (!PERSIST) {
-        blend_fwd_tile<P, MODE, NB>(b, blockIdx.x, sm, ranges, pval, rec, img, T_final, last, ne, lists_ok, part);
+        const int walk = blend_fwd_tile<P, MODE, NB>(b, blockIdx.x, sm, ranges, pval, rec, img, T_final, last, ne,
+                                                     lists_ok, part);
+        if (MODE != FWD_IMPORTANCE) tile_done<NW>(walk, blockIdx.x, &s_walk, &s_arrived, walk_counts);
     } else {
         for (;;) {
             if (threadIdx.x == 0) s_item = atomicAdd(queue, 1u);
             __syncthreads();
             const uint32_t item = s_item;
+            if (item < n_tiles && threadIdx.x == 0) s_tile = tile_order ? tile_order[item] : item;
             __syncthreads();
             if (item >= n_tiles) break;
-            blend_fwd_tile<P, MODE, NB>(b, tile_order ? tile_order[item] : item, sm, ranges, pval, rec, img,
-                                        T_final, last, ne, lists_ok, part);
+            const int walk = blend_fwd_tile<P, MODE, NB>(b, s_tile, sm, ranges, pval, rec, img, T_final, last, ne,
+                                                         lists_ok, part);
+            // from shared memory: no register holds the tile across the walk (the next
+            // item overwrites s_tile only after a barrier that every warp has passed)
+            if (MODE != FWD_IMPORTANCE) tile_done<NW>(walk, s_tile, &s_walk, &s_arrived, walk_counts);
         }
     }
     if (MODE == FWD_COUNT) add_evals(ne, evals);
@@ -404,7 +444,8 @@ static void fwd_launch(const Batch *db, uint32_t n_tiles, const uint2 *ranges, c
                        unsigned long long *evals, cudaStream_t s) {
     const unsigned grid = PERSIST ? (unsigned)sh.grid : n_tiles;
     (void)launch_chain(k_blend_fwd<P, MODE, PERSIST, NB>, dim3(grid), dim3(BLEND_THREADS / P), s,
-        db, ranges, pval, rec, img, T_final, last, sh.tile_order, sh.queue, n_tiles, evals, sh.status);
+        db, ranges, pval, rec, img, T_final, last, sh.tile_order, sh.queue, n_tiles, evals, sh.status,
+        sh.walk_counts);
 }
 
 // The plain forward takes the batch size of the tuning; the counting form

@@ -98,7 +98,7 @@ constexpr int RS_RADIX = 256;
 // forward and the backward of one call).
 struct WsLayout {
     size_t batch, counters, rec, tiles_touched, rect, clamp, dkey0, dval0, dkey1, dval1,
-        dup_flags, ranges, order, order_scratch, bin, scan_words, hist, aux_depth, aux_tile, fixed_end;
+        dup_flags, ranges, order, order_scratch, walk, bin, scan_words, hist, aux_depth, aux_tile, fixed_end;
     size_t pval_final, pkey_final, pval_tmp, pkey_tmp, total;
     uint64_t M, n_tiles, cap;
     int tile_bits, tile_passes;
@@ -351,6 +351,25 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 void count_launches(int n);
 
 // ---- launchers (host side, defined in the .cu files) ----
+// Buckets by list length on a log scale with 8 buckets per octave (exponent and
+// the 3 bits below the leading one), longest bucket first; inside a bucket the
+// order is whatever the atomics give (it only steers scheduling).
+constexpr int TB_BUCKETS = 256;
+__device__ __forceinline__ uint32_t len_bucket(uint32_t len) {
+    len |= 1u;
+    const uint32_t e = 31u - (uint32_t)__clz(len);              // 0..31
+    const uint32_t m = e >= 3u ? (len >> (e - 3u)) & 7u : (len << (3u - e)) & 7u;
+    return e * 8u + m;                                           // 0..255
+}
+
+// Tiles by descending walk length (a tile's largest last position): written by the
+// setup kernel's last blocks while the others zero their regions (n = 0: none).
+struct TileOrder {
+    const uint32_t *counts = nullptr;   // [TB_BUCKETS] tiles per walk-length bucket
+    const uint32_t *place = nullptr;    // [n] bucket << 24 | rank inside it
+    uint32_t *order = nullptr;          // [n]
+    uint32_t n = 0;
+};
 // Up to N device regions of 32-bit words that the setup kernel zeroes.
 // Regions the setup kernel fills: word i of region r gets even[r] if i is
 // even, else 0 (even[r] = 0: plain zeroing).
@@ -361,7 +380,7 @@ struct ZeroRegions {
     uint32_t even[N] = {};
 };
 cudaError_t launch_setup(const Batch &b, Batch *dst, uint64_t *counters, cudaStream_t s,
-                         const ZeroRegions &z = ZeroRegions());
+                         const ZeroRegions &z = ZeroRegions(), const TileOrder &o = TileOrder());
 // clamp [M]: bit ch set where colour channel ch was clamped by max(c, 0).
 // view_pairs, view_visible (zeroed): receive each view's pairs and its entries
 // with at least one pair.
@@ -492,6 +511,14 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
 // scratch: TILE_ORDER_WORDS zeroed words whose first 256 already hold the
 // bucket counts (filled by the tile sort).
 constexpr int TILE_ORDER_WORDS = 512;
+// Tile counts whose backward gets an order of its own: its 8-pixel form starts at
+// 5632 tiles, and with two or three tiles per resident warp the longest of the last
+// decide when the kernel ends (8160 tiles, 5.4M pairs: 610 -> 575 us; 3.9M: 564 -> 555).
+// With fewer tiles several warps share each (3600: 305 us with either order, and the
+// forward pays 1 us for the ranks); with more, a warp takes several tiles and the
+// forward's order ends as evenly (six scenes in four views each: 6.64 ms with either).
+constexpr uint32_t WALK_ORDER_MIN = 5632, WALK_ORDER_MAX = 16384;
+inline bool walk_ordered(uint64_t n_tiles) { return n_tiles > WALK_ORDER_MIN && n_tiles <= WALK_ORDER_MAX; }
 cudaError_t launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t *scratch,
                               cudaStream_t s);
 
@@ -504,6 +531,8 @@ struct BlendShape {
     int grid;                     // persistent: resident blocks
     bool importance;              // forward: accumulate SceneDesc::importance
     const uint64_t *status;       // the forward's status word: SG_ERR_TIMEOUT = lists unusable
+    uint32_t *walk_counts;        // forward: TileOrder::counts (zeroed), then ::place, for the backward's
+                                  // tile order (null: none wanted)
     int batch;                    // Gaussians staged per shared-memory batch
 };
 

@@ -226,17 +226,38 @@ struct BatchParam {
 };
 static_assert(offsetof(Batch, view) % 8 == 0, "batch header");
 
+constexpr int SETUP_THREADS = 256;
+static_assert(SETUP_THREADS == TB_BUCKETS, "one bucket per thread");
+__host__ __device__ inline unsigned order_blocks(const TileOrder &o) {
+    return (o.n + SETUP_THREADS - 1) / SETUP_THREADS;
+}
+
 // Writes the table into the workspace, zeroes the counters and the regions the
 // caller names (e.g. tile ranges, sort scratch, the backward's accumulators),
 // and seeds the entry and tile counts. Block 0 writes the table and counters;
 // every block zeroes its share of the regions (16-byte stores where a region
-// starts on a 16-byte boundary).
+// starts on a 16-byte boundary). The blocks past those write the tile order o.
 template <int NV, int NS>
-__global__ void __launch_bounds__(256) k_setup(const BatchParam<NV, NS> p, Batch *dst, uint64_t *counters,
-                                               ZeroRegions z) {
+__global__ void __launch_bounds__(SETUP_THREADS) k_setup(const BatchParam<NV, NS> p, Batch *dst, uint64_t *counters,
+                                                         ZeroRegions z, TileOrder o) {
     chain_enter();
+    const unsigned zero_blocks = gridDim.x - order_blocks(o);
+    if (blockIdx.x >= zero_blocks) {
+        // longest walks first: exclusive scan over the buckets in reverse
+        __shared__ uint32_t base[TB_BUCKETS];
+        __shared__ uint32_t shs[33];
+        const uint32_t t = (blockIdx.x - zero_blocks) * SETUP_THREADS + threadIdx.x;
+        const uint32_t place = t < o.n ? o.place[t] : 0u;
+        uint32_t tot;
+        base[TB_BUCKETS - 1 - threadIdx.x] =
+            block_exclusive<uint32_t>(o.counts[TB_BUCKETS - 1 - threadIdx.x], tot, shs);
+        __syncthreads();
+        const uint32_t at = base[place >> 24] + (place & 0xFFFFFFu);
+        if (t < o.n && at < o.n) o.order[at] = t;
+        return;
+    }
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t nth = (uint64_t)zero_blocks * blockDim.x;
     for (int r = 0; r < ZeroRegions::N; ++r) {
         uint32_t *ptr = z.ptr[r];
         const uint64_t words = z.words[r];
@@ -271,7 +292,8 @@ __global__ void __launch_bounds__(256) k_setup(const BatchParam<NV, NS> p, Batch
 }
 
 template <int NV, int NS>
-static cudaError_t setup_t(const Batch &b, Batch *dst, uint64_t *counters, const ZeroRegions &z, cudaStream_t s) {
+static cudaError_t setup_t(const Batch &b, Batch *dst, uint64_t *counters, const ZeroRegions &z,
+                           const TileOrder &o, cudaStream_t s) {
     BatchParam<NV, NS> p;
     std::memcpy(p.head, &b, sizeof(p.head));
     std::memcpy(p.view, b.view, (size_t)b.n_views * sizeof(ViewDesc));
@@ -280,15 +302,17 @@ static cudaError_t setup_t(const Batch &b, Batch *dst, uint64_t *counters, const
     uint64_t words = 0;
     for (int r = 0; r < ZeroRegions::N; ++r) words += z.words[r];
     const uint64_t blocks = std::min<uint64_t>(std::max<uint64_t>(div_up(words, 256 * 32), 1), 4 * 152);
-    (void)launch_chain(k_setup<NV, NS>, dim3((unsigned)blocks), dim3(256), s, p, dst, counters, z);
+    (void)launch_chain(k_setup<NV, NS>, dim3((unsigned)blocks + order_blocks(o)), dim3(SETUP_THREADS), s, p, dst,
+                       counters, z, o);
     count_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_setup(const Batch &b, Batch *dst, uint64_t *counters, cudaStream_t s, const ZeroRegions &z) {
+cudaError_t launch_setup(const Batch &b, Batch *dst, uint64_t *counters, cudaStream_t s, const ZeroRegions &z,
+                         const TileOrder &o) {
     static_assert(sizeof(BatchParam<SG_MAX_VIEWS, SG_MAX_SCENES>) < 32000, "batch must fit the kernel parameters");
-    if (b.n_views <= 4 && b.n_scenes <= 2) return setup_t<4, 2>(b, dst, counters, z, s);
-    return setup_t<SG_MAX_VIEWS, SG_MAX_SCENES>(b, dst, counters, z, s);
+    if (b.n_views <= 4 && b.n_scenes <= 2) return setup_t<4, 2>(b, dst, counters, z, o, s);
+    return setup_t<SG_MAX_VIEWS, SG_MAX_SCENES>(b, dst, counters, z, o, s);
 }
 
 // ---------------------------------------------------------------------------

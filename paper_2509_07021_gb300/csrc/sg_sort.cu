@@ -317,16 +317,7 @@ uint64_t sort_flag_words(uint64_t max_n, int passes) {
     return (tiles + div_up(tiles, LB_WINDOW)) * RS_RADIX * (uint64_t)passes;
 }
 
-// Buckets by list length on a log scale with 8 buckets per octave (exponent and
-// the 3 bits below the leading one), longest bucket first; inside a bucket the
-// order is whatever the atomics give (it only steers scheduling).
-constexpr int TB_BUCKETS = 256;
-__device__ __forceinline__ uint32_t len_bucket(const uint2 r) {
-    const uint32_t len = (r.y - r.x) | 1u;
-    const uint32_t e = 31u - (uint32_t)__clz(len);              // 0..31
-    const uint32_t m = e >= 3u ? (len >> (e - 3u)) & 7u : (len << (3u - e)) & 7u;
-    return e * 8u + m;                                           // 0..255
-}
+__device__ __forceinline__ uint32_t len_bucket(const uint2 r) { return len_bucket(r.y - r.x); }
 
 // After the radix tile sort: tiles that got no pair get the range (0, 0), every
 // tile joins its list-length bucket (len_bucket), and the sort's status is
