@@ -369,7 +369,7 @@ size_t bwd_bytes(const Batch &b) { return bwd_layout(b).total; }
 //   3600 tiles (877k pairs)  134/580  133/393  197/334  278/544
 //   8160 tiles (2.7M pairs)  325/1448 313/945  307/756  384/615
 // (resident blocks: the forward keeps 2432 tiles of 4 pixels per thread in
-// flight, the backward 3648 of 8).
+// flight, the backward 4256 of 8).
 int auto_pixels(bool backward, uint64_t n_tiles) {
     if (backward) return n_tiles <= 2560 ? 1 : n_tiles <= 3072 ? 2 : n_tiles <= 5632 ? 4 : 8;
     return n_tiles <= 3600 ? 1 : n_tiles <= 7680 ? 2 : 4;

@@ -67,10 +67,14 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 static_assert(BWD_BATCH_MAX % 32 == 0 && FWD_BATCH_MAX % 32 == 0, "batch sizes");
-// Minimum resident blocks requested for the 8-pixels-per-thread backward.
-#ifndef SG_BWD8_MIN_BLOCKS
-#define SG_BWD8_MIN_BLOCKS 24
-#endif
+// Resident blocks per SM requested for the backward.
+// 8 pixels per thread: 28 (72 registers, 8 bytes spilled) against 24 (80, none): 5.4M
+// pairs at 1920x1080 575 -> 565 us, 16 views 9.17 -> 8.86 ms, six scenes in four views
+// 6.64 -> 6.40; 32 (64 registers, batches of 32) 578 us.
+// 1 pixel: 4 (64 registers) against 3: 2500 tiles 78 -> 70 us, where a tile fewer
+// waits for a block; 494 tiles, nearly all resident at once, 52 -> 54.
+// 4 pixels: the compiler's 80 registers; 14 or 16 blocks 313 -> 344, 352 us (3600 tiles).
+constexpr int bwd_min_blocks(int P) { return P == 8 ? 28 : P == 1 ? 4 : 1; }
 
 template <int NB>
 struct StagedN {
@@ -732,7 +736,7 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
 }
 
 template <int P, bool COUNT, bool PERSIST>
-__global__ void __launch_bounds__(BLEND_THREADS / P, P == 8 ? SG_BWD8_MIN_BLOCKS : 1)
+__global__ void __launch_bounds__(BLEND_THREADS / P, bwd_min_blocks(P))
 k_blend_bwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
             const uint32_t *__restrict__ pval, const Rec *__restrict__ rec,
             const float *__restrict__ T_final, const int32_t *__restrict__ last,
