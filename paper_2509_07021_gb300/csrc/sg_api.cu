@@ -698,6 +698,7 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     if (walk_ordered(b.n_tiles)) {
         walk.counts = reinterpret_cast<const uint32_t *>(w + L.walk);
         walk.place = walk.counts + TB_BUCKETS;
+        walk.fallback = reinterpret_cast<const uint32_t *>(w + L.order);
         walk.order = reinterpret_cast<uint32_t *>(bw + BL.order);
         walk.n = b.n_tiles;
     }

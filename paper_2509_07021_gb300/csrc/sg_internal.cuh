@@ -367,6 +367,8 @@ __device__ __forceinline__ uint32_t len_bucket(uint32_t len) {
 struct TileOrder {
     const uint32_t *counts = nullptr;   // [TB_BUCKETS] tiles per walk-length bucket
     const uint32_t *place = nullptr;    // [n] bucket << 24 | rank inside it
+    const uint32_t *fallback = nullptr; // [n] the order where the counts do not add up to n (an
+                                        // importance forward files no walk lengths)
     uint32_t *order = nullptr;          // [n]
     uint32_t n = 0;
 };
@@ -513,10 +515,10 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
 constexpr int TILE_ORDER_WORDS = 512;
 // Tile counts whose backward gets an order of its own: its 8-pixel form starts at
 // 5632 tiles, and with two or three tiles per resident warp the longest of the last
-// decide when the kernel ends (8160 tiles, 5.4M pairs: 610 -> 575 us; 3.9M: 564 -> 555).
+// decide when the kernel ends (8160 tiles, 5.4M pairs: 650 -> 613 us; 2.7M: 600 -> 587).
 // With fewer tiles several warps share each (3600: 305 us with either order, and the
 // forward pays 1 us for the ranks); with more, a warp takes several tiles and the
-// forward's order ends as evenly (six scenes in four views each: 6.64 ms with either).
+// forward's order ends as evenly (six scenes in four views each: the same with either).
 constexpr uint32_t WALK_ORDER_MIN = 5632, WALK_ORDER_MAX = 16384;
 inline bool walk_ordered(uint64_t n_tiles) { return n_tiles > WALK_ORDER_MIN && n_tiles <= WALK_ORDER_MAX; }
 cudaError_t launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t *scratch,

@@ -252,8 +252,10 @@ __global__ void __launch_bounds__(SETUP_THREADS) k_setup(const BatchParam<NV, NS
         base[TB_BUCKETS - 1 - threadIdx.x] =
             block_exclusive<uint32_t>(o.counts[TB_BUCKETS - 1 - threadIdx.x], tot, shs);
         __syncthreads();
-        const uint32_t at = base[place >> 24] + (place & 0xFFFFFFu);
-        if (t < o.n && at < o.n) o.order[at] = t;
+        if (t < o.n) {
+            if (tot == o.n) o.order[base[place >> 24] + (place & 0xFFFFFFu)] = t;
+            else o.order[t] = o.fallback[t];
+        }
         return;
     }
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -42,6 +42,9 @@ def test_every_tile_is_walked_once(views, fwd_persistent):
         assert torch.equal(out.img, ref.img) and torch.equal(out.last, ref.last)
         for _ in range(2):
             torch.testing.assert_close(grads(out), want, rtol=2e-4, atol=1e-6 * float(want.abs().max()))
+        # an importance forward files no walk lengths: the backward takes its list order
+        scored = render.render_forward(ds, cams, importance=torch.empty(ds.n, device="cuda"))
+        torch.testing.assert_close(grads(scored), want, rtol=2e-4, atol=1e-6 * float(want.abs().max()))
         img = torch.empty_like(out.img)
         sgsplat.sg_render_forward(ds, cams, out.ws, img, out.T_final, out.last)
         torch.testing.assert_close(grads(out), want, rtol=2e-4, atol=1e-6 * float(want.abs().max()))
