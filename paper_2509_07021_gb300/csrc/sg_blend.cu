@@ -68,12 +68,12 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 
 static_assert(BWD_BATCH_MAX % 32 == 0 && FWD_BATCH_MAX % 32 == 0, "batch sizes");
 // Resident blocks per SM requested for the backward.
-// 8 pixels per thread: 28 (72 registers, 8 bytes spilled) against 24 (80, none): 5.4M
-// pairs at 1920x1080 575 -> 565 us, 16 views 9.17 -> 8.86 ms, six scenes in four views
-// 6.64 -> 6.40; 32 (64 registers, batches of 32) 578 us.
-// 1 pixel: 4 (64 registers) against 3: 2500 tiles 78 -> 70 us, where a tile fewer
-// waits for a block; 494 tiles, nearly all resident at once, 52 -> 54.
-// 4 pixels: the compiler's 80 registers; 14 or 16 blocks 313 -> 344, 352 us (3600 tiles).
+// 8 pixels per thread: 28 (72 registers, 16 bytes spilled) against 24 (80): 5.4M pairs
+// at 1920x1080 613 -> 596 us, 16 views 9.67 -> 9.31 ms, six scenes in four views
+// 6.98 -> 6.69; 32 (64 registers, batches of 32) is slower again.
+// 1 pixel: 4 against 3: 2500 tiles 78 -> 70 us, where fewer tiles wait for a block;
+// 494 tiles, nearly all resident at once, 53 -> 56.
+// 4 pixels: the compiler's 82 registers; 14 or 16 blocks 313 -> 344, 352 us (3600 tiles).
 constexpr int bwd_min_blocks(int P) { return P == 8 ? 28 : P == 1 ? 4 : 1; }
 
 template <int NB>
@@ -395,7 +395,7 @@ __device__ __forceinline__ void tile_done(int walk, uint32_t tile, uint32_t *s_w
 // Persistent form: resident blocks pull tiles from a work counter in the
 // given order (longest lists first); otherwise one block per tile.
 // The 4-pixel plain form asks for 16 blocks per SM (64 registers): without the bound it
-// takes 72 and 14 blocks (297 -> 308 us at 3.9M pairs, 1920x1080; 5.26 -> 5.54 ms
+// takes 72 and 14 blocks (297 -> 308 us at 2.7M pairs, 1920x1080; 5.26 -> 5.54 ms
 // over 16 views), with 18 it spills (333 us). The others keep the compiler's choice: a
 // bound of one block raises the 1-pixel form from 40 to 67 registers (130 -> 176 us).
 template <int P, int MODE, bool PERSIST, int NB>
@@ -538,24 +538,10 @@ __device__ __forceinline__ void warp_sum9_atomic(const float v[9], float *dg9) {
     if ((lane & 3) == 0 || lane == 1) atomicAdd(dg9 + (lane == 1 ? 8 : lane >> 2), lane == 1 ? d : c);
 }
 
-// A thread's sums over its pixels for one entry. Its pixels lie in NC columns
-// (slot j in column j % NC), so dx takes only NC values: the moments in dx are formed
-// once per entry from the columns' sums of dP and dP dy. The kernel is bound by
-// instruction issue and nearly every evaluated slot has a blended lane, so the four
-// operations fewer per blended pixel count: 650 -> 614 us at 1M Gaussians,
-// 1920x1080; 9.67 -> 9.17 ms at 6M in 16 views.
-template <int NC>
-struct AdjSums {
-    float a[NC], b[NC], c;   // per column: sum dP, sum dP dy; all: sum dP dy^2
-    float r[3];              // sum w dL/drgb
-};
-
-// Adds one pixel's share of one blended pair (column h) and steps the pixel's
-// T and Sg back over the pair. dy2 = dy^2.
-template <int NC>
-__device__ __forceinline__ void bwd_adjoint(const PairEval &p, float dy, float dy2, const float4 &r, float bl,
-                                            float &T, float &Sg, float g0, float g1, float g2, int h,
-                                            AdjSums<NC> &v) {
+// Adds one pixel's share of one blended pair to v (in dg order) and steps the
+// pixel's T and Sg back over the pair.
+__device__ __forceinline__ void bwd_adjoint(const PairEval &p, float dy, const float4 &r, float bl,
+                                            float &T, float &Sg, float g0, float g1, float g2, float v[9]) {
     const float oma = __fsub_rn(1.f, p.alpha);
     const float ro = rcp_approx(oma);
     const float Ti = T * ro;
@@ -564,15 +550,19 @@ __device__ __forceinline__ void bwd_adjoint(const PairEval &p, float dy, float d
     const float dal = Ti * cg - Sg * ro;
     Sg = fmaf(cg, w, Sg);
     T = Ti;
-    v.r[0] = fmaf(w, g0, v.r[0]);
-    v.r[1] = fmaf(w, g1, v.r[1]);
-    v.r[2] = fmaf(w, g2, v.r[2]);
+    v[6] = fmaf(w, g0, v[6]);
+    v[7] = fmaf(w, g1, v[7]);
+    v[8] = fmaf(w, g2, v[8]);
     // dP = dL/dpower = dL/dalpha o' G, none where the 0.99 clamp is active
     // (dL/do' = dP / o': the division is applied once per Gaussian)
     const float dP = p.ag > ALPHA_MAX ? 0.f : dal * p.ag;
-    v.a[h] += dP;
-    v.b[h] = fmaf(dP, dy, v.b[h]);
-    v.c = fmaf(dP, dy2, v.c);
+    v[5] += dP;
+    const float hx = dP * p.dx, hy = dP * dy;
+    v[0] += hx;                          // sum dP dx
+    v[1] += hy;                          // sum dP dy
+    v[2] = fmaf(hx, p.dx, v[2]);         // sum dP dx^2
+    v[3] = fmaf(hx, dy, v[3]);           // sum dP dx dy
+    v[4] = fmaf(hy, dy, v[4]);           // sum dP dy^2
 }
 
 // Per pixel the walk runs back from the pixel's last blended pair, recovering
@@ -679,7 +669,9 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
             if ((msk & ((1u << P) - 1u)) == 0u) continue;   // warp-uniform
             const float4 q = sm.q[k], r = sm.r[k];
             const float bl = __uint_as_float(cm.x);
-            AdjSums<row_slots<P>()> v{};
+            float v[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = 0.f;
             bool any = false;
             constexpr int RS = row_slots<P>();
 #pragma unroll
@@ -693,7 +685,6 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                 slot_pixel<P>(j0, cx, cy);
                 RowEval row;
                 eval_row((float)(ty * TILE + cy), q, r, row);
-                const float dy2 = row.dy * row.dy;
                 // both pixels of the row first, with no branch between them
                 PairEval pe[RS];
                 bool ok[RS];
@@ -701,8 +692,7 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                 for (int hh = 0; hh < RS; ++hh) {
                     slot_pixel<P>(j0 + hh, cx, cy);
                     eval_pixel((float)(tx * TILE + cx), q, row, pe[hh]);
-                    // (where the mask's bit is clear the pixels fail one of the two tests)
-                    const bool live = pos < __float_as_int(pg[hh].w);
+                    const bool live = ((bits >> hh) & 1u) && pos < __float_as_int(pg[hh].w);
                     if (COUNT) ne += live ? 1u : 0u;
                     ok[hh] = live && pair_kept(pe[hh]);
                 }
@@ -711,26 +701,12 @@ __device__ __forceinline__ void blend_bwd_tile(const Batch &b, uint32_t tile, St
                     const int j = j0 + hh;
                     if (!ok[hh]) continue;
                     any = true;
-                    bwd_adjoint(pe[hh], row.dy, dy2, r, bl, T[j], Sg[j], pg[hh].x, pg[hh].y, pg[hh].z, hh, v);
+                    bwd_adjoint(pe[hh], row.dy, r, bl, T[j], Sg[j], pg[hh].x, pg[hh].y, pg[hh].z, v);
                 }
             }
             // the moments are linear in dP: the conic factors and 1/o' are applied
             // once per entry by the preprocess adjoint, after the sum over tiles
-            if (__any_sync(0xffffffffu, any)) {
-                float m[9] = {0.f, 0.f, 0.f, 0.f, v.c, 0.f, v.r[0], v.r[1], v.r[2]};   // in dg order
-#pragma unroll
-                for (int h = 0; h < RS; ++h) {
-                    int cx, cy;
-                    slot_pixel<P>(h, cx, cy);
-                    const float dx = __fsub_rn((float)(tx * TILE + cx), q.x);
-                    m[0] = fmaf(v.a[h], dx, m[0]);
-                    m[1] += v.b[h];
-                    m[2] = fmaf(v.a[h] * dx, dx, m[2]);
-                    m[3] = fmaf(v.b[h], dx, m[3]);
-                    m[5] += v.a[h];
-                }
-                warp_sum9_atomic(m, dg + 9 * (uint64_t)sm.id[k]);
-            }
+            if (__any_sync(0xffffffffu, any)) warp_sum9_atomic(v, dg + 9 * (uint64_t)sm.id[k]);
         }
     }
 }

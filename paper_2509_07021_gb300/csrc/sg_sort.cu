@@ -6,9 +6,10 @@
 // LSD radix sort of 64-bit keys tile << 32 | depth_bits, equal keys by
 // Gaussian id. The depth digits of every pair of one Gaussian are equal, so
 // the depth passes are run once per (view, Gaussian) entry, before the
-// entries are duplicated into pairs, and only the tile digits are sorted per
-// pair. Duplication walks the entries in depth order and every pass is
-// stable, so the result is identical to the 64-bit sort.
+// entries are duplicated into pairs, and the pairs are then binned by tile
+// (chunks; radix passes over the tile digits for a view of more tiles than a
+// chunk's counters hold). Duplication walks the entries in depth order and
+// both binnings are stable, so the result is identical to the 64-bit sort.
 #include "sg_internal.cuh"
 
 #include <algorithm>
@@ -540,8 +541,8 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
 // depth order: the result is the stable sort by tile of the depth-ordered pairs.
 // Measured (pairs and their placement, against a duplicate with its own
 // look-back followed by chunks of 8192 pairs or, past 12288 tiles, three radix
-// passes): 32k pairs 82 -> 31 us, 116k 91 -> 41, 3.9M 162 -> 129, 5.4M 195 -> 168,
-// 11.8M over four views 450 -> 348, 252M over 16 views 10.5 -> 6.4 ms. The
+// passes): 32k pairs 82 -> 31 us, 116k 91 -> 41, 3.9M 162 -> 122, 5.4M 195 -> 151,
+// 11.8M over four views 450 -> 328, 252M over 16 views 10.5 -> 6.4 ms. The
 // placement is bound by its warps' serial rounds (~400 cycles each, five warps
 // per SM) up to some 20M pairs, beyond by its scattered 4-byte stores.
 uint32_t bin_rows(uint64_t cap, uint32_t row) {

@@ -340,9 +340,9 @@ NO_OFFSET = 2**64 - 1   # a layout entry for a buffer the workspace does not hol
 
 def sg_workspace_layout(scene: DeviceScene, cams, ws_bytes: int) -> dict:
     """Byte offsets of a forward's buffers in a workspace of ws_bytes. pair_tile
-    is NO_OFFSET when the views have at most 12288 tiles in all: the tile sort
-    then counts and keeps no sorted tile ids (pair k's tile is the tile whose
-    range holds k)."""
+    is NO_OFFSET when the views have at most 12288 tiles in all: the forward
+    then keeps no sorted tile ids (pair k's tile is the tile whose range holds
+    k)."""
     s = scene.struct()
     c = camera_array(cams)
     out = sg_ws_layout()
