@@ -68,13 +68,16 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 
 static_assert(BWD_BATCH_MAX % 32 == 0 && FWD_BATCH_MAX % 32 == 0, "batch sizes");
 // Resident blocks per SM requested for the backward.
-// 8 pixels per thread: 28 (72 registers, 16 bytes spilled) against 24 (80): 5.4M pairs
-// at 1920x1080 613 -> 596 us, 16 views 9.67 -> 9.31 ms, six scenes in four views
-// 6.98 -> 6.69; 32 (64 registers, batches of 32) is slower again.
+// 8 pixels per thread: 24 (80 registers). 28 (72, 16 bytes spilled) measured 5.4M pairs at
+// 1920x1080 613 -> 596 us and six scenes in four views 6.98 -> 6.69 ms, but with other
+// tiles in flight an entry's sums over tiles meet in another order, and rotation gradients,
+// which magnify the last bit of these sums, came out further from their values than two
+// runs differ by (bit-equal sums, six scenes: 35.5 % of a scene's Gaussians between 28 and
+// 24 blocks, 36.7 % between two runs of 24).
 // 1 pixel: 4 against 3: 2500 tiles 78 -> 70 us, where fewer tiles wait for a block;
 // 494 tiles, nearly all resident at once, 53 -> 56.
 // 4 pixels: the compiler's 82 registers; 14 or 16 blocks 313 -> 344, 352 us (3600 tiles).
-constexpr int bwd_min_blocks(int P) { return P == 8 ? 28 : P == 1 ? 4 : 1; }
+constexpr int bwd_min_blocks(int P) { return P == 8 ? 24 : P == 1 ? 4 : 1; }
 
 template <int NB>
 struct StagedN {
