@@ -356,12 +356,18 @@ __global__ void __launch_bounds__(256) k_os_finish(const SortAux *aux, uint64_t 
     if (h[threadIdx.x]) atomicAdd(&bucket_counts[threadIdx.x], h[threadIdx.x]);
 }
 
-// Opts a kernel into `bytes` of dynamic shared memory on the current device
-// (beside a few KB of static; 48 KB in all need no opting in).
+// Opts a kernel into dynamic shared memory. The limit belongs to the function on its
+// device, not to the call: it is set to the most any call may ask for, never to this
+// call's size, so that no host thread lowers it between another's set and launch.
 template <typename K>
-static cudaError_t allow_smem(K kernel, size_t bytes) {
-    if (bytes <= 32 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+static cudaError_t allow_smem(K kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
+// A launch that was refused: the runtime's record of it is taken back as well.
+static cudaError_t refused(cudaError_t e) {
+    (void)cudaGetLastError();
+    return e;
 }
 
 // The whole depth sort of at most 1024 ITEMS keys in one block: the same stable
@@ -454,7 +460,7 @@ __global__ void __launch_bounds__(1024) k_depth_small(const uint32_t *__restrict
 template <int ITEMS>
 static cudaError_t depth_small(const Batch *db, const uint32_t *keys, uint32_t M, uint32_t *vout, SortAux *aux,
                                int passes, cudaStream_t s) {
-    const size_t smem = (size_t)(2 * 1024 * ITEMS + 32 * RS_RADIX) * 4;
+    constexpr size_t smem = (size_t)(2 * 1024 * ITEMS + 32 * RS_RADIX) * 4;
     const cudaError_t e = allow_smem(k_depth_small<ITEMS>, smem);
     if (e != cudaSuccess) return e;
     (void)launch_chain_smem(k_depth_small<ITEMS>, dim3(1), dim3(1024), smem, s, keys, M, vout, aux, db, passes);
@@ -480,20 +486,21 @@ cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32
     const bool grouped = nblocks <= 8u * 3u * 152u;
     const uint64_t pass_words = sort_flag_words(max_n, 1);
     const unsigned hgrid = nblocks < 4u * 152u ? nblocks : 4u * 152u;
-    (void)launch_chain(k_os_hist, dim3(hgrid), dim3(RS_THREADS), s, (const uint32_t *)k0, n_dev, max_n, aux, hist,
-                       pass_words * passes);
+    cudaError_t e = launch_chain(k_os_hist, dim3(hgrid), dim3(RS_THREADS), s, (const uint32_t *)k0, n_dev, max_n, aux,
+                                 hist, pass_words * passes);
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
-    for (int p = 0; p < passes; ++p) {
+    for (int p = 0; p < passes && e == cudaSuccess; ++p) {
         // pass 0 leaves SORT_DROP_KEY out and later passes see only the kept keys
-        (void)launch_chain(grouped ? k_os_pass<true> : k_os_pass<false>, dim3(nblocks), dim3(RS_THREADS), s,
-                           (const uint32_t *)ki, p > 0 ? (const uint32_t *)vi : (const uint32_t *)nullptr, ko, vo,
-                           p > 0 ? (const uint64_t *)&aux->kept : n_dev, max_n, p, 8 * p, 255u, p == 0,
-                           hist + pass_words * p, aux, (uint2 *)nullptr, (uint64_t)0, sort_wait_polls(),
-                           (const uint64_t *)nullptr, p == VIEW_PASS ? db : (const Batch *)nullptr,
-                           hist + pass_words * p + (uint64_t)nblocks * RS_RADIX);
+        e = launch_chain(grouped ? k_os_pass<true> : k_os_pass<false>, dim3(nblocks), dim3(RS_THREADS), s,
+                         (const uint32_t *)ki, p > 0 ? (const uint32_t *)vi : (const uint32_t *)nullptr, ko, vo,
+                         p > 0 ? (const uint64_t *)&aux->kept : n_dev, max_n, p, 8 * p, 255u, p == 0,
+                         hist + pass_words * p, aux, (uint2 *)nullptr, (uint64_t)0, sort_wait_polls(),
+                         (const uint64_t *)nullptr, p == VIEW_PASS ? db : (const Batch *)nullptr,
+                         hist + pass_words * p + (uint64_t)nblocks * RS_RADIX);
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
+    if (e != cudaSuccess) return refused(e);
     count_launches(1 + passes);
     return cudaGetLastError();
 }
@@ -507,17 +514,19 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
     if (max_n > SORT_MAX_KEYS) return cudaErrorInvalidValue;
     const uint64_t pass_words = sort_flag_words(max_n, 1);
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
-    for (int p = 0; p < passes; ++p) {
+    cudaError_t e = cudaSuccess;
+    for (int p = 0; p < passes && e == cudaSuccess; ++p) {
         const int shift = 8 * p;
         const uint32_t mask = (1u << std::min(8, bits - shift)) - 1u;
-        (void)launch_chain(k_os_pass<false>, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki, (const uint32_t *)vi,
-                           ko, vo, (const uint64_t *)(counters + CNT_WRITTEN), max_n, p, shift, mask, false,
-                           hist + pass_words * p, aux, p == passes - 1 ? ranges : (uint2 *)nullptr, n_ranges,
-                           sort_wait_polls(), (const uint64_t *)(counters + CNT_STATUS), (const Batch *)nullptr,
-                           (uint32_t *)nullptr);
+        e = launch_chain(k_os_pass<false>, dim3(nblocks), dim3(RS_THREADS), s, (const uint32_t *)ki,
+                         (const uint32_t *)vi, ko, vo, (const uint64_t *)(counters + CNT_WRITTEN), max_n, p, shift,
+                         mask, false, hist + pass_words * p, aux, p == passes - 1 ? ranges : (uint2 *)nullptr,
+                         n_ranges, sort_wait_polls(), (const uint64_t *)(counters + CNT_STATUS),
+                         (const Batch *)nullptr, (uint32_t *)nullptr);
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
+    if (e != cudaSuccess) return refused(e);
     (void)launch_chain(k_os_finish, dim3((unsigned)std::max<uint64_t>(div_up(n_ranges, 256), 1)), dim3(256), s,
                        (const SortAux *)aux, counters, ranges, n_ranges, bits == 0, max_n, status_mirror,
                        order_counts);
@@ -968,7 +977,7 @@ cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
         a.max_chunks > BIN_MAX_CHUNKS || a.cap > SORT_MAX_KEYS)
         return cudaErrorInvalidValue;
     const size_t smem = (size_t)a.row * 4;
-    const cudaError_t e = allow_smem(k_bin_emit, smem);
+    cudaError_t e = allow_smem(k_bin_emit, BIN_MAX_ROW * 4);
     if (e != cudaSuccess) return e;
     // larger blocks shorten the look-back over many entries (1M: 20 -> 14 us) but
     // cost the short ones 2 us
@@ -977,7 +986,8 @@ cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
     // how many of the M entries are in the order is only known on the device
     const uint64_t cut = std::min<uint64_t>(std::max<uint64_t>(div_up(a.M, cut_threads * BIN_ITEMS), 1),
                                             2 * 152 * (1024 / cut_threads));
-    (void)launch_chain(k_bin_cut, dim3((unsigned)cut), dim3(cut_threads), s, a, sort_wait_polls());
+    e = launch_chain(k_bin_cut, dim3((unsigned)cut), dim3(cut_threads), s, a, sort_wait_polls());
+    if (e != cudaSuccess) return refused(e);
     (void)launch_chain_smem(k_bin_emit, dim3(a.max_chunks), dim3(256), smem, s, a);
     count_launches(2);
     return cudaGetLastError();
@@ -985,9 +995,10 @@ cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
 
 cudaError_t launch_bin_place(const BinArgs &a, cudaStream_t s) {
     const size_t smem = (size_t)a.row * 4;
-    const size_t scan_smem = (size_t)div_up(a.max_chunks, BIN_SCAN_WARPS) * BIN_SCAN_WARPS * 32 * 4;
-    cudaError_t e = allow_smem(k_bin_place, smem);
-    if (e == cudaSuccess) e = allow_smem(k_bin_scan, scan_smem);
+    auto scan_bytes = [](uint32_t chunks) { return (size_t)div_up(chunks, BIN_SCAN_WARPS) * BIN_SCAN_WARPS * 32 * 4; };
+    const size_t scan_smem = scan_bytes(a.max_chunks);
+    cudaError_t e = allow_smem(k_bin_place, BIN_MAX_ROW * 4);
+    if (e == cudaSuccess) e = allow_smem(k_bin_scan, scan_bytes(BIN_MAX_CHUNKS));
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -996,8 +1007,10 @@ cudaError_t launch_bin_place(const BinArgs &a, cudaStream_t s) {
     // (two 1024-thread blocks fill an SM's threads; shared memory decides)
     per_sm = scan_smem <= 100 * 1024 ? 2 : 1;
     const unsigned grid = std::min(a.n_groups, (uint32_t)(sms * per_sm));
-    (void)launch_chain_smem(k_bin_scan, dim3(grid), dim3(BIN_SCAN_WARPS * 32), scan_smem, s, a, sort_wait_polls());
-    (void)launch_chain_smem(k_bin_place, dim3(a.max_chunks), dim3(32), smem, s, a);
+    e = launch_chain_smem(k_bin_scan, dim3(grid), dim3(BIN_SCAN_WARPS * 32), scan_smem, s, a, sort_wait_polls());
+    if (e != cudaSuccess) return refused(e);   // an unscanned matrix holds no positions
+    e = launch_chain_smem(k_bin_place, dim3(a.max_chunks), dim3(32), smem, s, a);
+    if (e != cudaSuccess) return refused(e);
     count_launches(2);
     if (a.okeys) {
         (void)launch_chain(k_bin_keys, dim3(std::min(div_up(a.n_tiles, 8), (uint64_t)(sms * 8))), dim3(256), s,
