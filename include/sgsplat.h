@@ -152,7 +152,8 @@ typedef struct sg_sizes {
     uint64_t n_pairs;          /* (tile, Gaussian) pairs of the last forward */
     uint64_t pair_capacity;    /* pairs the queried workspace holds */
     uint64_t ws_fixed_bytes;   /* forward workspace part independent of pairs */
-    uint64_t ws_per_pair_bytes;/* forward workspace bytes per pair of capacity */
+    uint64_t ws_per_pair_bytes;/* forward workspace bytes per pair of capacity, at most: fixed +
+                                  per pair x pairs holds that many */
     uint64_t ws_bytes;         /* forward workspace for pair_capacity */
     uint64_t bwd_ws_bytes;     /* backward scratch */
 } sg_sizes;
@@ -176,7 +177,7 @@ typedef struct sg_sizes {
  *   rect          [M] 2 x uint32: x0 | x1 << 16, y0 | y1 << 16 (tiles, half
  *                 open; the 3-sigma rectangle; empty = culled)
  *   depth_order   [M] uint32: the entries with tiles_touched > 0 sorted by
- *                 (depth bits, entry), first. Scratch of the forward: its
+ *                 (view, depth bits, entry), first. Scratch of the forward: its
  *                 memory is reused by the tile sort, so a finished forward no
  *                 longer holds it.
  *   ranges        [n_tiles] 2 x uint32 [start, end) into the pair arrays
@@ -321,6 +322,7 @@ int sg_workspace_query(const sg_scene *scene, const sg_camera *cams, int n_views
  *   unmodified. The copy goes to 64 bytes of pinned host memory that each
  *   calling thread allocates once.
  * img: device [n_views] x [3][H][W] binary32, views packed one after another.
+ *   Its memory also serves the sorts as scratch until the blend writes every pixel.
  * T_final: device [n_views] x [H][W] binary32, transmittance after the walk.
  * last: device [n_views] x [H][W] int32, 1 + position (inside the pixel's
  *   tile list) of the last blended Gaussian, 0 if none.

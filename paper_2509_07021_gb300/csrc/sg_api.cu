@@ -218,7 +218,6 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
         d.tiles_x = (c.width + TILE - 1) / TILE;
         d.tiles_y = (c.height + TILE - 1) / TILE;
         d.scene = s;
-        d.n = (int32_t)scenes[s].n;
         d.tile_off = (uint32_t)tiles;
         d.grp_off = (uint32_t)groups;
         groups += div_up((uint64_t)d.tiles_x * d.tiles_y, 32);
@@ -257,6 +256,12 @@ constexpr uint64_t kNoKeyTiles = 12288;
 // Pairs per row of the binning's count matrix that the per-pair size reports.
 constexpr uint64_t kMatrixShare = 8192;
 
+// The workspace holds what the forward leaves for the backward and the pairs. What only the
+// sorts need, the depth sort's look-back flags and the binning's count matrix, lives in the
+// image, which the blend writes after the placement has read the last count (12 bytes per
+// pixel hold 760 rows of a counter per tile, fewer where the frame's edge cuts many tiles).
+// Regions that follow cap hold a rounding unit at least: fixed + per pair x pairs bounds
+// the total.
 WsLayout make_layout(const Batch &b, uint64_t cap) {
     WsLayout L{};
     const uint64_t M = b.n_entries, T = b.n_tiles;
@@ -269,7 +274,11 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
     // chunks where one chunk's counters of the largest view fit shared memory
     L.chunked = row <= BIN_MAX_ROW;
     L.bin_row = (uint32_t)row;
-    L.bin_chunks = L.chunked ? bin_chunks(cap, L.bin_row) : 0u;
+    const uint64_t img_rows = 3 * n_pixels_of(b) / row, own_rows = (uint64_t)b.n_views + 1;
+    L.matrix_in_img = img_rows >= own_rows;
+    if (L.chunked)
+        L.bin_chunks = (uint32_t)std::min<uint64_t>(bin_chunks(cap, L.bin_row, b.n_views),
+                                                    L.matrix_in_img ? img_rows : own_rows);
     L.batch = take(sizeof(Batch));
     L.counters = take(CNT_N * sizeof(uint64_t));
     L.rec = take(M * sizeof(Rec));
@@ -279,14 +288,12 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
     L.dup_flags = take(div_up(M, 256) * 8 + 8);   // look-back words of the chunk cutter / the duplicate
     L.ranges = take(T * 8);
     L.order = take(T * 4);   // tile order of the persistent blends (by list length)
-    // the forward's tile order: its counts and cursors; the backward's: its counts,
-    // then each tile's place (see TileOrder)
+    // the forward's tile order: its counts and cursors; the backward's: its counts
     L.order_scratch = take((TILE_ORDER_WORDS + TB_BUCKETS) * 4);
-    L.walk = L.order_scratch + TILE_ORDER_WORDS * 4;
-    take(walk_ordered(T) ? 4 * T : 0);
     L.bin = take(sizeof(BinTab));
+    const uint64_t cuts = std::min<uint64_t>(BIN_MAX_CHUNKS, b.n_views + std::max<uint64_t>(cap / BIN_MIN_CHUNK, 1)) + 1;
+    L.bin_start = take(L.chunked ? 8 * cuts + ALIGN : 0);   // first entries, then first pairs
     L.scan_words = take(8 * (1 + (uint64_t)b.n_groups));
-    L.fixed_end = o;
     L.tile_bits = tile_bits_for(T);
     L.tile_passes = L.chunked ? 0 : radix_passes(L.tile_bits);
     const bool keys = T > kNoKeyTiles;   // the layout keeps the sorted tile ids
@@ -294,10 +301,14 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
     // placed ones (radix passes alternate between the two). The depth sort's
     // four buffers live in B: B is first written by the placement, after
     // the pairs' kernel has read the depth order. The backward reads only the final
-    // entries (chunked: B; radix: A after an even number of passes, B after an odd one).
-    const size_t pairs4 = al(cap * 4), m4 = al(M * 4);
-    const size_t A = take(keys ? 2 * pairs4 : al(cap * 2) + pairs4);
-    const size_t B = take(std::max((keys ? 2 : 1) * pairs4, 4 * m4));
+    // entries (chunked: B; radix: A after an even number of passes, B after an odd one)
+    // and, chunked, the tiles' places by walk length, which take A after the placement.
+    const size_t pairs4 = al(cap * 4), m4 = al(M * 4), unit = 2 * ALIGN;
+    const size_t a_bytes = std::max(keys ? 2 * pairs4 : al(cap * 2) + pairs4, unit);
+    const size_t B = take(std::max({(keys ? 2 : 1) * pairs4, 4 * m4, unit}));
+    const size_t A = take(a_bytes);
+    L.walk = L.chunked && walk_ordered(T) && 4 * T <= a_bytes;
+    L.walk_place = A;
     L.dkey0 = B;
     L.dval0 = B + m4;
     L.dkey1 = B + 2 * m4;
@@ -314,14 +325,16 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
         L.pkey_tmp = tmp;
         L.pval_tmp = tmp + pairs4;
     }
-    // look-back flags of the depth sort's passes (one more with several views),
-    // then the binning's count matrix or the flags of the tile sort's radix passes
-    const uint64_t tile_words = L.chunked ? (uint64_t)bin_rows(cap, L.bin_row) * L.bin_row
-                                          : sort_flag_words(cap, L.tile_passes);
-    const uint64_t flag_words = std::max<uint64_t>(sort_flag_words(M, b.n_views > 1 ? 5 : 4), tile_words);
-    L.hist = take(flag_words * 4);
-    L.aux_depth = take(SORT_AUX_BYTES);
-    L.aux_tile = take(SORT_AUX_BYTES);
+    // look-back flags of the depth sort's passes (one more with several views), where the
+    // image cannot hold them, then those of the tile sort's radix passes (chunked: the
+    // count matrix of a frame that cannot hold it)
+    const uint64_t depth_words = depth_flag_words(M, b.n_views > 1 ? 5 : 4);
+    L.depth_in_img = depth_words <= 3 * n_pixels_of(b);
+    const uint64_t tile_words = !L.chunked ? sort_flag_words(std::max<uint64_t>(cap, 1), L.tile_passes)
+                                           : L.matrix_in_img ? 0 : own_rows * row;
+    L.hist = take(std::max<uint64_t>(L.depth_in_img ? 0 : depth_words, tile_words) * 4);
+    L.aux_depth = take(sizeof(SortAux));
+    L.aux_tile = take(L.chunked ? 0 : sizeof(SortAux));
     L.total = o;
     L.M = M;
     L.n_tiles = T;
@@ -404,10 +417,11 @@ void fill_sizes(const Batch &b, const WsLayout &L, uint64_t n_pairs, sg_sizes *o
     out->n_pairs = n_pairs;
     out->pair_capacity = L.cap;
     out->ws_fixed_bytes = make_layout(b, 0).total;
-    // pair buffers (16-bit tile ids and entries, then the placed entries; with
-    // sorted tile ids kept, 32-bit ids and entries twice), plus a share of the
-    // count matrix or of the radix passes' look-back words
-    out->ws_per_pair_bytes = b.n_tiles > kNoKeyTiles ? 17 : 10 + div_up(4 * (uint64_t)L.bin_row, kMatrixShare);
+    // at most: pair buffers (16-bit tile ids and entries, then the placed entries: 10; with
+    // sorted tile ids kept, 32-bit ids and entries twice: 16), with room for a share of the
+    // count matrix, or for the radix passes' look-back words (a third of a byte a pass)
+    out->ws_per_pair_bytes = b.n_tiles > kNoKeyTiles ? 17 + (L.tile_passes > 3 ? 1 : 0)
+                                                     : 10 + div_up(4 * (uint64_t)L.bin_row, kMatrixShare);
     out->ws_bytes = L.total;
     out->bwd_ws_bytes = bwd_bytes(b);
 }
@@ -533,8 +547,8 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
     {
         // once per entry; entries that reach no tile are left out of the order
         StageTimer t(ST_DEPTH_SORT, stream);
-        SG_CUDA(launch_depth_sort(db, n_views, dkey0, dval0, dkey1, dval1, counters + CNT_ENTRIES, M, hist, aux_depth,
-                                  stream),
+        SG_CUDA(launch_depth_sort(db, n_views, dkey0, dval0, dkey1, dval1, counters + CNT_ENTRIES, M,
+                                  L.depth_in_img ? reinterpret_cast<uint32_t *>(img) : hist, aux_depth, stream),
                 "depth sort");
     }
     const uint32_t *order = n_views > 1 ? dval1 : dval0;   // entries by (view, depth)
@@ -565,11 +579,13 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
         a.rec = rec;
         a.counters = counters;
         a.tab = tab;
+        a.start = reinterpret_cast<uint32_t *>(w + L.bin_start);
+        a.pair = a.start + L.bin_chunks + 1;
         a.poff = dkey1;   // the depth keys are no longer needed
         a.flags = dup_flags;
         a.pkey = reinterpret_cast<uint16_t *>(pk_tmp);
         a.pval = pv_tmp;
-        a.matrix = hist;
+        a.matrix = L.matrix_in_img ? reinterpret_cast<uint32_t *>(img) : hist;
         a.words = reinterpret_cast<uint64_t *>(w + L.scan_words);
         a.ranges = ranges;
         a.order_counts = order_counts;
@@ -608,7 +624,10 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
                      reinterpret_cast<uint32_t *>(counters + CNT_QUEUE), shape);
     if (st != SG_OK) return st;
     shape.status = counters + CNT_STATUS;
-    if (walk_ordered(b.n_tiles)) shape.walk_counts = reinterpret_cast<uint32_t *>(w + L.walk);
+    if (L.walk) {
+        shape.walk_counts = order_counts + TILE_ORDER_WORDS;
+        shape.walk_place = reinterpret_cast<uint32_t *>(w + L.walk_place);
+    }
     shape.importance = want_importance && !counting;
     if (shape.importance)
         for (int s = 0; s < n_scenes; ++s)
@@ -695,9 +714,9 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     // is only its bound (a list's tail lies behind stopped pixels). With two or three
     // tiles per resident warp the last ones to start decide when the kernel ends.
     TileOrder walk;
-    if (walk_ordered(b.n_tiles)) {
-        walk.counts = reinterpret_cast<const uint32_t *>(w + L.walk);
-        walk.place = walk.counts + TB_BUCKETS;
+    if (L.walk) {
+        walk.counts = reinterpret_cast<const uint32_t *>(w + L.order_scratch) + TILE_ORDER_WORDS;
+        walk.place = reinterpret_cast<const uint32_t *>(w + L.walk_place);
         walk.fallback = reinterpret_cast<const uint32_t *>(w + L.order);
         walk.order = reinterpret_cast<uint32_t *>(bw + BL.order);
         walk.n = b.n_tiles;

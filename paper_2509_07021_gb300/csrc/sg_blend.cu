@@ -279,7 +279,7 @@ __device__ __forceinline__ int blend_fwd_tile(const Batch &b, uint32_t tile, Sta
             }
             // only an entry of this view's scene (a stale id from another view is left out)
             const uint32_t li = sm.id[k] - (uint32_t)vw->ent_off;
-            if (sum != 0.f && li < (uint32_t)vw->n) atomicAdd(imp + li, sum);
+            if (sum != 0.f && li < (uint32_t)b.scene[vw->scene].n) atomicAdd(imp + li, sum);
         }
         pending = 0;
     };
@@ -379,7 +379,7 @@ __device__ __forceinline__ int blend_fwd_tile(const Batch &b, uint32_t tile, Sta
 // a barrier lies between a block's tiles.
 template <int NW>
 __device__ __forceinline__ void tile_done(int walk, uint32_t tile, uint32_t *s_walk, uint32_t *s_arrived,
-                                          uint32_t *counts) {
+                                          uint32_t *counts, uint32_t *place) {
     if (counts == nullptr) return;
     walk = __reduce_max_sync(0xffffffffu, walk);
     if ((threadIdx.x & 31) != 0) return;
@@ -392,7 +392,7 @@ __device__ __forceinline__ void tile_done(int walk, uint32_t tile, uint32_t *s_w
         *s_arrived = 0u;
     }
     const uint32_t bucket = len_bucket(len);
-    counts[TB_BUCKETS + tile] = bucket << 24 | atomicAdd(&counts[bucket], 1u);
+    place[tile] = bucket << 24 | atomicAdd(&counts[bucket], 1u);
 }
 
 // Persistent form: resident blocks pull tiles from a work counter in the
@@ -408,7 +408,7 @@ k_blend_fwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
             float *__restrict__ img, float *__restrict__ T_final, int32_t *__restrict__ last,
             const uint32_t *__restrict__ tile_order, uint32_t *__restrict__ queue, uint32_t n_tiles,
             unsigned long long *__restrict__ evals, const uint64_t *__restrict__ status,
-            uint32_t *__restrict__ walk_counts) {
+            uint32_t *__restrict__ walk_counts, uint32_t *__restrict__ walk_place) {
     chain_enter();
     __shared__ StagedN<NB> sm;
     __shared__ float part[MODE == FWD_IMPORTANCE ? (BLEND_THREADS / P) * (NB + 1) : 1];
@@ -426,7 +426,7 @@ k_blend_fwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
     if (!PERSIST) {
         const int walk = blend_fwd_tile<P, MODE, NB>(b, blockIdx.x, sm, ranges, pval, rec, img, T_final, last, ne,
                                                      lists_ok, part);
-        if (MODE != FWD_IMPORTANCE) tile_done<NW>(walk, blockIdx.x, &s_walk, &s_arrived, walk_counts);
+        if (MODE != FWD_IMPORTANCE) tile_done<NW>(walk, blockIdx.x, &s_walk, &s_arrived, walk_counts, walk_place);
     } else {
         for (;;) {
             if (threadIdx.x == 0) s_item = atomicAdd(queue, 1u);
@@ -439,7 +439,7 @@ k_blend_fwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
                                                          lists_ok, part);
             // from shared memory: no register holds the tile across the walk (the next
             // item overwrites s_tile only after a barrier that every warp has passed)
-            if (MODE != FWD_IMPORTANCE) tile_done<NW>(walk, s_tile, &s_walk, &s_arrived, walk_counts);
+            if (MODE != FWD_IMPORTANCE) tile_done<NW>(walk, s_tile, &s_walk, &s_arrived, walk_counts, walk_place);
         }
     }
     if (MODE == FWD_COUNT) add_evals(ne, evals);
@@ -452,7 +452,7 @@ static void fwd_launch(const Batch *db, uint32_t n_tiles, const uint2 *ranges, c
     const unsigned grid = PERSIST ? (unsigned)sh.grid : n_tiles;
     (void)launch_chain(k_blend_fwd<P, MODE, PERSIST, NB>, dim3(grid), dim3(BLEND_THREADS / P), s,
         db, ranges, pval, rec, img, T_final, last, sh.tile_order, sh.queue, n_tiles, evals, sh.status,
-        sh.walk_counts);
+        sh.walk_counts, sh.walk_place);
 }
 
 // The plain forward takes the batch size of the tuning; the counting form

@@ -27,11 +27,9 @@ struct ViewDesc {
     float bg[3];
     int32_t W, H, tiles_x, tiles_y;
     int32_t scene;        // index into Batch::scene
-    int32_t n;            // Gaussians of that scene
     uint32_t tile_off;    // first global tile id of the view
     uint32_t grp_off;     // first group of 32 tiles of the view (the binning's scan)
     float limx, limy;     // guard band: 1.3 tan(fov / 2) per axis
-    uint32_t pad0;
     uint64_t pix_off;     // first pixel of the view in T_final / last (img: x3)
     uint64_t ent_off;     // first (view, Gaussian) entry of the view
 };
@@ -98,12 +96,15 @@ constexpr int RS_RADIX = 256;
 // forward and the backward of one call).
 struct WsLayout {
     size_t batch, counters, rec, tiles_touched, rect, clamp, dkey0, dval0, dkey1, dval1,
-        dup_flags, ranges, order, order_scratch, walk, bin, scan_words, hist, aux_depth, aux_tile, fixed_end;
+        dup_flags, ranges, order, order_scratch, walk_place, bin, bin_start, scan_words, hist, aux_depth, aux_tile;
     size_t pval_final, pkey_final, pval_tmp, pkey_tmp, total;
     uint64_t M, n_tiles, cap;
     int tile_bits, tile_passes;
-    bool chunked;         // tile sort by chunks (launch_bin) instead of radix passes
-    uint32_t bin_chunks;  // most chunks; their count matrix takes the look-back flags' region
+    bool chunked;         // tile sort by chunks (launch_bin_pairs) instead of radix passes
+    bool matrix_in_img;   // the count matrix takes the image's memory (else hist's)
+    bool depth_in_img;    // so do, before it, the depth sort's look-back flags
+    bool walk;            // the forward files walk lengths for the backward's tile order
+    uint32_t bin_chunks;  // most chunks: rows of the matrix
     uint32_t bin_row;     // words per row of the matrix: the largest view's tiles, padded to 4
 };
 
@@ -393,7 +394,6 @@ cudaError_t launch_preprocess_backward(const Batch &hb, const Batch *db,
                                        const uint32_t *tiles_touched, const uint8_t *clamp, const float *dg,
                                        uint64_t M, cudaStream_t s);
 
-constexpr size_t SORT_AUX_BYTES = 16384;
 // Most keys one sort takes (its look-back words carry 30-bit counts).
 constexpr uint64_t SORT_MAX_KEYS = (1ull << 30) - 1;
 constexpr uint32_t SORT_DROP_KEY = 0xFFFFFFFFu;
@@ -402,8 +402,10 @@ int radix_passes(int bits);
 // up and records SG_ERR_TIMEOUT (0: the default, 2^20).
 void set_sort_wait_polls(uint32_t polls);
 uint32_t sort_wait_polls();
-// Look-back flag words of `passes` passes over up to max_n keys.
+// Look-back flag words of `passes` passes over up to max_n keys (of the depth sort: with
+// the group words of its grouped look-back).
 uint64_t sort_flag_words(uint64_t max_n, int passes);
+uint64_t depth_flag_words(uint64_t max_n, int passes);
 
 // Stable sort of the entries by (view, depth bits), entries whose key in k0 is
 // SORT_DROP_KEY left out (k0: one key per entry; the values, entry indices, are
@@ -418,7 +420,6 @@ struct SortAux {
     uint32_t status;              // 0 or SG_ERR_TIMEOUT
     uint64_t kept;                // keys other than SORT_DROP_KEY (drop mode)
 };
-static_assert(sizeof(SortAux) <= SORT_AUX_BYTES, "sort aux region");
 cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
                               const uint64_t *n_dev, uint64_t max_n, uint32_t *hist, SortAux *aux, cudaStream_t s);
 
@@ -443,11 +444,8 @@ struct BinTab {
     unsigned long long view_pairs[SG_MAX_VIEWS];   // pairs of each view (preprocess)
     uint32_t n_chunks;                             // chunks in use
     uint32_t first_chunk[SG_MAX_VIEWS + 1];        // first chunk of each view
-    uint32_t start[BIN_MAX_CHUNKS + 1];            // first entry (depth order) of each chunk
-    uint32_t pair[BIN_MAX_CHUNKS + 1];             // first pair of each chunk
 };
-uint32_t bin_rows(uint64_t cap, uint32_t row);     // rows of the count matrix of a call with room for cap pairs
-uint32_t bin_chunks(uint64_t cap, uint32_t row);   // and the most chunks it uses
+uint32_t bin_chunks(uint64_t cap, uint32_t row, int n_views);   // most chunks of a call with room for cap pairs
 struct BinArgs {
     const Batch *db;
     int n_views;
@@ -460,11 +458,12 @@ struct BinArgs {
     const Rec *rec;
     uint64_t *counters;
     BinTab *tab;
+    uint32_t *start, *pair;          // max_chunks + 1 each: first entry (depth order) and first pair of a chunk
     uint32_t *poff;                  // scratch, M words: first pair of each entry of the order
     uint64_t *flags;                 // zeroed, a word per 256 entries (at most that many used): look-back
     uint16_t *pkey;                  // depth-ordered pairs: tile inside the view
     uint32_t *pval;                  //   and entry
-    uint32_t *matrix;                // max_chunks x row words
+    uint32_t *matrix;                // max_chunks x row words, 16-byte aligned
     uint64_t *words;                 // zeroed, 1 + n_groups: ticket and look-back of the scan
     uint2 *ranges;                   // every tile's [first, last + 1) ((0, 0): none)
     uint32_t *order_counts;          // zeroed tile-order bucket counts
@@ -533,8 +532,8 @@ struct BlendShape {
     int grid;                     // persistent: resident blocks
     bool importance;              // forward: accumulate SceneDesc::importance
     const uint64_t *status;       // the forward's status word: SG_ERR_TIMEOUT = lists unusable
-    uint32_t *walk_counts;        // forward: TileOrder::counts (zeroed), then ::place, for the backward's
-                                  // tile order (null: none wanted)
+    uint32_t *walk_counts;        // forward: TileOrder::counts (zeroed) and ::place, for the backward's
+    uint32_t *walk_place;         // tile order (null: none wanted)
     int batch;                    // Gaussians staged per shared-memory batch
 };
 

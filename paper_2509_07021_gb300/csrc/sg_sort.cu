@@ -314,7 +314,11 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_os_pass(
 int radix_passes(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
 
 uint64_t sort_flag_words(uint64_t max_n, int passes) {
-    const uint64_t tiles = div_up(max_n, RS_TILE);   // a word per tile and digit, and per group of tiles
+    return div_up(max_n, RS_TILE) * RS_RADIX * (uint64_t)passes;   // a word per tile and digit
+}
+
+uint64_t depth_flag_words(uint64_t max_n, int passes) {
+    const uint64_t tiles = div_up(max_n, RS_TILE);   // and a word per group of tiles and digit
     return (tiles + div_up(tiles, LB_WINDOW)) * RS_RADIX * (uint64_t)passes;
 }
 
@@ -484,7 +488,7 @@ cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32
     // Grouped look-back where the kept keys' tiles may all be resident at once
     // (three per SM) or not far more; beyond, inclusive prefixes are found near by.
     const bool grouped = nblocks <= 8u * 3u * 152u;
-    const uint64_t pass_words = sort_flag_words(max_n, 1);
+    const uint64_t pass_words = depth_flag_words(max_n, 1);
     const unsigned hgrid = nblocks < 4u * 152u ? nblocks : 4u * 152u;
     cudaError_t e = launch_chain(k_os_hist, dim3(hgrid), dim3(RS_THREADS), s, (const uint32_t *)k0, n_dev, max_n, aux,
                                  hist, pass_words * passes);
@@ -554,20 +558,18 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
 // 11.8M over four views 450 -> 328, 252M over 16 views 10.5 -> 6.4 ms. The
 // placement is bound by its warps' serial rounds (~400 cycles each, five warps
 // per SM) up to some 20M pairs, beyond by its scattered 4-byte stores.
-uint32_t bin_rows(uint64_t cap, uint32_t row) {
+uint32_t bin_chunks(uint64_t cap, uint32_t row, int n_views) {
     // Resident placing blocks, each holding one row of cursors in shared memory:
     // five one-warp blocks per SM, four below 1M pairs (a smaller matrix). More
     // place no faster and cost the matrix's scan (4 / 5 / 6 per SM: emission, scan and
     // placement 155 / 151 / 164 us at 5.4M pairs, 125 / 122 / 129 at 3.9M).
-    const uint32_t want = cap > (1u << 20) ? 5u : 4u;
-    return 152u * std::max(std::min(want, (227u * 1024u) / (row * 4u + 1024u)), 1u);
-}
-
-uint32_t bin_chunks(uint64_t cap, uint32_t row) {
     // Past 16M pairs the chunks' open output sectors (chunks x tiles x 32 bytes,
     // over every view) no longer fit L2: four per SM place faster (252M pairs:
     // eight 5.0 ms, four 3.8).
-    return std::min(bin_rows(cap, row), cap > (16u << 20) ? 4u * 152u : BIN_MAX_CHUNKS);
+    const uint32_t want = cap > (1u << 20) && cap <= (16u << 20) ? 5u : 4u;
+    const uint64_t fit = 152u * std::max(std::min(want, (227u * 1024u) / (row * 4u + 1024u)), 1u);
+    // one chunk a view, and another for every BIN_MIN_CHUNK pairs: no more are cut
+    return (uint32_t)std::min<uint64_t>(fit, (uint64_t)n_views + std::max<uint64_t>(cap / BIN_MIN_CHUNK, 1));
 }
 
 __device__ __forceinline__ uint32_t bin_view_of_chunk(const BinTab &tab, int n_views, uint32_t c) {
@@ -639,13 +641,13 @@ __global__ void __launch_bounds__(BIN_CUT_THREADS) k_bin_cut(BinArgs a, uint32_t
         if (tid == 0) {
             t.n_chunks = total_chunks;
             t.first_chunk[a.n_views] = total_chunks;
-            t.start[total_chunks] = (uint32_t)V;
-            t.pair[total_chunks] = (uint32_t)K;
+            a.start[total_chunks] = (uint32_t)V;
+            a.pair[total_chunks] = (uint32_t)K;
             // chunks whose threshold is 0: the first view's first chunk, and
             // every chunk of the views before the first entry
             for (int v = 0; v < a.n_views && s_base[v] == 0u; ++v) {
                 const uint32_t last = s_base[v + 1] == 0u ? s_first[v + 1] : s_first[v] + 1u;
-                for (uint32_t c = s_first[v]; c < last; ++c) t.start[c] = t.pair[c] = 0u;
+                for (uint32_t c = s_first[v]; c < last; ++c) a.start[c] = a.pair[c] = 0u;
             }
         }
     }
@@ -706,15 +708,15 @@ __global__ void __launch_bounds__(BIN_CUT_THREADS) k_bin_cut(BinArgs a, uint32_t
             const bool last = x1 == s_base[v + 1];
             if (last) q1 = vc - 1u;   // thresholds past the view's cost: empty chunks at its end
             for (uint32_t q = q0; q <= q1; ++q) {
-                a.tab->start[s_first[v] + q] = (uint32_t)(j0 + i + 1);
-                a.tab->pair[s_first[v] + q] = end;
+                a.start[s_first[v] + q] = (uint32_t)(j0 + i + 1);
+                a.pair[s_first[v] + q] = end;
             }
             if (last) {   // the first chunk of the next view with entries, and all of the empty views before it
                 for (int u = v + 1; u < a.n_views && s_base[u] == x1; ++u) {
                     const uint32_t stop = s_base[u + 1] == x1 ? s_first[u + 1] : s_first[u] + 1u;
                     for (uint32_t c = s_first[u]; c < stop; ++c) {
-                        a.tab->start[c] = (uint32_t)(j0 + i + 1);
-                        a.tab->pair[c] = end;
+                        a.start[c] = (uint32_t)(j0 + i + 1);
+                        a.pair[c] = end;
                     }
                 }
             }
@@ -744,7 +746,7 @@ __global__ void __launch_bounds__(256) k_bin_emit(BinArgs a) {
     for (uint32_t q = threadIdx.x; q < q4; q += blockDim.x) bin_smem[q] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     const uint32_t V = (uint32_t)min(a.M, a.aux->kept);
-    const uint32_t e0 = min(tab.start[c], V), e1 = min(tab.start[c + 1], V);
+    const uint32_t e0 = min(a.start[c], V), e1 = min(a.start[c + 1], V);
     const int lane = threadIdx.x & 31;
     for (uint32_t jb = e0 + (threadIdx.x & ~31u); jb < e1; jb += blockDim.x) {
         const uint32_t j = jb + lane;
@@ -910,7 +912,7 @@ __global__ void __launch_bounds__(32) k_bin_place(BinArgs a) {
     const uint32_t c = blockIdx.x;
     if (c >= tab.n_chunks) return;
     const uint32_t K = (uint32_t)min(a.counters[CNT_WRITTEN], a.cap);
-    const uint32_t lo = min(tab.pair[c], K), hi = min(tab.pair[c + 1], K);
+    const uint32_t lo = min(a.pair[c], K), hi = min(a.pair[c + 1], K);
     if (lo >= hi) return;
     const ViewDesc &vw = a.db->view[bin_view_of_chunk(tab, a.n_views, c)];
     const uint32_t T = (uint32_t)vw.tiles_x * (uint32_t)vw.tiles_y;
