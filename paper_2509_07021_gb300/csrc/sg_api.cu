@@ -352,11 +352,11 @@ uint64_t capacity_for(const Batch &b, size_t ws_bytes) {
     return lo;
 }
 
-// Backward scratch: batch table, counters, the [M][9] 2D gradients and the
-// persistent backward's own tile order (where walk_ordered; elsewhere it takes the
-// forward's).
+// Backward scratch: batch table, counters, the [M][9] 2D gradients and, last, the
+// persistent backward's own tile order (where walk_ordered). A scratch without room for
+// the order is enough: the backward then walks the tiles in the forward's order.
 struct BwdLayout {
-    size_t batch, counters, dg, order, total;
+    size_t batch, counters, dg, needed, order, total;
 };
 
 BwdLayout bwd_layout(const Batch &b) {
@@ -366,12 +366,11 @@ BwdLayout bwd_layout(const Batch &b) {
     L.batch = take(sizeof(Batch));
     L.counters = take(CNT_N * sizeof(uint64_t));
     L.dg = take(9 * b.n_entries * sizeof(float));
+    L.needed = o;
     L.order = take(walk_ordered(b.n_tiles) ? 4 * (size_t)b.n_tiles : 0);
     L.total = o;
     return L;
 }
-
-size_t bwd_bytes(const Batch &b) { return bwd_layout(b).total; }
 
 // Pixels per thread while the tuning holds the defaults: with few tiles a
 // warp's walk of its list is the critical path, so a tile is given to more
@@ -423,7 +422,7 @@ void fill_sizes(const Batch &b, const WsLayout &L, uint64_t n_pairs, sg_sizes *o
     out->ws_per_pair_bytes = b.n_tiles > kNoKeyTiles ? 17 + (L.tile_passes > 3 ? 1 : 0)
                                                      : 10 + div_up(4 * (uint64_t)L.bin_row, kMatrixShare);
     out->ws_bytes = L.total;
-    out->bwd_ws_bytes = bwd_bytes(b);
+    out->bwd_ws_bytes = bwd_layout(b).total;
 }
 
 // Per-thread pinned host words, mapped into the device, and an event for the
@@ -689,8 +688,9 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     if (!ws || !aligned(ws, ALIGN)) return fail(SG_ERR_INVALID_ARG, "workspace NULL or not 256-byte aligned");
     if (!bwd_ws || !aligned(bwd_ws, ALIGN))
         return fail(SG_ERR_INVALID_ARG, "backward scratch NULL or not 256-byte aligned");
-    if (bwd_ws_bytes < bwd_bytes(b))
-        return fail(SG_ERR_WORKSPACE, "backward scratch of %zu bytes, %zu needed", bwd_ws_bytes, bwd_bytes(b));
+    const BwdLayout BL = bwd_layout(b);
+    if (bwd_ws_bytes < BL.needed)
+        return fail(SG_ERR_WORKSPACE, "backward scratch of %zu bytes, %zu needed", bwd_ws_bytes, BL.needed);
     const uint64_t cap = capacity_for(b, ws_bytes);
     if (cap == UINT64_MAX) return fail(SG_ERR_WORKSPACE, "workspace smaller than its fixed part");
     const WsLayout L = make_layout(b, cap);
@@ -700,7 +700,6 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     const uint2 *ranges = reinterpret_cast<const uint2 *>(w + L.ranges);
     const uint32_t *pv_final = reinterpret_cast<const uint32_t *>(w + L.pval_final);
     char *bw = static_cast<char *>(bwd_ws);
-    const BwdLayout BL = bwd_layout(b);
     Batch *db = reinterpret_cast<Batch *>(bw + BL.batch);
     uint64_t *counters = reinterpret_cast<uint64_t *>(bw + BL.counters);
     float *dg = reinterpret_cast<float *>(bw + BL.dg);
@@ -714,7 +713,7 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     // is only its bound (a list's tail lies behind stopped pixels). With two or three
     // tiles per resident warp the last ones to start decide when the kernel ends.
     TileOrder walk;
-    if (L.walk) {
+    if (L.walk && bwd_ws_bytes >= BL.total) {
         walk.counts = reinterpret_cast<const uint32_t *>(w + L.order_scratch) + TILE_ORDER_WORDS;
         walk.place = reinterpret_cast<const uint32_t *>(w + L.walk_place);
         walk.fallback = reinterpret_cast<const uint32_t *>(w + L.order);
@@ -1203,7 +1202,7 @@ extern "C" int sg_render_backward_noalloc(const sg_scene *scene, const sg_camera
     b.scene[0].grads = grads[0];
     if (!T_final || !last || !d_img) return fail(SG_ERR_INVALID_ARG, "T_final, last and d_img must not be NULL");
     if (!ws || !aligned(ws, ALIGN)) return fail(SG_ERR_INVALID_ARG, "workspace NULL or not 256-byte aligned");
-    const size_t need = bwd_bytes(b);
+    const size_t need = bwd_layout(b).needed;   // one block per tile: no tile order
     if (need > (size_t)SG_NOALLOC_SCRATCH_BYTES)
         return fail(SG_ERR_WORKSPACE,
                     "no-alloc backward needs %zu bytes of scratch for %llu entries; the static scratch holds "

@@ -49,3 +49,16 @@ def test_smallest_frames(views):
     rng = np.random.default_rng(9)
     scene = synth.make_scene(rng, 700, lobes=1, means="cube", cube_side=1.2, masks="uniform")
     run_parity(scene, [synth.make_camera(w, h, 60.0) for w, h in views], seed=2)
+
+
+def test_backward_without_room_for_its_tile_order():
+    rng = np.random.default_rng(13)
+    ds = DeviceScene.from_host(synth.make_scene(rng, 3000, lobes=1, means="cube", cube_side=1.4, masks="uniform"))
+    cams = [synth.make_camera(1920, 1080, 1700.0)]
+    out = render.render_forward(ds, cams)
+    d = torch.ones_like(out.img)
+    want = render.render_backward(ds, cams, out, d)["c0"]
+    grads = render.alloc_grads(ds)
+    bwd = torch.empty(out.sizes["bwd_ws_bytes"] - 4 * out.sizes["n_tiles"], dtype=torch.uint8, device="cuda")
+    sgsplat.sg_render_backward(ds, cams, out.ws, out.T_final, out.last, d, bwd, grads)
+    torch.testing.assert_close(grads["c0"], want, rtol=2e-4, atol=1e-6 * float(want.abs().max()))
