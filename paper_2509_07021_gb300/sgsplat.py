@@ -287,8 +287,17 @@ assert _SCENE.size == ctypes.sizeof(sg_scene) and _CAMERA.size == ctypes.sizeof(
 def _pack_camera(cam):
     vm = np.asarray(cam.viewmat, np.float32).reshape(12)
     bg = np.asarray(cam.bg, np.float32).reshape(3)
-    return _CAMERA.pack(int(cam.width), int(cam.height), cam.fx, cam.fy, cam.cx, cam.cy, *vm.tolist(), cam.near,
-                        *bg.tolist())
+    try:
+        return _CAMERA.pack(int(cam.width), int(cam.height), cam.fx, cam.fy, cam.cx, cam.cy, *vm.tolist(), cam.near,
+                            *bg.tolist())
+    except (OverflowError, TypeError, struct.error):
+        # values outside binary32 or int32 go to the library, which judges them (as infinities),
+        # and whatever float() takes is a number here too: both need the fields one by one
+        c = sg_camera(int(cam.width), int(cam.height), float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy))
+        c.viewmat[:] = vm.tolist()
+        c.near_plane = float(cam.near)
+        c.bg[:] = bg.tolist()
+        return bytes(c)
 
 
 def camera_struct(cam):
