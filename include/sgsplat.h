@@ -239,9 +239,8 @@ int sg_profile_set_stages(uint32_t stage_mask);
  * tiles ordered by descending list length, instead of one block per tile.
  * sg_set_tuning(NULL) restores the defaults: both blends persistent, the
  * forward with 4 pixels per thread, the backward with 8, 64-Gaussian batches
- * (batch 0). While a blend's fields hold these defaults, the call's tile count
- * picks its pixels per thread (fewer for fewer tiles); a batch size other
- * than 0 pins the given shape.
+ * (batch 0), and auto_shapes, with which the call's tile count picks the pixels
+ * per thread (fewer for fewer tiles).
  */
 typedef struct sg_tuning {
     int32_t fwd_pixels_per_thread;
@@ -263,7 +262,10 @@ typedef struct sg_tuning {
      * end early. */
     int32_t fwd_batch;
     int32_t bwd_batch;
-    int32_t reserved[1];
+    /* Bit 0: the forward's, bit 1: the backward's pixels per thread follow the
+     * tile count while that blend's fields hold the defaults. 0: the fields
+     * are taken as they are. */
+    int32_t auto_shapes;
 } sg_tuning;
 int sg_set_tuning(const sg_tuning *t);
 int sg_get_tuning(sg_tuning *t);

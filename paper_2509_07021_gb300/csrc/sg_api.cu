@@ -103,8 +103,8 @@ struct StageTimer {
 
 // Process-wide kernel shape choices (sg_set_tuning); defaults from measurement
 // (1M Gaussians at 1920x1080: both blends persistent, 4 and 8 pixels per thread;
-// with fewer tiles the defaults stand for the tile count's choice, auto_pixels).
-constexpr sg_tuning kDefaultTuning = {4, 8, 1, 1, 0, 0, 0, {0}};
+// with fewer tiles auto_shapes lets the tile count choose, auto_pixels).
+constexpr sg_tuning kDefaultTuning = {4, 8, 1, 1, 0, 0, 0, 3};
 constexpr int kDefaultBatch = 64;
 sg_tuning &tuning() {
     static sg_tuning t = kDefaultTuning;
@@ -372,7 +372,7 @@ BwdLayout bwd_layout(const Batch &b) {
     return L;
 }
 
-// Pixels per thread while the tuning holds the defaults: with few tiles a
+// Pixels per thread under auto_shapes: with few tiles a
 // warp's walk of its list is the critical path, so a tile is given to more
 // warps; with many, fewer warps per tile issue less in all. The lines lie where the
 // measured times cross (us, forward / backward, 1, 2, 4, 8 pixels per thread):
@@ -388,7 +388,7 @@ int auto_pixels(bool backward, uint64_t n_tiles) {
 }
 
 // Blend shape of this call: pixels per thread from the tuning (from the tile
-// count while it holds the defaults), and for the persistent form the resident
+// count under auto_shapes), and for the persistent form the resident
 // grid, the work counter and the tile order.
 int blend_shape(bool backward, uint64_t n_tiles, const uint32_t *order, uint32_t *queue, BlendShape &sh) {
     const sg_tuning &t = tuning();
@@ -396,7 +396,7 @@ int blend_shape(bool backward, uint64_t n_tiles, const uint32_t *order, uint32_t
     sh.persistent = (backward ? t.bwd_persistent : t.fwd_persistent) != 0;
     const int nb = backward ? t.bwd_batch : t.fwd_batch;
     const sg_tuning &d = kDefaultTuning;
-    if (nb == 0 && sh.persistent &&
+    if (((t.auto_shapes >> (backward ? 1 : 0)) & 1) && nb == 0 && sh.persistent &&
         sh.pixels_per_thread == (backward ? d.bwd_pixels_per_thread : d.fwd_pixels_per_thread))
         sh.pixels_per_thread = auto_pixels(backward, n_tiles);
     sh.tile_order = sh.persistent ? order : nullptr;
@@ -815,6 +815,7 @@ int sg_set_tuning(const sg_tuning *t) {
     if (!(t->bwd_batch == 0 || t->bwd_batch == 32 || t->bwd_batch == 64))
         return fail(SG_ERR_INVALID_ARG, "bwd_batch must be 0, 32 or 64 (got %d)", t->bwd_batch);
     tuning() = *t;
+    tuning().auto_shapes &= 3;
     set_sort_wait_polls((uint32_t)t->sort_wait_polls);
     return SG_OK;
 }
@@ -927,7 +928,8 @@ int sg_autotune(const sg_scene *scene, const sg_camera *cams, int n_views, void 
         sg_tuning t = saved;
         t.fwd_pixels_per_thread = t.bwd_pixels_per_thread = 1 << (c >> 1);
         t.fwd_persistent = t.bwd_persistent = c & 1;
-        t.fwd_batch = t.bwd_batch = kDefaultBatch;   // the candidate itself, not the tile count's choice
+        t.fwd_batch = t.bwd_batch = kDefaultBatch;
+        t.auto_shapes = 0;   // the candidate itself, not the tile count's choice
         tuning() = t;
         float tf = 0.f, tb = 0.f;
         for (int r = 0; r <= reps && st == SG_OK; ++r) {
@@ -961,6 +963,7 @@ int sg_autotune(const sg_scene *scene, const sg_camera *cams, int n_views, void 
     t.fwd_persistent = bf & 1;
     t.bwd_pixels_per_thread = 1 << (bb >> 1);
     t.bwd_persistent = bb & 1;
+    t.auto_shapes = 0;
     int best_fb = 64, best_bb = 64;
     best_f = best_b = 1e30f;
     for (int c = 0; c < 3 && st == SG_OK; ++c) {

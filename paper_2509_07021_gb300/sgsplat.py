@@ -83,11 +83,11 @@ class sg_tuning(ctypes.Structure):
     _fields_ = [("fwd_pixels_per_thread", ctypes.c_int32), ("bwd_pixels_per_thread", ctypes.c_int32),
                 ("fwd_persistent", ctypes.c_int32), ("bwd_persistent", ctypes.c_int32),
                 ("sort_wait_polls", ctypes.c_int32), ("fwd_batch", ctypes.c_int32),
-                ("bwd_batch", ctypes.c_int32), ("reserved", ctypes.c_int32 * 1)]
+                ("bwd_batch", ctypes.c_int32), ("auto_shapes", ctypes.c_int32)]
 
 
 TUNING_FIELDS = ("fwd_pixels_per_thread", "bwd_pixels_per_thread", "fwd_persistent", "bwd_persistent",
-                 "sort_wait_polls", "fwd_batch", "bwd_batch")
+                 "sort_wait_polls", "fwd_batch", "bwd_batch", "auto_shapes")
 
 
 class SGError(RuntimeError):
@@ -449,15 +449,20 @@ def sg_render_backward_noalloc(scene: DeviceScene, cams, ws, T_final, last, d_im
 
 
 def sg_set_tuning(fwd_pixels_per_thread=None, bwd_pixels_per_thread=None, fwd_persistent=None,
-                  bwd_persistent=None, sort_wait_polls=None, fwd_batch=None, bwd_batch=None):
+                  bwd_persistent=None, sort_wait_polls=None, fwd_batch=None, bwd_batch=None, auto_shapes=None):
     """Sets the kernels' tuning (unset fields keep their value); no arguments
-    restores the defaults."""
+    restores the defaults. A blend whose shape is given here keeps it at every
+    tile count, unless auto_shapes says otherwise."""
     args = (fwd_pixels_per_thread, bwd_pixels_per_thread, fwd_persistent, bwd_persistent, sort_wait_polls,
-            fwd_batch, bwd_batch)
+            fwd_batch, bwd_batch, auto_shapes)
     if all(a is None for a in args):
         _check(lib().sg_set_tuning(None))
         return
     cur = sg_get_tuning()
+    for bit, given in ((1, (fwd_pixels_per_thread, fwd_persistent, fwd_batch)),
+                       (2, (bwd_pixels_per_thread, bwd_persistent, bwd_batch))):
+        if any(a is not None for a in given):
+            cur["auto_shapes"] &= ~bit
     t = sg_tuning()
     for name, val in zip(TUNING_FIELDS, args):
         setattr(t, name, int(cur[name] if val is None else val))
