@@ -177,7 +177,8 @@ typedef struct sg_sizes {
  *   rect          [M] 2 x uint32: x0 | x1 << 16, y0 | y1 << 16 (tiles, half
  *                 open; the 3-sigma rectangle; empty = culled)
  *   depth_order   [M] uint32: the entries with tiles_touched > 0 sorted by
- *                 (view, depth bits, entry), first. Scratch of the forward: its
+ *                 (view, depth bits, entry), in the largest frames by
+ *                 (depth bits, entry), first. Scratch of the forward: its
  *                 memory is reused by the tile sort, so a finished forward no
  *                 longer holds it.
  *   ranges        [n_tiles] 2 x uint32 [start, end) into the pair arrays

@@ -271,9 +271,12 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
     for (int v = 0; v < b.n_views; ++v)
         row = std::max<uint64_t>(row, (uint64_t)b.view[v].tiles_x * b.view[v].tiles_y);
     row = div_up(row, 4) * 4;
-    // chunks where one chunk's counters of the largest view fit shared memory
-    L.chunked = row <= BIN_MAX_ROW;
+    // chunks where one chunk's counters of the largest view fit shared memory, and enough
+    // chunks at once for the pairs
+    L.chunked = row <= BIN_MAX_ROW && cap <= bin_max_pairs((uint32_t)row);
     L.bin_row = (uint32_t)row;
+    // the chunks are cut view by view; the radix passes' digits hold the view
+    L.by_view = L.chunked && b.n_views > 1;
     const uint64_t img_rows = 3 * n_pixels_of(b) / row, own_rows = (uint64_t)b.n_views + 1;
     L.matrix_in_img = img_rows >= own_rows;
     if (L.chunked)
@@ -292,7 +295,7 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
     L.order_scratch = take((TILE_ORDER_WORDS + TB_BUCKETS) * 4);
     L.bin = take(sizeof(BinTab));
     const uint64_t cuts = std::min<uint64_t>(BIN_MAX_CHUNKS, b.n_views + std::max<uint64_t>(cap / BIN_MIN_CHUNK, 1)) + 1;
-    L.bin_start = take(L.chunked ? 8 * cuts + ALIGN : 0);   // first entries, then first pairs
+    L.bin_start = take(8 * cuts + ALIGN);   // chunks' first entries, then first pairs
     L.scan_words = take(8 * (1 + (uint64_t)b.n_groups));
     L.tile_bits = tile_bits_for(T);
     L.tile_passes = L.chunked ? 0 : radix_passes(L.tile_bits);
@@ -325,7 +328,7 @@ WsLayout make_layout(const Batch &b, uint64_t cap) {
         L.pkey_tmp = tmp;
         L.pval_tmp = tmp + pairs4;
     }
-    // look-back flags of the depth sort's passes (one more with several views), where the
+    // look-back flags of the depth sort's passes (one more by view), where the
     // image cannot hold them, then those of the tile sort's radix passes (chunked: the
     // count matrix of a frame that cannot hold it)
     const uint64_t depth_words = depth_flag_words(M, b.n_views > 1 ? 5 : 4);
@@ -546,11 +549,11 @@ int forward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, co
     {
         // once per entry; entries that reach no tile are left out of the order
         StageTimer t(ST_DEPTH_SORT, stream);
-        SG_CUDA(launch_depth_sort(db, n_views, dkey0, dval0, dkey1, dval1, counters + CNT_ENTRIES, M,
+        SG_CUDA(launch_depth_sort(db, L.by_view, dkey0, dval0, dkey1, dval1, counters + CNT_ENTRIES, M,
                                   L.depth_in_img ? reinterpret_cast<uint32_t *>(img) : hist, aux_depth, stream),
                 "depth sort");
     }
-    const uint32_t *order = n_views > 1 ? dval1 : dval0;   // entries by (view, depth)
+    const uint32_t *order = L.by_view ? dval1 : dval0;   // entries by ((view,) depth)
     CountReadback *rb = nullptr;   // plain form: where the duplicate leaves the pair count for the host
     if (sync) SG_CUDA(count_readback(rb), "pair count readback");
     // grids sized by the capacity (at most SORT_MAX_KEYS pairs); counts read on the device
@@ -856,7 +859,7 @@ static int layout_of(const sg_scene *scenes, int n_scenes, const sg_camera *cams
     out->rec = L.rec;
     out->tiles_touched = L.tiles_touched;
     out->rect = L.rect;
-    out->depth_order = n_views > 1 ? L.dval1 : L.dval0;
+    out->depth_order = L.by_view ? L.dval1 : L.dval0;
     out->ranges = L.ranges;
     out->pair_tile = L.pkey_final;
     out->pair_entry = L.pval_final;

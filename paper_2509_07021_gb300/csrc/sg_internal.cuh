@@ -101,6 +101,7 @@ struct WsLayout {
     uint64_t M, n_tiles, cap;
     int tile_bits, tile_passes;
     bool chunked;         // tile sort by chunks (launch_bin_pairs) instead of radix passes
+    bool by_view;         // the depth sort orders the entries by view first
     bool matrix_in_img;   // the count matrix takes the image's memory (else hist's)
     bool depth_in_img;    // so do, before it, the depth sort's look-back flags
     bool walk;            // the forward files walk lengths for the backward's tile order
@@ -407,12 +408,11 @@ uint32_t sort_wait_polls();
 uint64_t sort_flag_words(uint64_t max_n, int passes);
 uint64_t depth_flag_words(uint64_t max_n, int passes);
 
-// Stable sort of the entries by (view, depth bits), entries whose key in k0 is
-// SORT_DROP_KEY left out (k0: one key per entry; the values, entry indices, are
-// made by the first pass): the four depth digits, then, with several views, one pass whose
+// Stable sort of the entries by depth bits or (by_view) by (view, depth bits), entries whose
+// key in k0 is SORT_DROP_KEY left out (k0: one key per entry; the values, entry indices, are
+// made by the first pass): the four depth digits, then, by_view, one pass whose
 // digit is the entry's view (its counts, aux hist row VIEW_PASS, are
-// preprocess's). The order ends in (k0, v0) with one view, in (k1, v1) with
-// several; aux (zeroed by the caller) then holds the kept count and the status.
+// preprocess's). The order ends in (k0, v0), by_view in (k1, v1); aux (zeroed by the caller) then holds the kept count and the status.
 constexpr int VIEW_PASS = 4;
 struct SortAux {
     uint32_t hist[5][RS_RADIX];   // global digit counts per pass
@@ -420,13 +420,13 @@ struct SortAux {
     uint32_t status;              // 0 or SG_ERR_TIMEOUT
     uint64_t kept;                // keys other than SORT_DROP_KEY (drop mode)
 };
-cudaError_t launch_depth_sort(const Batch *db, int n_views, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
+cudaError_t launch_depth_sort(const Batch *db, bool by_view, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
                               const uint64_t *n_dev, uint64_t max_n, uint32_t *hist, SortAux *aux, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Binning by chunks: (tile, entry) pairs in (tile, depth, entry) order without
 // a sort of the pairs by key digits, for views of up to BIN_MAX_ROW tiles (one
-// chunk's tile counters fit shared memory). The depth-ordered entries of each
+// chunk's tile counters fit shared memory) and up to bin_max_pairs. The depth-ordered entries of each
 // view are cut into chunks of about equal cost; each chunk counts its
 // pairs per tile while it writes them out, one scan of the count matrix gives
 // every (chunk, tile) its first output position and every tile its range, and
@@ -445,6 +445,17 @@ struct BinTab {
     uint32_t n_chunks;                             // chunks in use
     uint32_t first_chunk[SG_MAX_VIEWS + 1];        // first chunk of each view
 };
+// Room for more pairs than this takes the radix passes: a view of more tiles leaves fewer
+// chunks a place on the chip (one per SM past 28.8k tiles, two past 18.9k), whose serial
+// rounds then take longer than two passes over the pairs. Measured (us, chunks / radix, from
+// the ordered entries to the placed pairs): 32400 tiles 7.8M pairs 372 / 413, 15.3M 687 / 661,
+// 21.5M 945 / 689, 56M 2618 / 2049; 49152 tiles 10.8M 496 / 499, 44M 2025 / 1291; 27600 tiles 13M
+// 420 / 635, 49M 1897 / 1786; 22600 tiles 42M 1565 / 1504; 16000 tiles 32.5M 1030 / 1129. The
+// line at two per SM lies between its points.
+inline uint64_t bin_max_pairs(uint32_t row) {
+    const uint32_t per_sm = (227u * 1024u) / (row * 4u + 1024u);
+    return per_sm <= 1u ? 12ull << 20 : per_sm == 2u ? 32ull << 20 : ~0ull;
+}
 uint32_t bin_chunks(uint64_t cap, uint32_t row, int n_views);   // most chunks of a call with room for cap pairs
 struct BinArgs {
     const Batch *db;

@@ -105,3 +105,28 @@ def test_default_shape_at_its_tile_counts(w, h):
     assert torch.equal(out.img, ref.img) and torch.equal(out.T_final, ref.T_final) and torch.equal(out.last, ref.last)
     for k in gr:
         assert torch.linalg.norm(g[k] - gr[k]) <= 2e-5 * torch.linalg.norm(gr[k]) + 1e-12, k
+
+
+@pytest.mark.parametrize("views,line", [([(3856, 2160)], 12 << 20), ([(2560, 2048), (300, 200)], 32 << 20)],
+                         ids=["one_chunk_per_sm", "two_chunks_per_sm"])
+def test_large_frames_at_the_pairs_where_the_route_changes(views, line):
+    """Past so much room for pairs a large frame takes the radix passes: on both sides of
+    the line the lists, the images and (a positive upstream gradient) the sums agree."""
+    rng = np.random.default_rng(8)
+    ds = DeviceScene.from_host(synth.make_scene(rng, 3000, lobes=1, means="cube", cube_side=1.4, masks="uniform"))
+    cams = [synth.make_camera(w, h, 0.9 * w) for w, h in views]
+    got = []
+    for cap in (line, line + 4096):
+        q = sgsplat.sg_workspace_query(ds, cams, cap)
+        ref = render._alloc_outputs(cams, torch.device("cuda"))
+        ws = torch.empty(q["ws_bytes"], dtype=torch.uint8, device="cuda")
+        st, sizes = sgsplat.sg_render_forward(ds, cams, ws, *ref, raise_on_error=False)
+        assert st == sgsplat.SG_OK and 0 < sizes["n_pairs"] <= cap <= sizes["pair_capacity"]
+        out = render.ForwardOut(*ref, ws, sizes)
+        gv = GpuView.plain(ds, cams, out)
+        c0 = render.render_backward(ds, cams, out, torch.ones_like(out.img))["c0"]
+        got.append((gv.pair_entry, gv.ranges, out, c0))
+    a, b = got
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    assert torch.equal(a[2].img, b[2].img) and torch.equal(a[2].last, b[2].last)
+    torch.testing.assert_close(a[3], b[3], rtol=2e-4, atol=1e-6 * float(b[3].abs().max()))
