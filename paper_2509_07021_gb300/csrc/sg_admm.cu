@@ -50,7 +50,7 @@ constexpr int SEL_PER = SEL_BINS / 256;          // bins per thread
 __host__ __device__ constexpr int sel_shift(int p) { return p == 0 ? 21 : p == 1 ? 10 : 0; }
 __host__ __device__ constexpr uint32_t sel_mask(int p) { return p == 2 ? 1023u : 2047u; }
 
-// Adds a block's digit counts to the pass's histogram and clears them.
+// Adds a block's digit counts to the pass's histogram.
 __device__ __forceinline__ void sel_flush(uint32_t *h, uint32_t *__restrict__ hist) {
     __syncthreads();
     for (int i = threadIdx.x; i < SEL_BINS; i += 256)
@@ -62,8 +62,8 @@ __device__ __forceinline__ void sel_clear(uint32_t *h) {
     __syncthreads();
 }
 
-// Writes every key and the first digit's histogram (state, histograms and
-// look-back words are zero on entry); thread 0 sets up the selection state.
+// The selection's kappa and mode, by one thread of the score kernel's grid. (Its other
+// words, the histograms and the look-back words are zero on entry.)
 __device__ __forceinline__ void sel_setup(int64_t n, int64_t kappa, SelState *st) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->kappa = kappa;

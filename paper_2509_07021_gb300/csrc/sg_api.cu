@@ -375,16 +375,30 @@ BwdLayout bwd_layout(const Batch &b) {
     return L;
 }
 
-// Pixels per thread under auto_shapes: with few tiles a
-// warp's walk of its list is the critical path, so a tile is given to more
-// warps; with many, fewer warps per tile issue less in all. The lines lie where the
-// measured times cross (us, forward / backward, 1, 2, 4, 8 pixels per thread):
-//    494 tiles (32k pairs)    27/61    36/84    56/105   78/157
-//   2500 tiles (116k pairs)   29/88    40/99    61/118   85/179
-//   3600 tiles (877k pairs)  134/580  133/393  197/334  278/544
-//   8160 tiles (2.7M pairs)  325/1448 313/945  307/756  384/615
-// (resident blocks: the forward keeps 2432 tiles of 4 pixels per thread in
-// flight, the backward 4256 of 8).
+// Pixels per thread under auto_shapes: with few tiles a warp's walk of its list is the
+// critical path, so a tile is given to more warps; with many, fewer warps per tile issue less
+// in all. Measured (us, forward / backward, 1, 2, 4, 8 pixels per thread; clustered scenes):
+//   tiles  pairs a tile     1         2         4         8
+//     494       57       22/46     28/63     37/78     60/121
+//     475     1336      172/395   217/536   323/619   630/951
+//    1200      130       51/143    67/181   100/217   157/319
+//    1200     1719      149/404   191/431   276/505   472/799
+//    2500       47       30/78     37/92     56/108    84/177
+//    2500      531      145/496   162/395   224/382   349/608
+//    2500     1936      223/731   250/638   298/618   479/801
+//    2880      317      119/381   137/357   194/358   308/553
+//    2880     1704      174/576   178/454   197/409   297/468
+//    3600       62       47/143    48/114    72/128   106/192
+//    3600      281      130/435   142/342   180/320   254/475
+//    3600      875      188/640   194/508   214/439   300/526
+//    5400       58       64/202    60/154    76/131   101/197
+//    5400      381      238/857   234/637   232/529   296/510
+//    5700      369      249/887   241/658   235/544   313/495
+//    7728      157      218/795   208/582   198/482   260/409
+//    8160      329      326/1177  316/860   302/715   387/589
+// The lines lie between these points. The count does not see the lists' length: where
+// they are long in few tiles the backward's choice is up to 1.3 times the best (2500 tiles),
+// and near the lines to more pixels a choice is 3 or 4 % above its neighbour (5400, 5700).
 int auto_pixels(bool backward, uint64_t n_tiles) {
     if (backward) return n_tiles <= 2560 ? 1 : n_tiles <= 3072 ? 2 : n_tiles <= 5632 ? 4 : 8;
     return n_tiles <= 3600 ? 1 : n_tiles <= 7680 ? 2 : 4;
@@ -429,8 +443,9 @@ void fill_sizes(const Batch &b, const WsLayout &L, uint64_t n_pairs, sg_sizes *o
 }
 
 // Per-thread pinned host words, mapped into the device, and an event for the
-// plain form's read of the pair count: the scan's spine kernel stores the count
-// and the depth sort's status there, and the host waits on the event after it.
+// plain form's read of the pair count: the kernel that knows the total (chunk cutter or
+// duplicate) stores it there, the tile sort's last one the status, and the host waits on
+// the event after them.
 struct CountReadback {
     uint64_t *host = nullptr;     // [0] pairs, [1] status
     uint64_t *dev_ptr = nullptr;  // the same words as the current device sees them
@@ -738,7 +753,7 @@ int backward_impl(const sg_scene *scenes, int n_scenes, const sg_camera *cams, c
     }
     {
         StageTimer t(ST_BLEND_BWD, stream);
-        SG_CUDA(launch_blend_backward(db, b.n_tiles, ranges, pv_final, rec, T_final, last, d_img, dg, M, shape,
+        SG_CUDA(launch_blend_backward(db, b.n_tiles, ranges, pv_final, rec, T_final, last, d_img, dg, shape,
                                       evals, stream),
                 "blend backward");
     }
@@ -1240,7 +1255,7 @@ extern "C" int sg_render_backward_noalloc(const sg_scene *scene, const sg_camera
     z.ptr[0] = reinterpret_cast<uint32_t *>(dg);
     z.words[0] = 9 * M;
     SG_CUDA(launch_setup(b, db, counters, stream, z), "setup");
-    SG_CUDA(launch_blend_backward(db, b.n_tiles, ranges, pv_final, rec, T_final, last, d_img, dg, M, shape,
+    SG_CUDA(launch_blend_backward(db, b.n_tiles, ranges, pv_final, rec, T_final, last, d_img, dg, shape,
                                   nullptr, stream),
             "blend backward");
     SG_CUDA(launch_preprocess_backward(b, db, tt, reinterpret_cast<const uint8_t *>(w + L.clamp), dg, M, stream), "preprocess backward");

@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(BLEND_THREADS / P, bwd_min_blocks(P))
 k_blend_bwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
             const uint32_t *__restrict__ pval, const Rec *__restrict__ rec,
             const float *__restrict__ T_final, const int32_t *__restrict__ last,
-            const float *__restrict__ d_img, float *__restrict__ dg, uint64_t M,
+            const float *__restrict__ d_img, float *__restrict__ dg,
             const uint32_t *__restrict__ tile_order, uint32_t *__restrict__ queue, uint32_t n_tiles,
             unsigned long long *__restrict__ evals, const uint64_t *__restrict__ status, int nb) {
     chain_enter();
@@ -752,26 +752,26 @@ k_blend_bwd(const Batch *__restrict__ bp, const uint2 *__restrict__ ranges,
 template <int P, bool PERSIST>
 static void bwd_p(const Batch *db, uint32_t n_tiles, const uint2 *ranges, const uint32_t *pval,
                   const Rec *rec, const float *T_final, const int32_t *last, const float *d_img, float *dg,
-                  uint64_t M, const BlendShape &sh, unsigned long long *evals, cudaStream_t s) {
+                  const BlendShape &sh, unsigned long long *evals, cudaStream_t s) {
     const unsigned grid = PERSIST ? (unsigned)sh.grid : n_tiles;
     if (evals)
         (void)launch_chain(k_blend_bwd<P, true, PERSIST>, dim3(grid), dim3(BLEND_THREADS / P), s,
-            db, ranges, pval, rec, T_final, last, d_img, dg, M, sh.tile_order, sh.queue, n_tiles, evals, sh.status, sh.batch);
+            db, ranges, pval, rec, T_final, last, d_img, dg, sh.tile_order, sh.queue, n_tiles, evals, sh.status, sh.batch);
     else
         (void)launch_chain(k_blend_bwd<P, false, PERSIST>, dim3(grid), dim3(BLEND_THREADS / P), s,
-            db, ranges, pval, rec, T_final, last, d_img, dg, M, sh.tile_order, sh.queue, n_tiles, nullptr, sh.status, sh.batch);
+            db, ranges, pval, rec, T_final, last, d_img, dg, sh.tile_order, sh.queue, n_tiles, nullptr, sh.status, sh.batch);
 }
 
 template <bool PERSIST>
 static cudaError_t bwd_dispatch(const Batch *db, uint32_t n_tiles, const uint2 *ranges, const uint32_t *pval,
                                 const Rec *rec, const float *T_final, const int32_t *last, const float *d_img,
-                                float *dg, uint64_t M, const BlendShape &sh, unsigned long long *evals,
+                                float *dg, const BlendShape &sh, unsigned long long *evals,
                                 cudaStream_t s) {
     switch (sh.pixels_per_thread) {
-        case 1: bwd_p<1, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, M, sh, evals, s); break;
-        case 2: bwd_p<2, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, M, sh, evals, s); break;
-        case 4: bwd_p<4, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, M, sh, evals, s); break;
-        case 8: bwd_p<8, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, M, sh, evals, s); break;
+        case 1: bwd_p<1, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, sh, evals, s); break;
+        case 2: bwd_p<2, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, sh, evals, s); break;
+        case 4: bwd_p<4, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, sh, evals, s); break;
+        case 8: bwd_p<8, PERSIST>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, sh, evals, s); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaSuccess;
@@ -779,7 +779,7 @@ static cudaError_t bwd_dispatch(const Batch *db, uint32_t n_tiles, const uint2 *
 
 cudaError_t launch_blend_backward(const Batch *db, uint32_t n_tiles, const uint2 *ranges,
                                   const uint32_t *pval, const Rec *rec, const float *T_final,
-                                  const int32_t *last, const float *d_img, float *dg, uint64_t M,
+                                  const int32_t *last, const float *d_img, float *dg,
                                   const BlendShape &sh, unsigned long long *evals, cudaStream_t s) {
     if (n_tiles == 0) return cudaSuccess;
     const bool persist = sh.persistent;
@@ -787,8 +787,8 @@ cudaError_t launch_blend_backward(const Batch *db, uint32_t n_tiles, const uint2
     if (sh.status == nullptr || sh.batch < 32 || sh.batch > BWD_BATCH_MAX || sh.batch % 32 != 0)
         return cudaErrorInvalidValue;
     cudaError_t e = persist
-        ? bwd_dispatch<true>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, M, sh, evals, s)
-        : bwd_dispatch<false>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, M, sh, evals, s);
+        ? bwd_dispatch<true>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, sh, evals, s)
+        : bwd_dispatch<false>(db, n_tiles, ranges, pval, rec, T_final, last, d_img, dg, sh, evals, s);
     if (e != cudaSuccess) return e;
     count_launches(1);
     return cudaGetLastError();

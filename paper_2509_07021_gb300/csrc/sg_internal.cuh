@@ -525,7 +525,8 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
 constexpr int TILE_ORDER_WORDS = 512;
 // Tile counts whose backward gets an order of its own: its 8-pixel form starts at
 // 5632 tiles, and with two or three tiles per resident warp the longest of the last
-// decide when the kernel ends (8160 tiles, 5.4M pairs: 650 -> 613 us; 2.7M: 600 -> 587).
+// decide when the kernel ends (8160 tiles, 5.4M pairs: 646 -> 613 us; 2.7M: 597 -> 588;
+// 6700, 3.4M: 632 -> 618; 16000, 9.1M: 1035 -> 1016).
 // With fewer tiles several warps share each (3600: 305 us with either order, and the
 // forward pays 1 us for the ranks); with more, a warp takes several tiles and the
 // forward's order ends as evenly (six scenes in four views each: the same with either).
@@ -555,8 +556,7 @@ cudaError_t launch_blend_forward(const Batch *db, uint32_t n_tiles, const uint2 
 cudaError_t launch_blend_backward(const Batch *db, uint32_t n_tiles, const uint2 *ranges,
                                   const uint32_t *pval, const Rec *rec, const float *T_final,
                                   const int32_t *last, const float *d_img, float *dg,
-                                  uint64_t M, const BlendShape &shape, unsigned long long *evals,
-                                  cudaStream_t s);
+                                  const BlendShape &shape, unsigned long long *evals, cudaStream_t s);
 // ADMM proximal + dual step (kind 0: opacity, 1: sharpness) and the penalty
 // gradient term; workspace bytes for n items.
 size_t admm_workspace_bytes(int64_t n);

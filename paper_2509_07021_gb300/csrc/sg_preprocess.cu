@@ -475,7 +475,7 @@ __device__ __forceinline__ uint32_t count_tiles(const TileReach &R, int x0, int 
 // (on false: a lane without a Gaussian) and share the tile rows; else each lane
 // walks its own rows.
 template <int DL, int DS, int CM, bool SPREAD>
-__device__ __forceinline__ uint32_t preprocess_entry(bool on,const ViewDesc &vw, const SceneDesc &sc, int64_t g, float px,
+__device__ __forceinline__ uint32_t preprocess_entry(bool on, const ViewDesc &vw, const SceneDesc &sc, int64_t g, float px,
                                                  float py, float pz, const Geo3 &g3, float o, float gm,
                                                  const ColourBase &cb, uint64_t e,
                                                  Rec *__restrict__ rec, uint32_t *__restrict__ tiles_touched,
@@ -827,7 +827,7 @@ __device__ __forceinline__ void adjoint_gaussian(const Batch &b, const SceneDesc
 
     float d_mean[3] = {0.f, 0.f, 0.f}, d_scale[3] = {0.f, 0.f, 0.f}, d_q[4] = {0.f, 0.f, 0.f, 0.f};
     float d_opac = 0.f, d_gmask = 0.f, d_c0[3] = {0.f, 0.f, 0.f};
-    bool first = true;   // first visible view writes lobe gradients, later views add
+    bool first = true;   // no visible view yet: the first writes the SH gradients, later ones add
     constexpr bool multi_view = !ONE_VIEW;
     Geo3 g3;
     geo3_recipe(s0, s1, s2, q0, q1, q2, q3, g3);

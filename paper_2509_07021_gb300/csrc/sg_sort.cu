@@ -8,7 +8,7 @@
 // the depth passes are run once per (view, Gaussian) entry, before the
 // entries are duplicated into pairs, and the pairs are then binned by tile
 // (chunks; radix passes over the tile digits for a view of more tiles than a
-// chunk's counters hold). Duplication walks the entries in depth order and
+// chunk's counters hold, and for large views with many pairs). Duplication walks the entries in depth order and
 // both binnings are stable, so the result is identical to the 64-bit sort.
 #include "sg_internal.cuh"
 
@@ -327,30 +327,22 @@ __device__ __forceinline__ uint32_t len_bucket(const uint2 r) { return len_bucke
 // After the radix tile sort: tiles that got no pair get the range (0, 0), every
 // tile joins its list-length bucket (len_bucket), and the sort's status is
 // merged into the call's (and written to the host word).
-// no_pass: one tile, so no pass ran and the pairs are tile 0's.
 __global__ void __launch_bounds__(256) k_os_finish(const SortAux *aux, uint64_t *counters, uint2 *ranges,
-                                                   uint64_t n_ranges, bool no_pass, uint64_t max_n,
-                                                   uint64_t *status_mirror, uint32_t *bucket_counts) {
+                                                   uint64_t n_ranges, uint64_t *status_mirror,
+                                                   uint32_t *bucket_counts) {
     chain_enter();
     __shared__ uint32_t h[TB_BUCKETS];
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool ok = counters[CNT_STATUS] == (uint64_t)SG_OK;
     if (i == 0) {
         if (aux->status) counters[CNT_STATUS] = aux->status;
         if (status_mirror) *status_mirror = counters[CNT_STATUS];
     }
     uint2 rg = make_uint2(0u, 0u);
     if (i < n_ranges) {
-        if (no_pass) {
-            const uint64_t n = ok ? min(counters[CNT_WRITTEN], max_n) : 0ull;
-            if (i == 0 && n > 0) rg = make_uint2(0u, (uint32_t)n);
+        rg = ranges[i];
+        if (rg.x == RANGE_EMPTY) {
+            rg = make_uint2(0u, 0u);
             ranges[i] = rg;
-        } else {
-            rg = ranges[i];
-            if (rg.x == RANGE_EMPTY) {
-                rg = make_uint2(0u, 0u);
-                ranges[i] = rg;
-            }
         }
     }
     h[threadIdx.x] = 0u;
@@ -535,8 +527,7 @@ cudaError_t launch_tile_radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uin
     }
     if (e != cudaSuccess) return refused(e);
     (void)launch_chain(k_os_finish, dim3((unsigned)std::max<uint64_t>(div_up(n_ranges, 256), 1)), dim3(256), s,
-                       (const SortAux *)aux, counters, ranges, n_ranges, bits == 0, max_n, status_mirror,
-                       order_counts);
+                       (const SortAux *)aux, counters, ranges, n_ranges, status_mirror, order_counts);
     count_launches(passes + 1);
     return cudaGetLastError();
 }
