@@ -246,9 +246,8 @@ int build_batch(const sg_scene *scenes, int n_scenes, const sg_camera *cams, con
 }
 
 uint64_t n_pixels_of(const Batch &b) {
-    uint64_t p = 0;
-    for (int v = 0; v < b.n_views; ++v) p += (uint64_t)b.view[v].W * b.view[v].H;
-    return p;
+    const ViewDesc &last = b.view[b.n_views - 1];
+    return last.pix_off + (uint64_t)last.W * last.H;
 }
 
 // Calls whose views have at most this many tiles in all keep no sorted tile ids.

@@ -352,11 +352,13 @@ __global__ void __launch_bounds__(256) k_os_finish(const SortAux *aux, uint64_t 
     if (h[threadIdx.x]) atomicAdd(&bucket_counts[threadIdx.x], h[threadIdx.x]);
 }
 
-// Opts a kernel into dynamic shared memory. The limit belongs to the function on its
+// Opts a kernel into dynamic shared memory where this call's `bytes` need it (beside a few
+// KB of static; 48 KB in all need no opting in). The limit belongs to the function on its
 // device, not to the call: it is set to the most any call may ask for, never to this
 // call's size, so that no host thread lowers it between another's set and launch.
 template <typename K>
-static cudaError_t allow_smem(K kernel, size_t most) {
+static cudaError_t allow_smem(K kernel, size_t bytes, size_t most) {
+    if (bytes <= 32 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
@@ -457,7 +459,7 @@ template <int ITEMS>
 static cudaError_t depth_small(const Batch *db, const uint32_t *keys, uint32_t M, uint32_t *vout, SortAux *aux,
                                int passes, cudaStream_t s) {
     constexpr size_t smem = (size_t)(2 * 1024 * ITEMS + 32 * RS_RADIX) * 4;
-    const cudaError_t e = allow_smem(k_depth_small<ITEMS>, smem);
+    const cudaError_t e = allow_smem(k_depth_small<ITEMS>, smem, smem);
     if (e != cudaSuccess) return e;
     (void)launch_chain_smem(k_depth_small<ITEMS>, dim3(1), dim3(1024), smem, s, keys, M, vout, aux, db, passes);
     count_launches(1);
@@ -973,7 +975,7 @@ cudaError_t launch_bin_pairs(const BinArgs &a, cudaStream_t s) {
         a.max_chunks > BIN_MAX_CHUNKS || a.cap > SORT_MAX_KEYS)
         return cudaErrorInvalidValue;
     const size_t smem = (size_t)a.row * 4;
-    cudaError_t e = allow_smem(k_bin_emit, BIN_MAX_ROW * 4);
+    cudaError_t e = allow_smem(k_bin_emit, smem, BIN_MAX_ROW * 4);
     if (e != cudaSuccess) return e;
     // larger blocks shorten the look-back over many entries (1M: 20 -> 14 us) but
     // cost the short ones 2 us
@@ -993,8 +995,8 @@ cudaError_t launch_bin_place(const BinArgs &a, cudaStream_t s) {
     const size_t smem = (size_t)a.row * 4;
     auto scan_bytes = [](uint32_t chunks) { return (size_t)div_up(chunks, BIN_SCAN_WARPS) * BIN_SCAN_WARPS * 32 * 4; };
     const size_t scan_smem = scan_bytes(a.max_chunks);
-    cudaError_t e = allow_smem(k_bin_place, BIN_MAX_ROW * 4);
-    if (e == cudaSuccess) e = allow_smem(k_bin_scan, scan_bytes(BIN_MAX_CHUNKS));
+    cudaError_t e = allow_smem(k_bin_place, smem, BIN_MAX_ROW * 4);
+    if (e == cudaSuccess) e = allow_smem(k_bin_scan, scan_smem, scan_bytes(BIN_MAX_CHUNKS));
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
