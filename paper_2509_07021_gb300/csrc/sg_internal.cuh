@@ -313,7 +313,8 @@ __device__ __forceinline__ uint64_t block_lookback64(uint64_t *__restrict__ dfla
 // schedule its blocks while the kernel before it drains; its first statement
 // waits until that kernel has completed and its writes are visible, so the
 // chain keeps plain stream order. Right after the wait it lets the next kernel
-// be scheduled in turn. Both instructions are no-ops for a kernel launched
+// be scheduled in turn (the binning kernels do not, see chain_wait, and k_duplicate is
+// launched in plain order). Both instructions are no-ops for a kernel launched
 // without the attribute.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void chain_enter() {
